@@ -33,6 +33,12 @@ struct msa_ctx {
   int K = 0, o = 0, e = 0, precision = MSA_AUTO, sat_limit = 32767, smax = 0, smin = 0;
   std::vector<int8_t> hM;
   std::string letters;
+  // the matrix's diagonal dominates (2 s(a, b) <= s(a, a) + s(b, b)): self
+  // scores are diagonal sums; letters with a negative diagonal score, and
+  // whether the loaded set holds one
+  bool diag_dominant = false, neg_letters = false;
+  uint32_t neg_diag = 0;
+  int64_t self_cells = 0;  // DP cells the last self_scores call needed
   uint8_t hlut[256];
   std::string err;
 
@@ -130,6 +136,8 @@ SeqSet seqset(msa_ctx *ctx);
 Scoring scoring(msa_ctx *ctx);
 int run_pairs(msa_ctx *ctx, const std::vector<int2> &pairs_in, const std::vector<int32_t> &dst_in,
               int32_t *d_out);
+// S(k, k) of the sequences at the sorted positions idx (null = all n) into d_out
+int self_scores(msa_ctx *ctx, const std::vector<int32_t> *idx, int32_t *d_out);
 int selector_center(msa_ctx *ctx, int64_t *center_out);
 // refs: ascending sorted positions of a reference sample, empty = every sequence
 int selector_center_refined(msa_ctx *ctx, int k, const std::vector<int32_t> &refs,
@@ -147,8 +155,9 @@ struct SetView {
 };
 int run_center(msa_ctx *ctx, int mode, const std::vector<int32_t> &qsorted,
                const SetView *view = nullptr, int q_begin = 0, int q_end = -1);
-// the device error word -> an MSA_E* code (synchronises the stream)
-int check_derr(msa_ctx *ctx);
+// the device error word -> an MSA_E* code (synchronises the stream); bits
+// (nullable): the word itself
+int check_derr(msa_ctx *ctx, unsigned *bits = nullptr);
 // cell precision and lanes per group of the alignment to a center of length Lc
 bool align_packed(msa_ctx *ctx, int Lc);
 int align_lanes(msa_ctx *ctx, int Lc, bool packed);

@@ -82,10 +82,11 @@ void stage_collect(msa_ctx *ctx, int s) {
     cudaGetLastError();
 }
 
-int check_derr(msa_ctx *ctx) {
+int check_derr(msa_ctx *ctx, unsigned *bits) {
   unsigned h[2] = {0, 0};
   CK(cudaMemcpyAsync(h, ctx->derr, sizeof h, cudaMemcpyDeviceToHost, ctx->st));
   CK(cudaStreamSynchronize(ctx->st));
+  if (bits) *bits = h[0];
   if (h[0] & MSA_DERR_LETTER) return fail(ctx, MSA_EINVAL, "letter outside the alphabet");
   if (h[0] & MSA_DERR_TRACE) return fail(ctx, MSA_ECUDA, "inconsistent traceback codes");
   if (h[0] & MSA_DERR_OVERFLOW) return fail(ctx, MSA_ENOMEM, "int16 overflow list full");
@@ -154,6 +155,54 @@ int run_pairs(msa_ctx *ctx, const std::vector<int2> &pairs_in, const std::vector
     CK((++ctx->launches, launch_pairs)(G, ss, sc, job, grid, ctx->st));
   }
   return MSA_OK;
+}
+
+// Self scores: diagonal sums where the matrix allows it (k_self_diag), int32
+// alignments of a sequence with itself else.  Sets without a letter of
+// negative diagonal score (the usual case) cost one launch and no host wait.
+int self_scores(msa_ctx *ctx, const std::vector<int32_t> *idx, int32_t *d_out) {
+  const int count = idx ? (int)idx->size() : ctx->n;
+  auto pos = [&](int x) { return idx ? (*idx)[x] : x; };
+  std::vector<int2> sp;
+  std::vector<int32_t> dst;
+  auto align = [&]() -> int {  // the listed positions by alignment
+    for (int32_t x : dst) {
+      const int64_t L = ctx->len_sorted[pos(x)];
+      ctx->self_cells += L * L;
+      sp.push_back(make_int2(pos(x), pos(x)));
+    }
+    return run_pairs(ctx, sp, dst, d_out);
+  };
+  ctx->self_cells = 0;
+  if (!ctx->diag_dominant) {
+    dst.resize(count);
+    std::iota(dst.begin(), dst.end(), 0);
+    return align();
+  }
+  int32_t *d_idx = nullptr, *exc = nullptr;
+  if (idx) {
+    TRY(ensure(ctx, ctx->pair_dst, sizeof(int32_t) * std::max(count, 1)));
+    d_idx = P<int32_t>(ctx->pair_dst);
+    CK(cudaMemcpyAsync(d_idx, idx->data(), sizeof(int32_t) * count, cudaMemcpyHostToDevice, ctx->st));
+  }
+  if (ctx->neg_letters) {
+    TRY(ensure(ctx, ctx->pair_out, sizeof(int32_t) * ((size_t)count + 1)));
+    exc = P<int32_t>(ctx->pair_out);
+    CK(cudaMemsetAsync(exc, 0, sizeof(int32_t), ctx->st));
+  }
+  const SeqSet ss = seqset(ctx);
+  CK((++ctx->launches, launch_self_diag)(ss.res, ss.pstart, ss.len, d_idx, count, ctx->dM, ctx->K,
+                                         d_out, exc, ctx->st));
+  if (!exc) return MSA_OK;
+  int32_t ne = 0;
+  CK(cudaMemcpyAsync(&ne, exc, sizeof ne, cudaMemcpyDeviceToHost, ctx->st));
+  CK(cudaStreamSynchronize(ctx->st));
+  if (ne == 0) return MSA_OK;
+  dst.resize(ne);
+  CK(cudaMemcpyAsync(dst.data(), exc + 1, sizeof(int32_t) * ne, cudaMemcpyDeviceToHost, ctx->st));
+  CK(cudaStreamSynchronize(ctx->st));
+  std::sort(dst.begin(), dst.end());
+  return align();
 }
 
 // ------------------------------------------------------------ center planning
@@ -594,7 +643,7 @@ int run_center(msa_ctx *ctx, int mode, const std::vector<int32_t> &qsorted, cons
   stage_collect(ctx, ST_CENTER_K);
   const float center_ms = ctx->stage_ms[ST_CENTER_K];
   int64_t cells = 0;
-  if (mode == 0) {  // pairs q < s (the self scores are counted by their own pass)
+  if (mode == 0) {  // pairs q < s
     for (int x = q_begin; x < q_end; ++x) cells += (int64_t)lens[x] * suffix[x + 1];
   } else {
     for (int q : qsorted) cells += (int64_t)lens[q] * suffix[0];
@@ -1026,6 +1075,13 @@ int msa_create(msa_ctx **out, const msa_params *p, void *cuda_stream) {
     delete ctx;
     return MSA_EINVAL;
   }
+  ctx->diag_dominant = true;
+  for (int a = 0; a < ctx->K; ++a) {
+    const int saa = ctx->hM[a * (ctx->K + 1)];
+    if (saa < 0) ctx->neg_diag |= 1u << a;
+    for (int b = 0; b < a; ++b)
+      if (2 * ctx->hM[a * ctx->K + b] > saa + ctx->hM[b * (ctx->K + 1)]) ctx->diag_dominant = false;
+  }
   memset(ctx->hlut, 255, sizeof ctx->hlut);
   for (int a = 0; a < ctx->K; ++a) ctx->hlut[(uint8_t)ctx->letters[a]] = (uint8_t)a;
   ctx->st = (cudaStream_t)cuda_stream;
@@ -1175,10 +1231,12 @@ int msa_load(msa_ctx *ctx, const uint8_t *letters, const int64_t *offsets, int64
   CK(cudaMemcpyAsync(ctx->d_srcoff.p, offsets, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, ctx->st));
   CK(cudaMemsetAsync(ctx->derr, 0, 2 * sizeof(unsigned), ctx->st));
   CK((++ctx->launches, launch_encode)(src, P<int64_t>(ctx->d_srcoff), P<int32_t>(ctx->d_perm), P<int64_t>(ctx->d_pstart),
-                   P<int32_t>(ctx->d_len), ctx->n, ctx->dLut, ctx->K, P<uint8_t>(ctx->res), ctx->derr,
-                   ctx->st));
+                   P<int32_t>(ctx->d_len), ctx->n, ctx->dLut, ctx->K, ctx->neg_diag, P<uint8_t>(ctx->res),
+                   ctx->derr, ctx->st));
   stage_end(ctx, ST_ENCODE);
-  int rc = check_derr(ctx);
+  unsigned bits = 0;
+  int rc = check_derr(ctx, &bits);
+  ctx->neg_letters = (bits & MSA_DERR_NEG_DIAG) != 0;
   stage_collect(ctx, ST_ENCODE);
   if (rc != MSA_OK) {
     ctx->n = 0;
@@ -1247,18 +1305,9 @@ int msa_select_center(msa_ctx *ctx, int mode, const int64_t *refs, int64_t nref,
   CK(cudaMemsetAsync(ctx->pairsum.p, 0, sizeof(unsigned long long) * n, ctx->st));
   CK(cudaMemsetAsync(ctx->derr, 0, 2 * sizeof(unsigned), ctx->st));
   // self scores of every sequence first: every pair's similarity needs both
-  {
-    std::vector<int2> sp(n);
-    std::vector<int32_t> dst(n);
-    for (int k = 0; k < n; ++k) { sp[k] = make_int2(k, k); dst[k] = k; }
-    TRY(run_pairs(ctx, sp, dst, P<int32_t>(ctx->self)));
-  }
+  TRY(self_scores(ctx, nullptr, P<int32_t>(ctx->self)));
   TRY(run_center(ctx, mode == MSA_CENTER_EXACT ? 0 : 1, qs));
-  {
-    double sumsq = 0;
-    for (int k = 0; k < n; ++k) sumsq += (double)ctx->len_sorted[k] * ctx->len_sorted[k];
-    ctx->cells[0] += (int64_t)sumsq;
-  }
+  ctx->cells[0] += ctx->self_cells;
   CK((++ctx->launches, launch_center_finalize)(mode == MSA_CENTER_EXACT ? 0 : 1, n, (int)qs.size(),
                             P<int32_t>(ctx->d_perm), P<unsigned long long>(ctx->pairsum),
                             P<long long>(ctx->rowsum), ctx->dsmall + 1, ctx->dsmall + 2,
@@ -1297,12 +1346,7 @@ int msa_center_partial(msa_ctx *ctx, const int64_t *refs, int64_t nref, int32_t 
   if (sampled) TRY(reference_positions(ctx, refs, nref, qs));
   CK(cudaMemsetAsync(ctx->pairsum.p, 0, sizeof(unsigned long long) * n, ctx->st));
   CK(cudaMemsetAsync(ctx->derr, 0, 2 * sizeof(unsigned), ctx->st));
-  {  // every pair's similarity needs both self scores
-    std::vector<int2> sp(n);
-    std::vector<int32_t> dst(n);
-    for (int k = 0; k < n; ++k) { sp[k] = make_int2(k, k); dst[k] = k; }
-    TRY(run_pairs(ctx, sp, dst, P<int32_t>(ctx->self)));
-  }
+  TRY(self_scores(ctx, nullptr, P<int32_t>(ctx->self)));  // every pair's similarity needs both
   if (sampled) {
     // the references (queries) in contiguous chunks of about equal length sum
     std::vector<int32_t> mine;

@@ -2,9 +2,19 @@
 #pragma once
 #include "common.cuh"
 
+// neg_diag: bit a set when letter a scores negative against itself; such a
+// letter in the set raises MSA_DERR_NEG_DIAG (not an error).
 cudaError_t launch_encode(const uint8_t *letters, const int64_t *src_off, const int32_t *perm,
                           const int64_t *pstart, const int32_t *len, int n, const uint8_t *lut,
-                          int padc, uint8_t *res, unsigned *err, cudaStream_t st);
+                          int padc, uint32_t neg_diag, uint8_t *res, unsigned *err,
+                          cudaStream_t st);
+
+// Diagonal self scores of count sequences (idx: sorted indices, null = all);
+// exc (null where no letter scores negative against itself): exc[0] counts
+// the list positions in exc[1..] whose sequences hold such a letter.
+cudaError_t launch_self_diag(const uint8_t *res, const int64_t *pstart, const int32_t *len,
+                             const int32_t *idx, int count, const int8_t *M, int K, int32_t *out,
+                             int32_t *exc, cudaStream_t st);
 
 // res/pstart/center/M/K/o/e: the walk recomputes the score of each cell on
 // its path (the codes hold a source only where H > 0).
@@ -40,6 +50,3 @@ cudaError_t launch_center_finalize(int mode, int n, int nref, const int32_t *per
 
 cudaError_t launch_apply_overflow(int mode, const int2 *ovf, const int32_t *scores, int count,
                                   unsigned long long *pairsum, const int32_t *self, cudaStream_t st);
-
-cudaError_t launch_self_pairs(int n, int2 *pairs, int32_t *dst, cudaStream_t st);
-cudaError_t launch_extract_scores(const int32_t *seg, int n, int32_t *out, cudaStream_t st);

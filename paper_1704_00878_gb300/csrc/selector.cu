@@ -371,10 +371,7 @@ int selector_center_refined(msa_ctx *ctx, int k, const std::vector<int32_t> &ref
   std::vector<unsigned long long> ps(k);  // sum_j center_sim(q, j) per candidate
   if (refs.empty()) {
     // self scores of every sequence (every candidate meets every sequence)
-    std::vector<int2> sp(n);
-    std::vector<int32_t> dst(n);
-    for (int x = 0; x < n; ++x) { sp[x] = make_int2(x, x); dst[x] = x; }
-    TRY(run_pairs(ctx, sp, dst, P<int32_t>(ctx->self)));
+    TRY(self_scores(ctx, nullptr, P<int32_t>(ctx->self)));
     CK(cudaMemsetAsync(ctx->pairsum.p, 0, sizeof(unsigned long long) * n, ctx->st));
     TRY(run_center(ctx, 2, qs));
     stage_end(ctx, ST_CENTER);
@@ -402,10 +399,7 @@ int selector_center_refined(msa_ctx *ctx, int k, const std::vector<int32_t> &ref
     CK(cudaMemcpyAsync(s->vstart.p, vstart.data(), sizeof(int64_t) * nv, cudaMemcpyHostToDevice, ctx->st));
     CK(cudaMemcpyAsync(s->vlen.p, view.len.data(), sizeof(int32_t) * nv, cudaMemcpyHostToDevice, ctx->st));
     // self scores of the view's entries (references, then candidates)
-    std::vector<int2> sp(nv);
-    std::vector<int32_t> dst(nv);
-    for (int v = 0; v < nv; ++v) { sp[v] = make_int2(view.idx[v], view.idx[v]); dst[v] = v; }
-    TRY(run_pairs(ctx, sp, dst, P<int32_t>(s->vself)));
+    TRY(self_scores(ctx, &view.idx, P<int32_t>(s->vself)));
     CK(cudaMemsetAsync(ctx->pairsum.p, 0, sizeof(unsigned long long) * nv, ctx->st));
     view.ss = SeqSet{P<uint8_t>(ctx->res), P<int64_t>(s->vstart), P<int32_t>(s->vlen), nv};
     view.self = P<int32_t>(s->vself);
