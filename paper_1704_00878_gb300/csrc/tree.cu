@@ -2,23 +2,15 @@
 // NJ trees, Figure 4, citing Saitou and Nei): fixed-point p-distances between
 // the merged rows, then neighbour joining on those integers.
 //
-// Distances: a CTA takes a 64 x 64 tile of row pairs (tiles on and above the
-// diagonal), stages 256 columns of its 2 x 64 rows in shared memory and
-// compares four columns per 32-bit word: x = a ^ b, a byte is nonzero iff
-// ((x & 0x7f7f7f7f) + 0x7f7f7f7f | x) has its top bit set; the residue flags
-// are the same test against '-' in every byte; per pair two SWAR byte
-// counters (compared, mismatched) gather up to 64 words before they are
-// summed into 32-bit totals.
+// Distances: the rows become bit planes of their symbol indices (32 columns
+// per word), a CTA takes a 64 x 64 tile of row pairs and combines the planes
+// with three-input logic operations (k_planes, k_pdist).
 //
 // Neighbour joining: the matrix stays on the device (int32 -- every entry and
-// joined distance within 2^30, else ERANGE -- positions in
-// ascending slot order); every join is two launches -- the minimum of Q over
-// the active pairs (warps over tiles of 8 rows x 256 columns, the last CTA to
-// finish reduces the CTAs' minima) and the join itself (CTAs over the rows: branch lengths,
-// the new node's row and column, the row sums updated in place; the last
-// CTA to finish adds up the new node's row sum).  When a quarter of the
-// positions are inactive the matrix is packed to the active ones, which keeps
-// the work of a join near m^2 / 2.  No launch waits on another.
+// joined distance within 2^30, else ERANGE -- positions in ascending slot
+// order); one cooperative launch runs the joins until half of the positions
+// are left (k_nj_joins), then the matrix is packed to the active ones; the
+// last few hundred positions run in one CTA.
 #include <algorithm>
 #include <climits>
 #include <vector>
@@ -28,309 +20,565 @@
 namespace msa_detail {
 namespace {
 
-constexpr int kTile = 64;    // rows per side of a distance tile
-constexpr int kWords = 64;   // 32-bit words (4 columns) per staged chunk
+constexpr int kTile = 64;        // rows per side of a distance tile
+constexpr int kPlaneWords = 15;  // 32-column words staged per step
+constexpr int kSlab = 16384;     // rows whose planes are held at once
 constexpr long long kDScale = 1LL << 20;
 constexpr long long kDLimit = 1LL << 30;  // |distance| bound of the joins (int32 matrix)
-constexpr int kArgThreads = 256;
-constexpr int kRowBlk = 8;    // rows of one warp task (tile) of the Q minimum
-constexpr int kColSeg = 256;  // columns of a tile: 8 per lane
-constexpr int kJoinThreads = 1024;
+constexpr int kJoinCtas = 16;      // CTAs of a large matrix's joins: one cluster
+constexpr int kSoloRows = 128;     // a matrix of at most this many positions: one CTA
+constexpr int kScanSeg = 512;      // columns of one warp task of a row scan: 16 per lane
+constexpr int kScanTasks = 256;    // scan results held at once (a row has at most 128 segments)
+constexpr int kJoinSmem = 215 * 1024;
 
-// 0x80 in every byte of w that is nonzero
-__device__ __forceinline__ uint32_t bytes_nonzero(uint32_t w) {
-  return (((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w) & 0x80808080u;
+// ---------------------------------------------------------------- distances
+// Bit planes of the listed rows (list null: rows r0, r0 + 1, ...): per 32
+// columns a word per bit of the symbol index and a word of residue flags
+// (not '-').  lo = planes 0-3 (0-2 and the flags where three planes hold the
+// alphabet), hi = plane 4 and the flags.  One warp per word, one ballot per
+// plane; words past the row's columns are zero.
+template <bool WIDE>
+__global__ void __launch_bounds__(256) k_planes(const uint8_t *__restrict__ msa, int64_t W,
+                                                const int32_t *__restrict__ list, int r0, int rows,
+                                                int words, const uint8_t *__restrict__ lut, int K,
+                                                uint4 *__restrict__ lo, uint2 *__restrict__ hi) {
+  __shared__ uint8_t slut[256];
+  slut[threadIdx.x] = lut[threadIdx.x];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5, total = (int64_t)rows * words;
+  for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < total; x += warps) {
+    const int i = (int)(x / words), w = (int)(x - (int64_t)i * words);
+    const int row = list ? list[r0 + i] : r0 + i;
+    const int64_t c = (int64_t)w * 32 + lane;
+    const int s = c < W ? slut[msa[(size_t)row * W + c]] : K + 1;
+    const bool res = s <= K;  // K + 1 is the gap
+    const unsigned v = res ? (unsigned)s : 0u;
+    unsigned p[5];
+#pragma unroll
+    for (int b = 0; b < (WIDE ? 5 : 3); ++b) p[b] = __ballot_sync(MSA_FULL_MASK, (v >> b) & 1u);
+    const unsigned m = __ballot_sync(MSA_FULL_MASK, res);
+    if (lane == 0) {
+      if (WIDE) {
+        lo[x] = make_uint4(p[0], p[1], p[2], p[3]);
+        hi[x] = make_uint2(p[4], m);
+      } else {
+        lo[x] = make_uint4(p[0], p[1], p[2], m);
+      }
+    }
+  }
 }
 
-// acc + (w >> 7) as one multiply-add (high half of w * 2^25) on the FMA pipe,
-// beside the integer pipe the comparisons keep busy
-__device__ __forceinline__ uint32_t add_top_bits(uint32_t acc, uint32_t w) {
-  uint32_t d;
-  asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(1u << 25), "r"(acc));
-  return d;
-}
-
-// sum of the four bytes of a SWAR counter
-__device__ __forceinline__ uint32_t byte_sum(uint32_t c) {
-  c = (c & 0x00ff00ffu) + ((c >> 8) & 0x00ff00ffu);
-  return (c & 0xffffu) + (c >> 16);
-}
-
-// Rows of a distance tile: list A x list B (row indices of the MSA; null =
-// the rows 0..nA-1 / 0..nB-1).  SYM: A and B are the same list, tiles on and
-// above the diagonal, D[a][b] and D[b][a] stored (ld = nA); NEAREST: every
-// tile of A x B, and per row of A the smallest (distance << 32 | position in
-// B) by an atomic minimum -- the nearest row of B, ties to its first position.
+// Tiles of 64 x 64 row pairs.  SYM: A and B are the same rows; D[a][b] and
+// D[b][a] stored (ld columns); NEAREST (near not null): per row of A the
+// smallest (distance << 32 | position in B) by an atomic minimum -- the
+// nearest row of B, ties to its first position.  a0 / b0: list positions of
+// the slabs' first rows.
 struct PdistJob {
-  const int32_t *ia, *ib;
-  int nA, nB;
-  bool sym;
-  long long *D;               // SYM
-  unsigned long long *near;   // NEAREST: one key per row of A
+  const uint4 *loA, *loB;
+  const uint2 *hiA, *hiB;
+  int words;       // per row, a multiple of kPlaneWords
+  int nA, nB;      // rows of the slabs
+  int a0, b0;
+  size_t ld;
+  unsigned long long *near;
 };
 
-__global__ void __launch_bounds__(256) k_pdist(const uint8_t *__restrict__ msa, int64_t W,
-                                               PdistJob job) {
+// Distances from the planes: per 32 columns of a pair one three-input logic
+// operation per plane gathers the differing symbols, two mask them to the
+// columns both rows have, and the bits of three words are added up by a
+// carry-save step before they are counted.  About 20 lane operations per 32
+// column pairs where comparing four letters per 32-bit word took 72: integer
+// (ALU) bound either way.  4,000 rows x 7,200 columns measured 5.4 ms with
+// byte comparisons (their unaligned byte staging included) and 1.07 ms with the
+// planes, the planes' own pass included.
+template <bool WIDE, class T>
+__global__ void __launch_bounds__(256, 2) k_pdist(PdistJob job, T *__restrict__ D) {
   const int ta = blockIdx.y, tb = blockIdx.x;
-  if (job.sym && tb < ta) return;
-  __shared__ uint32_t sA[kTile][kWords + 1], sB[kTile][kWords + 1];
+  const bool sym = job.near == nullptr;
+  if (sym && job.a0 + ta * kTile > job.b0 + tb * kTile) return;
+  __shared__ __align__(16) uint4 sAl[kTile][kPlaneWords], sBl[kTile][kPlaneWords];
+  __shared__ __align__(16) uint2 sAh[WIDE ? kTile : 1][kPlaneWords], sBh[WIDE ? kTile : 1][kPlaneWords];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int a0 = ta * kTile, b0 = tb * kTile;
-  constexpr uint32_t kGap4 = 0x2d2d2d2du;  // "----"
   uint32_t comp[4][4] = {}, mism[4][4] = {};
-  const int64_t nwords = (W + 3) / 4;
-  for (int64_t w0 = 0; w0 < nwords; w0 += kWords) {
+  for (int w0 = 0; w0 < job.words; w0 += kPlaneWords) {
     __syncthreads();
-    // stage 64 rows x 256 columns of each side; columns past W and rows past
-    // the lists are gaps
-    for (int idx = threadIdx.x; idx < kTile * kWords; idx += 256) {
-      const int r = idx / kWords, w = idx - r * kWords;
-      const int64_t c0 = (w0 + w) * 4;
-      uint32_t va = kGap4, vb = kGap4;
-      const int pa = a0 + r, pb = b0 + r;
-      const int ra = pa < job.nA ? (job.ia ? job.ia[pa] : pa) : -1;
-      const int rb = pb < job.nB ? (job.ib ? job.ib[pb] : pb) : -1;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int64_t c = c0 + u;
-        if (c < W) {
-          if (ra >= 0) va = (va & ~(0xffu << (8 * u))) | ((uint32_t)msa[(size_t)ra * W + c] << (8 * u));
-          if (rb >= 0) vb = (vb & ~(0xffu << (8 * u))) | ((uint32_t)msa[(size_t)rb * W + c] << (8 * u));
-        }
+    for (int idx = threadIdx.x; idx < kTile * kPlaneWords; idx += 256) {
+      const int r = idx / kPlaneWords, w = idx - r * kPlaneWords;
+      const size_t ga = (size_t)(a0 + r) * job.words + w0 + w, gb = (size_t)(b0 + r) * job.words + w0 + w;
+      const bool va = a0 + r < job.nA, vb = b0 + r < job.nB;
+      sAl[r][w] = va ? job.loA[ga] : make_uint4(0u, 0u, 0u, 0u);
+      sBl[r][w] = vb ? job.loB[gb] : make_uint4(0u, 0u, 0u, 0u);
+      if (WIDE) {
+        sAh[r][w] = va ? job.hiA[ga] : make_uint2(0u, 0u);
+        sBh[r][w] = vb ? job.hiB[gb] : make_uint2(0u, 0u);
       }
-      sA[r][w] = va;
-      sB[r][w] = vb;
     }
     __syncthreads();
-    uint32_t cc[4][4] = {}, cm[4][4] = {};  // byte counters: at most 64 per byte
-#pragma unroll 4
-    for (int w = 0; w < kWords; ++w) {
-      uint32_t a[4], fa[4], b[4], fb[4];
+#pragma unroll 1
+    for (int w = 0; w < kPlaneWords; w += 3) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = sA[ty + 16 * i][w];
-        fa[i] = bytes_nonzero(a[i] ^ kGap4);
-        b[i] = sB[tx + 16 * i][w];
-        fb[i] = bytes_nonzero(b[i] ^ kGap4);
-      }
+      for (int ih = 0; ih < 4; ih += 2) {  // two rows of A at a time (registers)
+        uint4 al[2][3];
+        uint2 ah[2][3];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            al[i][u] = sAl[ty + 16 * (ih + i)][w + u];
+            if (WIDE) ah[i][u] = sAh[ty + 16 * (ih + i)][w + u];
+          }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const uint32_t both = fa[i] & fb[j];
-          cc[i][j] = add_top_bits(cc[i][j], both);
-          cm[i][j] = add_top_bits(cm[i][j], bytes_nonzero(a[i] ^ b[j]) & both);
+          uint4 bl[3];
+          uint2 bh[3];
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            bl[u] = sBl[tx + 16 * j][w + u];
+            if (WIDE) bh[u] = sBh[tx + 16 * j][w + u];
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            uint32_t c[3], m[3];
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+              uint32_t x = al[i][u].x ^ bl[u].x;
+              x |= al[i][u].y ^ bl[u].y;
+              x |= al[i][u].z ^ bl[u].z;
+              if (WIDE) {
+                x |= al[i][u].w ^ bl[u].w;
+                x |= ah[i][u].x ^ bh[u].x;
+                c[u] = ah[i][u].y & bh[u].y;
+              } else {
+                c[u] = al[i][u].w & bl[u].w;
+              }
+              m[u] = x & c[u];
+            }
+            // one bits of three words: popc(sum) + 2 popc(carry)
+            comp[ih + i][j] += __popc(c[0] ^ c[1] ^ c[2]) +
+                               2 * __popc((c[0] & c[1]) | (c[2] & (c[0] | c[1])));
+            mism[ih + i][j] += __popc(m[0] ^ m[1] ^ m[2]) +
+                               2 * __popc((m[0] & m[1]) | (m[2] & (m[0] | m[1])));
+          }
         }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        comp[i][j] += byte_sum(cc[i][j]);
-        mism[i][j] += byte_sum(cm[i][j]);
       }
+    }
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int a = a0 + ty + 16 * i;
-    if (a >= job.nA) continue;
+    const int la = a0 + ty + 16 * i;
+    if (la >= job.nA) continue;
+    const int a = job.a0 + la;
     unsigned long long nearest = ~0ull;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int b = b0 + tx + 16 * j;
-      if (b >= job.nB) continue;
+      const int lb = b0 + tx + 16 * j;
+      if (lb >= job.nB) continue;
+      const int b = job.b0 + lb;
       const long long d = comp[i][j] ? ((long long)mism[i][j] * kDScale) / comp[i][j] : kDScale;
-      if (job.sym) {
-        job.D[(size_t)a * job.nA + b] = d;
-        if (ta != tb) job.D[(size_t)b * job.nA + a] = d;
+      if (sym) {
+        D[(size_t)a * job.ld + b] = (T)d;
+        D[(size_t)b * job.ld + a] = (T)d;
       } else {
         const unsigned long long key = ((unsigned long long)d << 32) | (unsigned)b;
         nearest = key < nearest ? key : nearest;
       }
     }
-    if (!job.sym && nearest != ~0ull) atomicMin(&job.near[a], nearest);
+    if (!sym && nearest != ~0ull) atomicMin(&job.near[a], nearest);
   }
 }
 
-struct Pick {
-  long long q, xy;  // Q, then position pair x * 2^32 + y (x < y)
+// ---------------------------------------------------------------- joins
+// The joins of a matrix of P active positions until m_stop of them are left,
+// in one launch of one cluster of NB CTAs (one CTA where P is small).  A join
+// is a chain of short dependent steps, so what bounds it is latency, and the
+// design keeps one cluster barrier per join and few trips to memory:
+//   - CTA c owns the positions k = c, c + NB, ...; every CTA keeps its own
+//     copy of all row sums and updates it itself from rows x and y, so only
+//     the CTAs' best pairs cross the barrier (through distributed shared
+//     memory);
+//   - the new node's row goes to a staging row (two, by join parity) that its
+//     owner copies over row x during the next join, when no CTA reads the old
+//     row any more; column x is written by each row's owner, the only one
+//     that scans that row;
+//   - a row is scanned (the smallest (m - 2) d(k, y) - r_y over y > k and the
+//     second) only when it may hold a Q below every known one.  Each owned
+//     row carries its best known partner, whose value is recomputed exactly
+//     each join, and a lower bound of its other entries: the second smallest
+//     after a scan, then moved each join by the least any entry can have
+//     changed -- it loses d(k, y) <= dmax_k as m - 2 falls by one and gains
+//     what r_y lost, at least the least loss of any active y; the new column's
+//     entry takes the partner's place or lowers the bound.  Rows whose bound
+//     exceeds the smallest Q of the pairs known (the CTAs' last best pairs)
+//     hold no better or equal pair but their partner's.  The new row's own
+//     minimum comes from the pass that computes it.
+// Smallest Q first, then the smallest (x, y): a skipped row's other pairs are
+// strictly worse than a known pair, so ties are decided exactly.  On 4,000
+// protein rows the first thousand joins scan about 5 rows each.  NJ of
+// 4,000 rows: 83.6 ms with one launch scanning every tile and one
+// joining, 27.9 ms so (latency: about 7 us a join, half of it row scans).
+struct NjPick {
+  long long q;
+  unsigned xy;  // x << 16 | y
+  int d;
 };
-__device__ __forceinline__ bool pick_less(const Pick &u, const Pick &v) {
+__device__ __forceinline__ bool pick_less(const NjPick &u, const NjPick &v) {
   return u.q < v.q || (u.q == v.q && u.xy < v.xy);
 }
-__device__ __forceinline__ Pick warp_min(Pick p) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    Pick o;
-    o.q = __shfl_xor_sync(MSA_FULL_MASK, p.q, off);
-    o.xy = __shfl_xor_sync(MSA_FULL_MASK, p.xy, off);
-    if (pick_less(o, p)) p = o;
-  }
-  return p;
+// smallest of the lanes' 64-bit values: the high halves first, then the low
+// halves of the lanes that hold the smallest high half
+__device__ __forceinline__ long long warp_min_ll(long long v) {
+  const int hi = __reduce_min_sync(MSA_FULL_MASK, (int)(v >> 32));
+  const unsigned lo = __reduce_min_sync(MSA_FULL_MASK, (int)(v >> 32) == hi ? (unsigned)v : 0xffffffffu);
+  return (long long)(((unsigned long long)(unsigned)hi << 32) | lo);
 }
-__device__ __forceinline__ Pick block_min(Pick p, Pick *sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  p = warp_min(p);
-  if (lane == 0) sh[w] = p;
-  __syncthreads();
-  if (w == 0) {
-    p = lane < nw ? sh[lane] : Pick{LLONG_MAX, LLONG_MAX};
-    p = warp_min(p);
-  }
-  return p;  // valid in warp 0
+__device__ __forceinline__ NjPick warp_min(const NjPick &p) {
+  NjPick o;
+  o.q = warp_min_ll(p.q);
+  o.xy = __reduce_min_sync(MSA_FULL_MASK, p.q == o.q ? p.xy : 0xffffffffu);
+  const unsigned who = __ballot_sync(MSA_FULL_MASK, p.q == o.q && p.xy == o.xy);
+  o.d = __shfl_sync(MSA_FULL_MASK, p.d, __ffs(who) - 1);
+  return o;
+}
+// sum of the lanes' 64-bit values (24-bit pieces, each below 2^31 over a warp)
+__device__ __forceinline__ long long warp_sum_ll(long long v) {
+  const unsigned a = __reduce_add_sync(MSA_FULL_MASK, (unsigned)(v & 0xffffff));
+  const unsigned b = __reduce_add_sync(MSA_FULL_MASK, (unsigned)((v >> 24) & 0xffffff));
+  const int c = __reduce_add_sync(MSA_FULL_MASK, (int)(v >> 48));
+  return (long long)a + ((long long)b << 24) + ((long long)c << 48);
 }
 
-// The active pair of smallest Q = (m - 2) d(x, y) - r_x - r_y, ties to the
-// smallest x, then y (positions ascend with the slots).  Warp tasks are tiles
-// of kRowBlk rows x kColSeg columns of the upper triangle: a lane loads -r_y
-// and the active flags of its kColSeg / 32 columns once per tile, then per
-// row one int32 distance per column and one 64-bit multiply-add
-// (m - 2) d - r_y, compared with the tile's best so far plus r_x.  Inside a
-// tile a lane meets its cells in ascending (x, y), so a strict comparison
-// keeps the first of equal values; tiles, lanes and CTAs then merge on
-// (Q, x, y).  The last CTA to finish reduces every CTA's minimum into sel.
-__global__ void __launch_bounds__(kArgThreads) k_nj_argmin(const int *__restrict__ D, int P,
-                                                           const long long *__restrict__ r,
-                                                           const uint8_t *__restrict__ act, int m,
-                                                           const int2 *__restrict__ tasks, int ntask,
-                                                           Pick *__restrict__ part,
-                                                           unsigned *__restrict__ ticket,
-                                                           int *__restrict__ sel) {
-  constexpr int U = kColSeg / 32;
-  __shared__ Pick sh[32];
-  __shared__ bool last;
-  const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  const int f = m - 2;
-  Pick best{LLONG_MAX, LLONG_MAX};
-  for (int task = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < ntask; task += warps) {
-    const int2 tk = tasks[task];
-    const int yb = tk.y + lane;
-    long long nry[U];
-    unsigned okm = 0;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int y = yb + 32 * u;
-      const bool ok = y < P && act[y];
-      okm |= (ok ? 1u : 0u) << u;
-      nry[u] = ok ? -r[y] : 0;
+struct NjJob {
+  int *D;                 // P x P
+  int P, m_stop, t0, n;   // all P positions active; join t0 is the next one
+  long long *r;           // row sums, written back at the end
+  uint8_t *act;           // written at the end: active positions
+  int *node;
+  int *joins;
+  long long *lengths;     // numerators of the branch lengths over 2 (m - 2)
+  int *stage;             // 2 x P staging rows
+  long long *rcopy;       // null: the row sums sit in shared memory, else grid x P
+  unsigned *err;
+};
+
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(r)
+               : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+
+// the distance of a pair from its value v = f d - r_y: (v + r_y) / f has no
+// remainder; an estimate within 2^8, then the remainder's quotient exactly
+__device__ __forceinline__ int pair_distance(long long v, long long ry, int f, float inv) {
+  v += ry;
+  const int d = __float2int_rn((float)v * inv);
+  return d + __float2int_rn((float)(v - (long long)f * d) * inv);
+}
+
+constexpr long long kNjHigh = 1LL << 60;     // bound of a row without a partner
+
+// NB CTAs (a power of two: owner and index of a position are a mask and a
+// shift) of NT threads.
+template <int NB, int NT>
+__global__ void __launch_bounds__(NT, 1) k_nj_joins(NjJob job) {
+  extern __shared__ __align__(16) long long nj_smem[];
+  constexpr int NW = NT / 32;
+  static_assert(NW <= 32 && NB <= 32, "one lane per warp, one per CTA");
+  __shared__ __align__(16) NjPick s_pick[2][NB];  // every CTA's best pair, by join parity
+  __shared__ NjPick s_wpick[NW];
+  __shared__ long long s_sum[NW], s_new[2][NW];
+  __shared__ int s_min[NW], s_top[NW], s_nlist;
+  __shared__ long long s_scan[2][kScanTasks];  // a scan task's smallest and second key, largest entry
+  __shared__ int s_stop[kScanTasks];
+  const int P = job.P, cta = NB > 1 ? (int)(blockIdx.x & (NB - 1)) : 0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nown = (P - cta + NB - 1) / NB, cap = (P + NB - 1) / NB;
+  long long *L = nj_smem;               // per owned row: lower bound of its entries but cy's
+  long long *r = L + cap;
+  int *cy, *cd, *dm, *list;
+  unsigned *act;
+  {
+    long long *p = r;
+    if (job.rcopy) r = job.rcopy + (size_t)cta * P;
+    else p += P;
+    cy = reinterpret_cast<int *>(p);    // the row's best known partner (-1 none), its distance,
+    cd = cy + cap;                      // an upper bound of the row's distances, the rows to
+    dm = cd + cap;                      // scan
+    list = dm + cap;
+    act = reinterpret_cast<unsigned *>(list + cap);
+  }
+  auto active = [&](int k) { return (act[k >> 5] >> (k & 31)) & 1u; };
+  auto wants_scan = [&](int i) { list[atomicAdd(&s_nlist, 1)] = i; };
+  // a row's partner, bound and largest entry from its smallest and second keys
+  auto set_row = [&](int i, long long b1, long long b2, int top, int f) {
+    L[i] = b2 == LLONG_MAX ? kNjHigh : b2 >> 16;
+    cy[i] = -1;
+    cd[i] = 0;
+    dm[i] = 0;
+    if (b1 != LLONG_MAX) {
+      const int y = (int)(b1 & 0xffff);
+      cy[i] = y;
+      cd[i] = pair_distance(b1 >> 16, r[y], f, 1.f / (float)f);
+      dm[i] = top;
     }
-    long long tq = LLONG_MAX;  // the tile's best Q for this lane, at (tx, ty)
-    int tx = 0, ty = 0;
-    const int xend = min(tk.x + kRowBlk, P);
-    for (int x = tk.x; x < xend; ++x) {
-      if (!act[x]) continue;  // the same x on every lane
-      const long long rx = r[x];
-      // columns y > x only: u from ceil((x + 1 - yb) / 32) on
-      const int lim = x + 1 - yb;
-      const int umin = lim <= 0 ? 0 : (lim + 31) >> 5;
-      const unsigned rm = umin >= U ? 0u : okm & (0xffffffffu << umin);
-      if (rm == 0) continue;
-      const int *row = D + (size_t)x * P;
-      int dv[U];
+  };
+  for (int k = tid; k < P; k += NT) r[k] = job.r[k];
+  for (int w = tid; w < (P + 31) / 32; w += NT)
+    act[w] = 32 * w + 32 <= P ? 0xffffffffu : (1u << (P - 32 * w)) - 1u;
+  if (tid == 0) s_nlist = 0;
+  __syncthreads();
+  for (int i = tid; i < nown; i += NT) wants_scan(i);
+  __syncthreads();
+  if constexpr (NB > 1) {  // every CTA has started before any writes to its shared memory
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  int m = P, t = job.t0, xprev = -1, xcur = -1;
+  int *stage_cur = job.stage, *stage_prev = job.stage + P;
+  int parity = 0;
+  const NjPick none{LLONG_MAX, 0xffffffffu, 0};
+  for (;;) {
+    const int f = m - 2;
+    // the listed rows' minima anew
+    const int nlist = s_nlist;
+    const int nseg = (P + kScanSeg - 1) / kScanSeg, chunk = kScanTasks / nseg;
+    for (int l0 = 0; l0 < nlist; l0 += chunk) {
+      const int rows = min(chunk, nlist - l0);
+      for (int task = warp; task < rows * nseg; task += NW) {
+        const int at = task / nseg, y0 = (task - at * nseg) * kScanSeg;
+        const int k = list[l0 + at] * NB + cta;
+        long long best = LLONG_MAX, next = LLONG_MAX;  // the smallest (value << 16 | y), the second
+        int top = INT_MIN;
+        if (y0 + kScanSeg > k + 1) {
+          const int *row = k == xcur ? stage_prev : job.D + (size_t)k * P;
+          int dv[kScanSeg / 32];
+          unsigned ok = 0;
 #pragma unroll
-      for (int u = 0; u < U; ++u) dv[u] = (rm >> u) & 1u ? row[yb + 32 * u] : 0;
-      // q < tq  <=>  f d - r_y < tq + r_x (no overflow: |Q| < 2^63 by far)
-      long long thr = tq == LLONG_MAX ? LLONG_MAX : tq + rx;
+          for (int u = 0; u < kScanSeg / 32; ++u) {
+            const int y = y0 + 32 * u + lane;
+            const bool v = y > k && y < P && ((act[(y0 >> 5) + u] >> lane) & 1u);
+            ok |= (v ? 1u : 0u) << u;
+            dv[u] = v ? __ldcg(row + y) : 0;
+          }
+#pragma unroll
+          for (int u = 0; u < kScanSeg / 32; ++u) {
+            if (!((ok >> u) & 1u)) continue;
+            const int y = y0 + 32 * u + lane;
+            const long long v = (((long long)f * dv[u] - r[y]) << 16) | (long long)y;
+            top = max(top, dv[u]);
+            next = min(next, max(best, v));
+            best = min(best, v);
+          }
+          const long long wbest = warp_min_ll(best);
+          next = warp_min_ll(best == wbest ? next : best);
+          best = wbest;
+          top = __reduce_max_sync(MSA_FULL_MASK, top);
+        }
+        if (lane == 0) {
+          s_scan[0][task] = best;
+          s_scan[1][task] = next;
+          s_stop[task] = top;
+        }
+      }
+      __syncthreads();
+      for (int at = tid; at < rows; at += NT) {
+        const int i = list[l0 + at];
+        long long b1 = LLONG_MAX, b2 = LLONG_MAX;
+        int top = INT_MIN;
+        for (int w = at * nseg; w < (at + 1) * nseg; ++w) {
+          b2 = min(min(b2, s_scan[1][w]), max(b1, s_scan[0][w]));
+          b1 = min(b1, s_scan[0][w]);
+          top = max(top, s_stop[w]);
+        }
+        set_row(i, b1, b2, top, f);
+      }
+      __syncthreads();
+    }
+    // this CTA's best pair among its rows' partners, to every CTA
+    NjPick best = none;
+    for (int i = tid; i < nown; i += NT) {
+      const int k = i * NB + cta;
+      if (cy[i] < 0 || !active(k)) continue;
+      const NjPick p{(long long)f * cd[i] - r[cy[i]] - r[k], ((unsigned)k << 16) | (unsigned)cy[i], cd[i]};
+      if (pick_less(p, best)) best = p;
+    }
+    best = warp_min(best);
+    if (lane == 0) s_wpick[warp] = best;
+    if (tid == 0) s_nlist = 0;
+    __syncthreads();
+    NjPick *slots = s_pick[parity];
+    if constexpr (NB > 1) {
+      if (warp == 0) {
+        best = warp_min(lane < NW ? s_wpick[lane] : none);
+        if (lane < NB)
+          asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                           cluster_addr(slots + cta, (uint32_t)lane)),
+                       "r"((unsigned)best.q), "r"((unsigned)((unsigned long long)best.q >> 32)),
+                       "r"(best.xy), "r"((unsigned)best.d)
+                       : "memory");
+      }
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    // lane c: CTA c's pair (one CTA: warp c's)
+    const NjPick mine = NB > 1 ? (lane < NB ? slots[lane] : none) : (lane < NW ? s_wpick[lane] : none);
+    best = warp_min(mine);
+    parity ^= 1;
+    if (best.xy == 0xffffffffu) {  // no pair (distances beyond their bound)
+      if (tid == 0) atomicOr(job.err, MSA_DERR_RANGE);
+      break;
+    }
+    // the join of x < y: the branch lengths' numerators, the new node n + t in
+    // position x, its distances floor((d(x,k) + d(y,k) - d(x,y)) / 2), the row
+    // sums, y retired
+    const int x = (int)(best.xy >> 16), y = (int)(best.xy & 0xffffu);
+    const long long dxy = best.d;
+    if (cta == 0 && tid == 0) {
+      job.lengths[2 * t] = f * dxy + r[x] - r[y];
+      job.lengths[2 * t + 1] = f * dxy - r[x] + r[y];
+      job.joins[2 * t] = job.node[x];
+      job.joins[2 * t + 1] = job.node[y];
+      job.node[x] = job.n + t;
+    }
+    xprev = xcur;
+    xcur = x;
+    const int *rowx = x == xprev ? stage_prev : job.D + (size_t)x * P;
+    const int *rowy = y == xprev ? stage_prev : job.D + (size_t)y * P;
+    // the last new row takes its place in the matrix (its owner; nobody reads
+    // that row of the matrix during this join)
+    const bool settle = xprev >= 0 && (xprev & (NB - 1)) == cta && xprev != x && xprev != y;
+    const bool ownx = (x & (NB - 1)) == cta;
+    const int f2 = f - 1;
+    long long sum = 0, nbest = LLONG_MAX, nnext = LLONG_MAX;
+    int cmin = INT_MAX, ntop = INT_MIN, big = 0;
+    // this thread's owned row: its entries of rows x and y, in flight early
+    const int kown = tid * NB + cta;
+    const int axown = kown < P ? __ldcg(rowx + kown) : 0, ayown = kown < P ? __ldcg(rowy + kown) : 0;
+    constexpr int U = 8;  // entries in flight per thread: loads first, then stores
+    for (int base = 0; base < P; base += U * NT) {
+      int a[U], b[U];
+      long long rk[U];
+      unsigned on = 0;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const long long v = (long long)f * dv[u] + nry[u];
-        if (((rm >> u) & 1u) && v < thr) {
-          thr = v;
-          tq = v - rx;
-          tx = x;
-          ty = yb + 32 * u;
+        if (base + u * NT >= P) break;  // the same for every thread
+        const int k = base + u * NT + tid;
+        const bool in = k < P && ((act[k >> 5] >> lane) & 1u) && k != x && k != y;
+        on |= (in ? 1u : 0u) << u;
+        a[u] = in ? __ldcg(rowx + k) : 0;
+        b[u] = in ? __ldcg(rowy + k) : 0;
+        rk[u] = in ? r[k] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (base + u * NT >= P) break;
+        if (!((on >> u) & 1u)) continue;
+        const int k = base + u * NT + tid;
+        // (entries within 2^30: the new one and the loss are within 1.5 * 2^30)
+        const long long both = (long long)a[u] + b[u];
+        const int dn = (int)((both - dxy) >> 1), loss = (int)(both - dn);
+        big = max(big, dn < 0 ? -dn : dn);
+        sum += dn;
+        cmin = min(cmin, loss);
+        rk[u] -= loss;
+        r[k] = rk[u];
+        if (ownx) {
+          stage_cur[k] = dn;
+          if (k > x) {  // the new row's own minimum
+            const long long v = (((long long)f2 * dn - rk[u]) << 16) | (long long)k;
+            nnext = min(nnext, max(nbest, v));
+            nbest = min(nbest, v);
+            ntop = max(ntop, dn);
+          }
         }
       }
     }
-    if (tq != LLONG_MAX) {
-      const Pick c{tq, ((long long)tx << 32) | (long long)ty};
-      if (pick_less(c, best)) best = c;
+    if (settle)
+      for (int k = tid; k < P; k += NT)
+        if (k != x) job.D[(size_t)xprev * P + k] = __ldcg(stage_prev + k);
+    if (big > (int)kDLimit) atomicOr(job.err, MSA_DERR_RANGE);
+    sum = warp_sum_ll(sum);
+    cmin = __reduce_min_sync(MSA_FULL_MASK, cmin);
+    if (lane == 0) { s_sum[warp] = sum; s_min[warp] = cmin; }
+    if (ownx) {
+      const long long wbest = warp_min_ll(nbest);
+      nnext = warp_min_ll(nbest == wbest ? nnext : nbest);
+      ntop = __reduce_max_sync(MSA_FULL_MASK, ntop);
+      if (lane == 0) { s_new[0][warp] = wbest; s_new[1][warp] = nnext; s_top[warp] = ntop; }
     }
-  }
-  best = block_min(best, sh);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = best;
-    __threadfence();
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  Pick p{LLONG_MAX, LLONG_MAX};
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-    const Pick o{__ldcg(&part[b].q), __ldcg(&part[b].xy)};  // written by other CTAs
-    if (pick_less(o, p)) p = o;
-  }
-  __syncthreads();
-  p = block_min(p, sh);
-  if (threadIdx.x == 0) {
-    sel[0] = (int)(p.xy >> 32);
-    sel[1] = (int)(p.xy & 0xffffffffLL);
-    *ticket = 0;
-  }
-}
-
-// Join t of the positions sel = {x, y} (x < y): branch lengths, the new
-// node n + t in position x, its distances floor((d(x,k) + d(y,k) - d(x,y)) / 2),
-// the row sums, y retired.  CTAs take ranges of k; the last CTA to finish
-// adds up their sums into r_x (every CTA has read r_x by then).
-__global__ void __launch_bounds__(kJoinThreads) k_nj_join(int *__restrict__ D, int P,
-                                                          long long *__restrict__ r,
-                                                          uint8_t *__restrict__ act,
-                                                          int *__restrict__ node, int m,
-                                                          const int *__restrict__ sel, int t, int n,
-                                                          int *__restrict__ joins,
-                                                          double *__restrict__ lengths,
-                                                          long long *__restrict__ part,
-                                                          unsigned *__restrict__ ticket,
-                                                          unsigned *__restrict__ err) {
-  __shared__ long long wsum[kJoinThreads / 32];
-  __shared__ bool last;
-  const int x = sel[0], y = sel[1];
-  const long long dxy = D[(size_t)x * P + y], rx = r[x], ry = r[y];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const long long f = m - 2;
-    const double den = (double)(2 * f);
-    lengths[2 * t] = (double)(f * dxy + rx - ry) / den;
-    lengths[2 * t + 1] = (double)(f * dxy - rx + ry) / den;
-    joins[2 * t] = node[x];
-    joins[2 * t + 1] = node[y];
-  }
-  long long sum = 0;
-  bool bad = false;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < P; k += gridDim.x * blockDim.x) {
-    if (!act[k] || k == x || k == y) continue;
-    const long long dxk = D[(size_t)x * P + k], dyk = D[(size_t)y * P + k];
-    const long long dn = (dxk + dyk - dxy) >> 1;
-    bad |= dn > kDLimit || dn < -kDLimit;
-    D[(size_t)x * P + k] = (int)dn;
-    D[(size_t)k * P + x] = (int)dn;
-    r[k] += dn - dxk - dyk;
-    sum += dn;
-  }
-  if (bad) atomicOr(err, MSA_DERR_RANGE);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(MSA_FULL_MASK, sum, off);
-  if (lane == 0) wsum[w] = sum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long s = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += wsum[i];
-    part[blockIdx.x] = s;
-    __threadfence();
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    --m;
+    ++t;
+    { int *z = stage_cur; stage_cur = stage_prev; stage_prev = z; }  // stage_prev: row x
+    cmin = __reduce_min_sync(MSA_FULL_MASK, lane < NW ? s_min[lane] : INT_MAX);
+    sum = warp_sum_ll(lane < NW ? s_sum[lane] : 0);
+    if (tid == 0) {
+      r[x] = sum;
+      act[y >> 5] &= ~(1u << (y & 31));
+    }
+    // the smallest Q of the last best pairs that live on
+    long long ub = LLONG_MAX;
+    {
+      const int pa = (int)(mine.xy >> 16), pb = (int)(mine.xy & 0xffffu);
+      if (mine.xy != 0xffffffffu && pa != x && pa != y && pb != x && pb != y)
+        ub = (long long)f2 * mine.d - r[pa] - r[pb];
+    }
+    ub = warp_min_ll(ub);
+    // the owned rows' new entries, partners and bounds; those that may hold a
+    // better pair (the settled row is complete: its copy came before the
+    // barrier)
+    for (int i = tid; i < nown; i += NT) {
+      const int k = i * NB + cta;
+      if (k == y || (k != x && !active(k))) continue;
+      if (k == x) {
+        long long b1 = LLONG_MAX, b2 = LLONG_MAX;
+        int top = INT_MIN;
+        for (int w = 0; w < NW; ++w) {
+          b2 = min(min(b2, s_new[1][w]), max(b1, s_new[0][w]));
+          b1 = min(b1, s_new[0][w]);
+          top = max(top, s_top[w]);
+        }
+        if (f2 > 0) set_row(i, b1, b2, top, f2);
+        continue;
+      }
+      const int ax = i == tid ? axown : __ldcg(rowx + k), ay = i == tid ? ayown : __ldcg(rowy + k);
+      const int dn = (int)(((long long)ax + ay - dxy) >> 1);
+      job.D[(size_t)k * P + x] = dn;
+      long long Li = L[i] + ((long long)cmin - dm[i]);
+      int cyi = cy[i], cdi = cd[i];
+      if (cyi == y || cyi == x) cyi = -1;
+      if (k < x) {  // the new entry: the best known pair, or part of the rest
+        const long long v = (long long)f2 * dn - sum;
+        const long long was = cyi >= 0 ? (long long)f2 * cdi - r[cyi] : LLONG_MAX;
+        if (cyi >= 0) Li = min(Li, max(v, was));
+        if (v < was) { cyi = x; cdi = dn; }
+        dm[i] = max(dm[i], dn);
+        cd[i] = cdi;
+      }
+      L[i] = Li;
+      cy[i] = cyi;
+      if (Li - r[k] <= ub) wants_scan(i);
+    }
+    __syncthreads();
+    if (m <= job.m_stop) break;
   }
   __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  __threadfence();
-  long long s = 0;
-  for (int b = 0; b < (int)gridDim.x; ++b) s += __ldcg(&part[b]);
-  r[x] = s;
-  node[x] = n + t;
-  act[y] = 0;
-  *ticket = 0;
+  // the last new row into the matrix; CTA 0 hands the state back
+  if (xcur >= 0 && (xcur & (NB - 1)) == cta)
+    for (int k = tid; k < P; k += NT)
+      if (k != xcur && active(k)) job.D[(size_t)xcur * P + k] = __ldcg(stage_prev + k);
+  if (cta == 0)
+    for (int k = tid; k < P; k += NT) {
+      job.r[k] = r[k];
+      job.act[k] = active(k) ? 1 : 0;
+    }
+  if constexpr (NB > 1) {  // nobody leaves while a pair may still arrive
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
 }
 
 // Positions of the active entries, ascending (one CTA; P <= 65536).
@@ -374,7 +622,7 @@ __global__ void __launch_bounds__(1024) k_nj_index(const uint8_t *__restrict__ a
 __global__ void k_nj_pack(const int *__restrict__ D, int P, const long long *__restrict__ r,
                           const int *__restrict__ node, const int *__restrict__ idx, int m,
                           int *__restrict__ D2, long long *__restrict__ r2,
-                          int *__restrict__ node2, uint8_t *__restrict__ act2) {
+                          int *__restrict__ node2) {
   const int u = blockIdx.y;
   const int su = idx[u];
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < m; v += gridDim.x * blockDim.x)
@@ -382,15 +630,21 @@ __global__ void k_nj_pack(const int *__restrict__ D, int P, const long long *__r
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     r2[u] = r[su];
     node2[u] = node[su];
-    act2[u] = 1;
   }
 }
 
-// The root: the two active positions joined at the middle of their edge.
-__global__ void k_nj_root(const int *__restrict__ D, int P, const uint8_t *__restrict__ act,
-                          const int *__restrict__ node, int t, int *__restrict__ joins,
-                          double *__restrict__ lengths) {
-  if (threadIdx.x != 0) return;
+// The branch lengths from their numerators (join t of n rows had m = n - t
+// active: over 2 (m - 2), one correctly rounded division), in place, and the
+// root: the two active positions joined at the middle of their edge.
+__global__ void k_nj_finish(const int *__restrict__ D, int P, const uint8_t *__restrict__ act,
+                            const int *__restrict__ node, int n, int *__restrict__ joins,
+                            double *__restrict__ lengths) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, last = n - 2;
+  if (i < 2 * last) {
+    const long long num = __double_as_longlong(lengths[i]);
+    lengths[i] = (double)num / (double)(2 * (long long)(last - (i >> 1)));
+  }
+  if (i != 0) return;
   int a = -1, b = -1;
   for (int k = 0; k < P; ++k)
     if (act[k]) {
@@ -399,10 +653,10 @@ __global__ void k_nj_root(const int *__restrict__ D, int P, const uint8_t *__res
     }
   if (a < 0 || b < 0) return;
   const double half = (double)D[(size_t)a * P + b] / 2.0;
-  joins[2 * t] = node[a];
-  joins[2 * t + 1] = node[b];
-  lengths[2 * t] = half;
-  lengths[2 * t + 1] = half;
+  joins[2 * last] = node[a];
+  joins[2 * last + 1] = node[b];
+  lengths[2 * last] = half;
+  lengths[2 * last + 1] = half;
 }
 
 // The int64 matrix into the int32 one the joins work on; entries beyond the
@@ -436,21 +690,71 @@ __global__ void k_nj_init(long long *__restrict__ r, const int *__restrict__ D, 
   }
 }
 
-// Distances among the merged rows idx[0..m) (device list, null = rows 0..m-1)
-// into the m x m matrix D (device).
-int list_distances(msa_ctx *ctx, const int32_t *idx, int m, long long *D) {
-  const int T = (m + kTile - 1) / kTile;
-  PdistJob job{idx, idx, m, m, true, D, nullptr};
+// Bit planes of a slab of listed rows (list: device, null = rows r0, ...).
+struct Planes {
+  DevBuf lo, hi;
+  int r0 = 0, rows = 0;
+};
+
+int make_planes(msa_ctx *ctx, Planes &p, const int32_t *list, int r0, int rows, int words) {
+  const size_t cells = (size_t)rows * words;
+  const bool wide = ctx->K > 7;
+  TRY(ensure(ctx, p.lo, sizeof(uint4) * cells));
+  if (wide) TRY(ensure(ctx, p.hi, sizeof(uint2) * cells));
+  const int blocks = (int)std::min<size_t>((cells + 31) / 32, 1 << 14);  // four words per warp or more
   ++ctx->launches;
-  k_pdist<<<dim3(T, T), 256, 0, ctx->st>>>(P<uint8_t>(ctx->msa), ctx->W, job);
+  auto fn = wide ? k_planes<true> : k_planes<false>;
+  fn<<<std::max(blocks, 1), 256, 0, ctx->st>>>(P<uint8_t>(ctx->msa), ctx->W, list, r0, rows, words,
+                                               ctx->dSymLut, ctx->K, P<uint4>(p.lo), P<uint2>(p.hi));
   CK(cudaGetLastError());
+  p.r0 = r0;
+  p.rows = rows;
   return MSA_OK;
+}
+
+// Distances of the rows ia[0..nA) (device list, null = rows 0..nA-1) against
+// ib[0..nB): into the matrix D (near null: both lists the same, nA x nA, T =
+// int or long long), or each row of A's nearest row of B into near.  The
+// planes are held a slab of rows at a time, fewer where a device memory limit
+// leaves less.
+template <class T>
+int distances(msa_ctx *ctx, const int32_t *ia, int nA, const int32_t *ib, int nB, T *D,
+              unsigned long long *near) {
+  const int words = (int)((ctx->W + 32 * kPlaneWords - 1) / (32 * kPlaneWords)) * kPlaneWords;
+  int slab = kSlab;
+  if (ctx->dev_limit) {
+    const size_t left = ctx->dev_limit > ctx->dev_bytes ? ctx->dev_limit - ctx->dev_bytes : 0;
+    const size_t per = 2 * sizeof(uint4) * 2 * (size_t)words;  // two slabs' rows
+    while (slab > kTile && (size_t)slab * per > left) slab /= 2;
+  }
+  Planes pa, pb;
+  int rc = [&]() -> int {
+    for (int a0 = 0; a0 < nA; a0 += slab) {
+      const int ra = std::min(slab, nA - a0);
+      TRY(make_planes(ctx, pa, ia, a0, ra, words));
+      for (int b0 = near ? 0 : a0; b0 < nB; b0 += slab) {
+        const int rb = std::min(slab, nB - b0);
+        const bool same = !near && b0 == a0;
+        if (!same && (nB > slab || pb.rows == 0)) TRY(make_planes(ctx, pb, ib, b0, rb, words));
+        Planes &q = same ? pa : pb;
+        PdistJob job{P<uint4>(pa.lo), P<uint4>(q.lo), P<uint2>(pa.hi), P<uint2>(q.hi), words,
+                     ra, rb, a0, b0, (size_t)nA, near};
+        ++ctx->launches;
+        auto fn = ctx->K > 7 ? k_pdist<true, T> : k_pdist<false, T>;
+        fn<<<dim3((rb + kTile - 1) / kTile, (ra + kTile - 1) / kTile), 256, 0, ctx->st>>>(job, D);
+        CK(cudaGetLastError());
+      }
+    }
+    return MSA_OK;
+  }();
+  for (DevBuf *b : {&pa.lo, &pa.hi, &pb.lo, &pb.hi}) release(ctx, *b);
+  return rc;
 }
 
 // Per cluster c of the sample: the smallest (d(t, s) << 32 | s) over sample
 // positions t in c and s outside it (the outgroup: the nearest sample row
 // outside, ties to the smaller row).
-__global__ void k_outgroups(const long long *__restrict__ D, int m, const int32_t *__restrict__ cl,
+__global__ void k_outgroups(const int *__restrict__ D, int m, const int32_t *__restrict__ cl,
                             unsigned long long *__restrict__ key) {
   const int t = blockIdx.y;
   const int c = cl[t];
@@ -468,106 +772,88 @@ __global__ void k_outgroups(const long long *__restrict__ D, int m, const int32_
   if ((threadIdx.x & 31) == 0 && best != ~0ull) atomicMin(&key[c], best);
 }
 
-int tree_distances(msa_ctx *ctx, DevBuf &D) {
-  if (!ctx->merged) return fail(ctx, MSA_ESTATE, "merge the alignment first");
-  const int n = ctx->n;
-  TRY(ensure(ctx, D, sizeof(long long) * (size_t)n * n));
-  return list_distances(ctx, nullptr, n, P<long long>(D));
-}
-
-// Neighbour joining of the n x n matrix in D (device, int64, left as it is).
-int nj_device(msa_ctx *ctx, DevBuf &D, int n, int32_t *joins_out, double *lengths_out) {
+// Row sums and the joins of the n x n int32 matrix in D1 (device; repacked in
+// place of copies as positions retire).  derr must be clear.
+int nj_device(msa_ctx *ctx, DevBuf &D1, int n, int32_t *joins_out, double *lengths_out) {
   if (n < 2) return MSA_OK;
-  DevBuf D1, D2, r, r2, node, node2, act, act2, idx, part, jpart, sel, joins, lengths, tasks;
+  DevBuf D2, r, r2, node, node2, act, idx, joins, lengths, stage, rcopy;
   auto cleanup = [&]() {
-    for (DevBuf *b : {&D1, &D2, &r, &r2, &node, &node2, &act, &act2, &idx, &part, &jpart, &sel, &joins,
-                      &lengths, &tasks})
+    for (DevBuf *b : {&D2, &r, &r2, &node, &node2, &act, &idx, &joins, &lengths, &stage, &rcopy})
       release(ctx, *b);
   };
   int rc = [&]() -> int {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->dev);
-    const int grid = std::max(1, sms) * 8;
-    const int jmax = std::max(1, sms);  // CTAs of a join
     TRY(ensure(ctx, r, sizeof(long long) * n));
     TRY(ensure(ctx, node, sizeof(int) * n));
     TRY(ensure(ctx, act, (size_t)n));
     TRY(ensure(ctx, idx, sizeof(int) * n));
-    TRY(ensure(ctx, part, sizeof(Pick) * grid));
-    TRY(ensure(ctx, sel, sizeof(int) * 2 + 2 * sizeof(unsigned)));
-    TRY(ensure(ctx, jpart, sizeof(long long) * jmax));
+    TRY(ensure(ctx, stage, sizeof(int) * 2 * (size_t)n));
     TRY(ensure(ctx, joins, sizeof(int) * 2 * (size_t)(n - 1)));
     TRY(ensure(ctx, lengths, sizeof(double) * 2 * (size_t)(n - 1)));
-    unsigned *ticket = reinterpret_cast<unsigned *>(P<int>(sel) + 2);
-    CK(cudaMemsetAsync(ticket, 0, 2 * sizeof(unsigned), ctx->st));
-    CK(cudaMemsetAsync(ctx->derr, 0, 2 * sizeof(unsigned), ctx->st));
-    TRY(ensure(ctx, D1, sizeof(int) * (size_t)n * n));
-    ctx->launches += 2;
-    k_nj_narrow<<<grid, 256, 0, ctx->st>>>(P<long long>(D), (size_t)n * n, P<int>(D1), ctx->derr);
+    ++ctx->launches;
+    k_nj_init<<<std::max(1, sms) * 8, 256, 0, ctx->st>>>(P<long long>(r), P<int>(D1), n, P<int>(node),
+                                                         P<uint8_t>(act));
     CK(cudaGetLastError());
-    k_nj_init<<<grid, 256, 0, ctx->st>>>(P<long long>(r), P<int>(D1), n, P<int>(node),
-                                         P<uint8_t>(act));
-    CK(cudaGetLastError());
-    // the Q minimum's warp tasks for a matrix of P positions: tiles of
-    // kRowBlk rows from x0, kColSeg columns from y0 > x0
-    std::vector<int2> htasks;
-    int ntask = 0;
-    auto make_tasks = [&](int Pm) -> int {
-      htasks.clear();
-      for (int x0 = 0; x0 + 1 < Pm; x0 += kRowBlk)
-        for (int y0 = x0 + 1; y0 < Pm; y0 += kColSeg) htasks.push_back(make_int2(x0, y0));
-      ntask = (int)htasks.size();
-      TRY(ensure(ctx, tasks, sizeof(int2) * std::max(ntask, 1)));
-      CK(cudaMemcpyAsync(tasks.p, htasks.data(), sizeof(int2) * ntask, cudaMemcpyHostToDevice, ctx->st));
-      return MSA_OK;
-    };
-    TRY(make_tasks(n));
-    DevBuf *cD = &D1, *cR = &r, *cN = &node, *cA = &act;
-    DevBuf *oD = &D2, *oR = &r2, *oN = &node2, *oA = &act2;
-    int Pn = n, m = n, t = 0;
-    // the Q minimum runs as many CTAs as stay resident (its warps loop over the tiles)
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nj_argmin, kArgThreads, 0);
-    const int aresident = std::min(grid, std::max(1, sms) * std::max(1, per_sm));
-    while (m > 2) {
+    DevBuf *cD = &D1, *cR = &r, *cN = &node;
+    DevBuf *oD = &D2, *oR = &r2, *oN = &node2;
+    int Pn = n, t = 0;
+    while (Pn > 2) {
+      // a large matrix until half of its positions are left, then packed
+      const bool solo = Pn <= kSoloRows;
+      const int grid = solo ? 1 : kJoinCtas, stop = solo ? 2 : std::max(kSoloRows, Pn / 2);
+      const size_t cap = (size_t)(Pn + grid - 1) / grid;
+      const size_t own = cap * (sizeof(long long) + 4 * sizeof(int)) + sizeof(unsigned) * (((size_t)Pn + 31) / 32);
+      const bool rshared = own + sizeof(long long) * (size_t)Pn <= (size_t)kJoinSmem;
+      if (!rshared) TRY(ensure(ctx, rcopy, sizeof(long long) * (size_t)Pn * grid));
+      const size_t smem = own + (rshared ? sizeof(long long) * (size_t)Pn : 0);
+      NjJob job{P<int>(*cD), Pn, stop, t, n, P<long long>(*cR), P<uint8_t>(act), P<int>(*cN),
+                P<int>(joins), P<long long>(lengths), P<int>(stage),
+                rshared ? nullptr : P<long long>(rcopy), ctx->derr};
+      ++ctx->launches;
+      // fewer threads make the block-wide steps of a join cheaper, more keep
+      // more of rows x and y in flight
+      const int threads = solo || Pn <= 1536 ? 256 : Pn <= 8192 ? 512 : 1024;
+      const void *fn = solo ? (const void *)k_nj_joins<1, 256>
+                     : threads == 256 ? (const void *)k_nj_joins<kJoinCtas, 256>
+                     : threads == 512 ? (const void *)k_nj_joins<kJoinCtas, 512>
+                                      : (const void *)k_nj_joins<kJoinCtas, 1024>;
+      CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kJoinSmem));
+      if (grid > 8) CK(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = (unsigned)grid;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)grid);
+      cfg.blockDim = dim3((unsigned)threads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = ctx->st;
+      cfg.attrs = &attr;
+      cfg.numAttrs = grid > 1 ? 1 : 0;
+      void *args[] = {&job};
+      CK(cudaLaunchKernelExC(&cfg, fn, args));
+      t += Pn - stop;
+      if (stop <= 2) break;
+      const int m = stop;
+      TRY(ensure(ctx, *oD, sizeof(int) * (size_t)m * m));
+      TRY(ensure(ctx, *oR, sizeof(long long) * m));
+      TRY(ensure(ctx, *oN, sizeof(int) * m));
       ctx->launches += 2;
-      // a warp per task at least: small matrices take few CTAs
-      const int agrid = std::max(1, std::min(aresident, (ntask + kArgThreads / 32 - 1) / (kArgThreads / 32)));
-      k_nj_argmin<<<agrid, kArgThreads, 0, ctx->st>>>(P<int>(*cD), Pn, P<long long>(*cR),
-                                                     P<uint8_t>(*cA), m, P<int2>(tasks), ntask,
-                                                     P<Pick>(part), ticket, P<int>(sel));
+      k_nj_index<<<1, 1024, 0, ctx->st>>>(P<uint8_t>(act), Pn, P<int>(idx));
       CK(cudaGetLastError());
-      const int jgrid = std::max(1, std::min(jmax, (Pn + kJoinThreads - 1) / kJoinThreads));
-      k_nj_join<<<jgrid, kJoinThreads, 0, ctx->st>>>(P<int>(*cD), Pn, P<long long>(*cR),
-                                                     P<uint8_t>(*cA), P<int>(*cN), m, P<int>(sel), t,
-                                                     n, P<int>(joins), P<double>(lengths),
-                                                     P<long long>(jpart), ticket + 1, ctx->derr);
+      k_nj_pack<<<dim3((m + 255) / 256, m), 256, 0, ctx->st>>>(P<int>(*cD), Pn, P<long long>(*cR), P<int>(*cN),
+                                                               P<int>(idx), m, P<int>(*oD),
+                                                               P<long long>(*oR), P<int>(*oN));
       CK(cudaGetLastError());
-      --m;
-      ++t;
-      if (m > 2 && Pn >= 512 && 4 * m <= 3 * Pn) {  // pack to the active positions
-        TRY(ensure(ctx, *oD, sizeof(int) * (size_t)m * m));
-        TRY(ensure(ctx, *oR, sizeof(long long) * m));
-        TRY(ensure(ctx, *oN, sizeof(int) * m));
-        TRY(ensure(ctx, *oA, (size_t)m));
-        ctx->launches += 2;
-        k_nj_index<<<1, 1024, 0, ctx->st>>>(P<uint8_t>(*cA), Pn, P<int>(idx));
-        CK(cudaGetLastError());
-        k_nj_pack<<<dim3((m + 255) / 256, m), 256, 0, ctx->st>>>(
-            P<int>(*cD), Pn, P<long long>(*cR), P<int>(*cN), P<int>(idx), m, P<int>(*oD),
-            P<long long>(*oR), P<int>(*oN), P<uint8_t>(*oA));
-        CK(cudaGetLastError());
-        std::swap(cD, oD);
-        std::swap(cR, oR);
-        std::swap(cN, oN);
-        std::swap(cA, oA);
-        Pn = m;
-        TRY(make_tasks(Pn));
-      }
+      std::swap(cD, oD);
+      std::swap(cR, oR);
+      std::swap(cN, oN);
+      Pn = m;
     }
     ++ctx->launches;
-    k_nj_root<<<1, 32, 0, ctx->st>>>(P<int>(*cD), Pn, P<uint8_t>(*cA), P<int>(*cN), t,
-                                      P<int>(joins), P<double>(lengths));
+    k_nj_finish<<<(2 * n + 255) / 256, 256, 0, ctx->st>>>(P<int>(*cD), Pn, P<uint8_t>(act), P<int>(*cN), n,
+                                                         P<int>(joins), P<double>(lengths));
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(joins_out, joins.p, sizeof(int) * 2 * (size_t)(n - 1), cudaMemcpyDefault,
                        ctx->st));
@@ -577,6 +863,26 @@ int nj_device(msa_ctx *ctx, DevBuf &D, int n, int32_t *joins_out, double *length
     return MSA_OK;
   }();
   cleanup();
+  return rc;
+}
+
+// Neighbour joining of the merged rows idx[0..m) (device list, null = all):
+// their distances into D (int32, m x m), then the joins on a copy of D where
+// keep is set (the caller needs the distances), else on D itself.
+int nj_rows(msa_ctx *ctx, const int32_t *idx, int m, DevBuf &D, bool keep, int32_t *joins_out,
+            double *lengths_out) {
+  TRY(ensure(ctx, D, sizeof(int) * (size_t)m * m));
+  TRY(distances<int>(ctx, idx, m, idx, m, P<int>(D), nullptr));
+  if (m < 2) return MSA_OK;
+  CK(cudaMemsetAsync(ctx->derr, 0, 2 * sizeof(unsigned), ctx->st));
+  if (!keep) return nj_device(ctx, D, m, joins_out, lengths_out);
+  DevBuf C;
+  int rc = [&]() -> int {
+    TRY(ensure(ctx, C, sizeof(int) * (size_t)m * m));
+    CK(cudaMemcpyAsync(C.p, D.p, sizeof(int) * (size_t)m * m, cudaMemcpyDeviceToDevice, ctx->st));
+    return nj_device(ctx, C, m, joins_out, lengths_out);
+  }();
+  release(ctx, C);
   return rc;
 }
 
@@ -715,11 +1021,9 @@ int cluster_tree(msa_ctx *ctx, const std::vector<int32_t> &S, int cap, int32_t *
     // 1. the sample tree, midpoint-rooted
     TRY(ensure(ctx, dlist, sizeof(int32_t) * std::max(n, 1)));
     CK(cudaMemcpyAsync(dlist.p, S.data(), sizeof(int32_t) * m, cudaMemcpyHostToDevice, ctx->st));
-    TRY(ensure(ctx, dS, sizeof(long long) * (size_t)m * m));
-    TRY(list_distances(ctx, P<int32_t>(dlist), m, P<long long>(dS)));
     std::vector<int32_t> sj(2 * std::max(m - 1, 0));
     std::vector<double> sl(2 * std::max(m - 1, 0));
-    if (m > 1) TRY(nj_device(ctx, dS, m, sj.data(), sl.data()));
+    TRY(nj_rows(ctx, P<int32_t>(dlist), m, dS, true, sj.data(), sl.data()));
     CK(cudaStreamSynchronize(ctx->st));
     Kids skids;
     int sroot = 0;
@@ -772,11 +1076,7 @@ int cluster_tree(msa_ctx *ctx, const std::vector<int32_t> &S, int cap, int32_t *
     {
       TRY(ensure(ctx, dnear, sizeof(unsigned long long) * n));
       CK(cudaMemsetAsync(dnear.p, 0xff, sizeof(unsigned long long) * n, ctx->st));
-      const int TA = (n + kTile - 1) / kTile, TB = (m + kTile - 1) / kTile;
-      PdistJob job{nullptr, P<int32_t>(dlist), n, m, false, nullptr, P<unsigned long long>(dnear)};
-      ++ctx->launches;
-      k_pdist<<<dim3(TB, TA), 256, 0, ctx->st>>>(P<uint8_t>(ctx->msa), ctx->W, job);
-      CK(cudaGetLastError());
+      TRY(distances<int>(ctx, nullptr, n, P<int32_t>(dlist), m, nullptr, P<unsigned long long>(dnear)));
       std::vector<unsigned long long> near(n);
       CK(cudaMemcpyAsync(near.data(), dnear.p, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost, ctx->st));
       CK(cudaStreamSynchronize(ctx->st));
@@ -791,7 +1091,7 @@ int cluster_tree(msa_ctx *ctx, const std::vector<int32_t> &S, int cap, int32_t *
       CK(cudaMemcpyAsync(dcl.p, leaf_cl.data(), sizeof(int32_t) * m, cudaMemcpyHostToDevice, ctx->st));
       CK(cudaMemsetAsync(dkey.p, 0xff, sizeof(unsigned long long) * q, ctx->st));
       ++ctx->launches;
-      k_outgroups<<<dim3((m + 255) / 256, m), 256, 0, ctx->st>>>(P<long long>(dS), m, P<int32_t>(dcl),
+      k_outgroups<<<dim3((m + 255) / 256, m), 256, 0, ctx->st>>>(P<int>(dS), m, P<int32_t>(dcl),
                                                                  P<unsigned long long>(dkey));
       CK(cudaGetLastError());
       std::vector<unsigned long long> key(q);
@@ -818,11 +1118,9 @@ int cluster_tree(msa_ctx *ctx, const std::vector<int32_t> &S, int cap, int32_t *
       if (u > kMaxTreeRows) return fail(ctx, MSA_ERANGE, "a cluster of %d rows (at most %d)", u, kMaxTreeRows);
       std::vector<int32_t> U32(U.begin(), U.end());
       CK(cudaMemcpyAsync(dlist.p, U32.data(), sizeof(int32_t) * u, cudaMemcpyHostToDevice, ctx->st));
-      TRY(ensure(ctx, dS2, sizeof(long long) * (size_t)u * u));
-      TRY(list_distances(ctx, P<int32_t>(dlist), u, P<long long>(dS2)));
       std::vector<int32_t> cj(2 * (u - 1));
       std::vector<double> cl(2 * (u - 1));
-      TRY(nj_device(ctx, dS2, u, cj.data(), cl.data()));
+      TRY(nj_rows(ctx, P<int32_t>(dlist), u, dS2, false, cj.data(), cl.data()));
       CK(cudaStreamSynchronize(ctx->st));
       Kids ck;
       int croot;
@@ -909,10 +1207,12 @@ int msa_tree_distances(msa_ctx *ctx, int64_t *dist_out) {
   TRY(set_device(ctx));
   DevBuf D;
   int rc = [&]() -> int {
-    stage_begin(ctx, ST_TREE);
-    TRY(tree_distances(ctx, D));
-    stage_end(ctx, ST_TREE);
+    if (!ctx->merged) return fail(ctx, MSA_ESTATE, "merge the alignment first");
     const size_t n = ctx->n;
+    TRY(ensure(ctx, D, sizeof(long long) * n * n));
+    stage_begin(ctx, ST_TREE);
+    TRY(distances<long long>(ctx, nullptr, ctx->n, nullptr, ctx->n, P<long long>(D), nullptr));
+    stage_end(ctx, ST_TREE);
     CK(cudaMemcpyAsync(dist_out, D.p, sizeof(long long) * n * n, cudaMemcpyDefault, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
     stage_collect(ctx, ST_TREE);
@@ -926,18 +1226,27 @@ int msa_nj(msa_ctx *ctx, const int64_t *dist, int64_t n, int32_t *joins_out, dou
   if (!ctx || !dist || n < 1 || n > kMaxTreeRows || ((!joins_out || !lengths_out) && n > 1))
     return MSA_EINVAL;
   TRY(set_device(ctx));
-  DevBuf D;
+  DevBuf D, D1;
   int rc = [&]() -> int {
-    TRY(ensure(ctx, D, sizeof(long long) * (size_t)n * n));
-    CK(cudaMemcpyAsync(D.p, dist, sizeof(long long) * (size_t)n * n, cudaMemcpyDefault, ctx->st));
+    const size_t count = (size_t)n * n;
+    TRY(ensure(ctx, D, sizeof(long long) * count));
+    CK(cudaMemcpyAsync(D.p, dist, sizeof(long long) * count, cudaMemcpyDefault, ctx->st));
     stage_begin(ctx, ST_TREE);
-    TRY(nj_device(ctx, D, (int)n, joins_out, lengths_out));
+    if (n > 1) {
+      TRY(ensure(ctx, D1, sizeof(int) * count));
+      CK(cudaMemsetAsync(ctx->derr, 0, 2 * sizeof(unsigned), ctx->st));
+      ++ctx->launches;
+      k_nj_narrow<<<1216, 256, 0, ctx->st>>>(P<long long>(D), count, P<int>(D1), ctx->derr);
+      CK(cudaGetLastError());
+      TRY(nj_device(ctx, D1, (int)n, joins_out, lengths_out));
+    }
     stage_end(ctx, ST_TREE);
     CK(cudaStreamSynchronize(ctx->st));
     stage_collect(ctx, ST_TREE);
     return MSA_OK;
   }();
   release(ctx, D);
+  release(ctx, D1);
   return rc;
 }
 
@@ -948,9 +1257,9 @@ int msa_nj_tree(msa_ctx *ctx, int32_t *joins_out, double *lengths_out) {
   TRY(set_device(ctx));
   DevBuf D;
   int rc = [&]() -> int {
+    if (!ctx->merged) return fail(ctx, MSA_ESTATE, "merge the alignment first");
     stage_begin(ctx, ST_TREE);
-    TRY(tree_distances(ctx, D));
-    TRY(nj_device(ctx, D, ctx->n, joins_out, lengths_out));
+    TRY(nj_rows(ctx, nullptr, ctx->n, D, false, joins_out, lengths_out));
     stage_end(ctx, ST_TREE);
     CK(cudaStreamSynchronize(ctx->st));
     stage_collect(ctx, ST_TREE);

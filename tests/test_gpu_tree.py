@@ -137,3 +137,42 @@ def test_clustered_tree_degenerate_cuts():
             joins, lengths, cluster = b.msa_nj_cluster_tree(h, sample, cap)
             assert (joins == oj).all() and (lengths == ol).all() and (cluster == oc).all()
             assert T.splits(joins, lengths, 90) == nj_splits
+
+
+@pytest.mark.parametrize("n", [5, 33, 511, 513, 1030])
+@pytest.mark.parametrize("kind", ["ties", "negative", "star"])
+def test_nj_around_the_launch_sizes(n, kind):
+    """Matrices at the sizes where the joins move from one CTA to a grid of
+    them and where the matrix is packed: small integers (almost every Q ties),
+    entries of both signs, and near-equal distances."""
+    if n > 600 and kind == "negative":
+        pytest.skip("the oracle's time")
+    b = binding()
+    rng = np.random.default_rng(n)
+    lo, hi = {"ties": (1, 4), "negative": (-(1 << 19), 1 << 19), "star": (500000, 540000)}[kind]
+    D = np.triu(rng.integers(lo, hi, size=(n, n)).astype(np.int64), 1)
+    D = D + D.T
+    oj, ol = T.nj(D)
+    with any_ctx() as h:
+        joins, lengths = b.msa_nj(h, D)
+    assert (joins == oj).all() and (lengths == ol).all()
+
+
+@pytest.mark.parametrize("kind", ["protein", "dna"])
+@pytest.mark.parametrize("n,length", [(3, 1), (64, 31), (65, 33), (130, 479), (5, 481), (66, 965)])
+def test_distances_around_the_tile_sizes(kind, n, length):
+    """Merged rows of about `length` columns (words of 32, steps of 480) and
+    row counts around the 64-row tiles, with three and five symbol planes."""
+    from seqgen import blosum62, dna_matrix, pack_sequences
+    b = binding()
+    rng = np.random.default_rng(length)
+    alph, M = blosum62() if kind == "protein" else dna_matrix()
+    pool = np.frombuffer(alph.encode(), dtype=np.uint8)
+    letters, offsets = pack_sequences(
+        [rng.choice(pool, size=max(1, length - int(rng.integers(0, 3)))) for _ in range(n)])
+    with make_ctx(alph, M, 11, 1) as h:
+        b.msa_load(h, letters, offsets)
+        b.msa_align_to_center(h, 0)
+        rows, _ = b.msa_merge_gaps(h)
+        d = b.msa_tree_distances(h)
+    assert (d == T.msa_distances(rows)).all()
