@@ -343,13 +343,29 @@ int align_subset_local(msa_ctx *ctx, int kc, const std::vector<int32_t> &subj, f
     TRY(ensure(ctx, vl, sizeof(int32_t) * nv));
     TRY(ensure(ctx, vp, sizeof(int32_t) * nv));
     TRY(ensure(ctx, vo, sizeof(int64_t) * nv));
-    TRY(ensure(ctx, ctx->codes, (size_t)std::max<int64_t>(acc, 8)));
-    TRY(ensure(ctx, ctx->best, sizeof(unsigned long long) * nv));
     CK(cudaMemcpyAsync(vs.p, vstart.data(), sizeof(int64_t) * nv, cudaMemcpyHostToDevice, ctx->st));
     CK(cudaMemcpyAsync(vl.p, vlen.data(), sizeof(int32_t) * nv, cudaMemcpyHostToDevice, ctx->st));
     CK(cudaMemcpyAsync(vp.p, vperm.data(), sizeof(int32_t) * nv, cudaMemcpyHostToDevice, ctx->st));
     CK(cudaMemcpyAsync(vo.p, offs.data(), sizeof(int64_t) * nv, cudaMemcpyHostToDevice, ctx->st));
     const SeqSet vss{P<uint8_t>(ctx->res), P<int64_t>(vs), P<int32_t>(vl), nv};
+    double total = 0.0;
+    int vmax = 0, few = 0;
+    for (int v = 0; v + 1 < nv; ++v) {
+      total += vlen[v];
+      vmax = std::max(vmax, vlen[v]);
+    }
+    if (align_few_wins(ctx, Lc, nv - 1, total / (nv - 1), vmax, &few)) {
+      cudaEvent_t e0 = ctx->ev[2 * ST_TRACE], e1 = ctx->ev[2 * ST_TRACE + 1];
+      CK(cudaEventRecord(e0, ctx->st));
+      TRY(align_few(ctx, vss, nv - 1, nv - 1, P<int32_t>(vp), Lc, vmax, few));
+      CK(cudaEventRecord(e1, ctx->st));
+      CK(cudaStreamSynchronize(ctx->st));
+      float t = 0.f;
+      if (cudaEventElapsedTime(&t, e0, e1) == cudaSuccess) ms += t;
+      return MSA_OK;
+    }
+    TRY(ensure(ctx, ctx->codes, (size_t)std::max<int64_t>(acc, 8)));
+    TRY(ensure(ctx, ctx->best, sizeof(unsigned long long) * nv));
     const Scoring sc = scoring(ctx);
     const int smem = codes_smem_bytes(ctx->K, npass * G * R);
     const int cta = align_cta(ctx, G, packed);

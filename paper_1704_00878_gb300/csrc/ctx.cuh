@@ -49,6 +49,7 @@ struct msa_ctx {
 
   // the loaded set (sorted by length, ascending, stable)
   int n = 0, maxlen = 0;
+  int64_t residues = 0;
   std::vector<int32_t> len_sorted, perm, inv;
   std::vector<int64_t> pstart;
   // host scratch kept between calls (a fresh multi-megabyte vector per call
@@ -100,6 +101,7 @@ struct msa_ctx {
   size_t codes_budget = (size_t)32 << 30;
   int align_group = 0;  // lanes per subject group of the codes kernels, 0 = modelled choice
   bool align_group_fixed = false;  // set by msa_set_align_group: every light pass uses it too
+  bool align_tuning = false;       // msa_align_autotune is timing the codes kernels
   int align_int32 = 0;  // 1: the alignment uses int32 cells even where packed ones fit
   int align_threads = 0;  // CTA size of the packed codes kernel, 0 = kCodes2Threads
   // traceback-light alignment (MSA_ALIGN_BOX): per position of its passes the
@@ -161,6 +163,11 @@ int check_derr(msa_ctx *ctx, unsigned *bits = nullptr);
 // cell precision and lanes per group of the alignment to a center of length Lc
 bool align_packed(msa_ctx *ctx, int Lc);
 int align_lanes(msa_ctx *ctx, int Lc, bool packed);
+// the few-subject kernel: whether it is modelled faster for n subjects (and
+// its grid), and the alignment of a set's first n entries to entry kc with it
+bool align_few_wins(msa_ctx *ctx, int Lc, int n, double mean_len, int max_len, int *grid_out);
+int align_few(msa_ctx *ctx, const SeqSet &ss, int kc, int n, const int32_t *perm, int Lc, int max_len,
+              int grid);
 // CTA size of the codes kernel for this group width and precision
 int align_cta(msa_ctx *ctx, int G, bool packed);
 SeqSet seqset(msa_ctx *ctx);

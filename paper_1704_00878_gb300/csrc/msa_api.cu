@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "msa.h"
+#include "few.cuh"
 #include "msa_kernels.cuh"
 #include "sw_kernels.cuh"
 
@@ -271,9 +272,7 @@ static bool codes_packed(msa_ctx *ctx, int Lc) {
 // group size of the alignment kernel for this set and a center of length Lc
 static int align_group(msa_ctx *ctx, int Lc, bool packed) {
   if (ctx->align_group > 0) return ctx->align_group;
-  double total = 0.0;
-  for (int L : ctx->len_sorted) total += L;
-  return codes_group(Lc, packed, ctx->K, ctx->n, ctx->n ? total / ctx->n : 0.0, ctx->maxlen);
+  return codes_group(Lc, packed, ctx->K, ctx->n, ctx->n ? (double)ctx->residues / ctx->n : 0.0, ctx->maxlen);
 }
 
 bool align_packed(msa_ctx *ctx, int Lc) { return codes_packed(ctx, Lc); }
@@ -282,6 +281,69 @@ int align_cta(msa_ctx *ctx, int G, bool packed) {
                                                                       : kCodes2Threads;
 }
 int align_lanes(msa_ctx *ctx, int Lc, bool packed) { return align_group(ctx, Lc, packed); }
+
+// The few-subject kernel takes the alignment where it is modelled faster than
+// the codes kernels and their traceback: their groups' steps (codes_group's
+// estimate; a step of 16 rows takes 0.58 us packed, 0.88 in int32 cells,
+// whether one warp or two share a scheduler) and a walk of about 0.65 us per
+// center residue, one thread per subject.  Measured on both sides of the line
+// (us, few / codes): 3,000 sequences of 60 residues 63 / 183, 10,000 171 / 183
+// (codes); 3,000 of 150 212 / 409, 10,000 624 / 422; 3,000 of 350 626 / 915,
+// 10,000 1,985 / 1,430; 1,000 of 1,000 1,586 / 4,135, 3,000 4,561 / 4,488;
+// 1,000 of 2,500 11,018 / 21,273.
+bool align_few_wins(msa_ctx *ctx, int Lc, int n, double mean_len, int max_len, int *grid_out) {
+  *grid_out = 0;
+  if (ctx->align_group_fixed || ctx->align_tuning) return false;
+  if ((double)n * Lc * mean_len > 4e10) return false;  // (30 ms of codes: far beyond the line)
+  const bool packed = codes_packed(ctx, Lc);
+  const int G = align_group(ctx, Lc, packed);
+  const int npass = (Lc + G * kCodesR - 1) / (G * kCodesR);
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->dev);
+  const double warps = 8.0 * std::max(sms, 1), units = packed ? std::ceil(n / 2.0) : n;
+  const double steps = std::max(units * G / 32 * npass * (mean_len + G - 1) / warps, npass * (max_len + G - 1.0));
+  const double codes = steps * (packed ? 0.58 : 0.88) + 0.65 * std::min((double)Lc, mean_len);
+  const int grid = few_grid(ctx->K, Lc, max_len, n);
+  if (grid < 1 || few_cost(Lc, n, mean_len, grid, sms) >= codes) return false;
+  *grid_out = grid;
+  return true;
+}
+
+// Subjects [0, n) of ss against its entry kc in at most `grid` CTAs, rows to
+// perm's input indices; queued on the context's stream.
+int align_few(msa_ctx *ctx, const SeqSet &ss, int kc, int n, const int32_t *perm, int Lc, int max_len,
+              int grid) {
+  const size_t slot = few_slot_codes(Lc, max_len), bytes = slot * sizeof(uint16_t);
+  if (bytes * grid > ctx->codes.cap || bytes * grid > ctx->codes_budget) {
+    size_t free_b = 0, total_b = 0;
+    CK(cudaMemGetInfo(&free_b, &total_b));
+    size_t budget = std::min(ctx->codes_budget, free_b / 2);
+    if (ctx->dev_limit) budget = std::min(budget, ctx->dev_limit > ctx->dev_bytes ? (ctx->dev_limit - ctx->dev_bytes) / 2 : 0);
+    budget = std::max(budget, std::min(ctx->codes.cap, ctx->codes_budget));
+    grid = std::max(1, (int)std::min<size_t>(grid, budget / bytes));
+  }
+  TRY(ensure(ctx, ctx->codes, bytes * grid));
+  FewJob job{};
+  job.center = kc;
+  job.se = n;
+  job.codes = P<uint16_t>(ctx->codes);
+  job.slot_codes = slot;
+  if (few_rounds(Lc)) {
+    TRY(ensure(ctx, ctx->scratch, sizeof(int2) * (size_t)grid * max_len));
+    job.edge = P<int2>(ctx->scratch);
+    job.edge_cols = max_len;
+  }
+  job.counter = ctx->dcounter;
+  job.perm = perm;
+  job.ins = P<uint16_t>(ctx->ins);
+  job.occ = P<uint8_t>(ctx->occ);
+  job.seg = P<int32_t>(ctx->seg);
+  job.score = P<int32_t>(ctx->score);
+  job.err = ctx->derr;
+  CK(cudaMemsetAsync(ctx->dcounter, 0, sizeof(unsigned long long), ctx->st));
+  CK((++ctx->launches, launch_align_few)(ss, scoring(ctx), job, Lc, max_len, grid, ctx->st));
+  return MSA_OK;
+}
 
 bool use_packed(msa_ctx *ctx, int Lq) {
   if (ctx->precision == MSA_INT32 || ctx->smin + ctx->o < 0) return false;
@@ -1206,6 +1268,7 @@ int msa_load(msa_ctx *ctx, const uint8_t *letters, const int64_t *offsets, int64
     pos += round_up_i64(ctx->len_sorted[k], 16) + MSA_SEQ_TAIL;
   }
   const int64_t total = offsets[n];
+  ctx->residues = total;
   TRY(ensure(ctx, ctx->res, pos));
   TRY(ensure(ctx, ctx->d_pstart, sizeof(int64_t) * n));
   TRY(ensure(ctx, ctx->d_len, sizeof(int32_t) * n));
@@ -1452,6 +1515,26 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
     ctx->light_used = true;
     ctx->aligned = true;
     return MSA_OK;
+  }
+
+  {
+    int few = 0;
+    if (align_few_wins(ctx, Lc, n, (double)ctx->residues / n, ctx->maxlen, &few)) {
+      stage_begin(ctx, ST_ALIGN);
+      TRY(align_few(ctx, seqset(ctx), kc, n, P<int32_t>(ctx->d_perm), Lc, ctx->maxlen, few));
+      stage_end(ctx, ST_ALIGN);
+      TRY(check_derr(ctx));
+      stage_collect(ctx, ST_ALIGN);
+      ctx->stage_ms[ST_ALIGN_K] = ctx->stage_ms[ST_ALIGN];
+      ctx->stage_ms[ST_TRACE] = 0.f;  // part of the same launch
+      ctx->cells[1] = ctx->residues * Lc;
+      if (scores_out) {
+        CK(cudaMemcpyAsync(scores_out, ctx->score.p, sizeof(int32_t) * n, cudaMemcpyDefault, ctx->st));
+        CK(cudaStreamSynchronize(ctx->st));
+      }
+      ctx->aligned = true;
+      return MSA_OK;
+    }
   }
 
   // batches of subjects (sorted order) whose codes fit the budget; when all
@@ -1842,9 +1925,10 @@ int msa_align_autotune(msa_ctx *ctx, int64_t center, double *rates_out, int32_t 
   struct ModeGuard {
     msa_ctx *c;
     int saved;
-    ~ModeGuard() { c->align_mode = saved; }
+    ~ModeGuard() { c->align_mode = saved; c->align_tuning = false; }
   } guard{ctx, ctx->align_mode};
   ctx->align_mode = MSA_ALIGN_FULL;
+  ctx->align_tuning = true;
   // rows: packed cells in 256-thread CTAs, int32 cells, packed cells in
   // 384-thread CTAs (groups of 8 lanes and more)
   double rates[3][kAlignWidths] = {};
