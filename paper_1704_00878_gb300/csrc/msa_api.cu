@@ -101,60 +101,108 @@ SeqSet seqset(msa_ctx *ctx) {
 }
 Scoring scoring(msa_ctx *ctx) { return Scoring{ctx->dM, ctx->K, ctx->o, ctx->e}; }
 
+static int sat_thresh(msa_ctx *ctx);
+
 // ------------------------------------------------------------ pair scores
-// Scores of (a, b) pairs given in sorted indices, int32 cells.  dst[x] is the
-// output slot of pair x.  Pairs are grouped by the query's pass height and
-// ordered by subject length so the groups of a warp stay in step.
+// Scores of (a, b) pairs given in sorted indices.  dst[x] is the output slot
+// of pair x.  The shorter sequence of a pair takes the rows (scores are
+// symmetric, as the matrix is).  Pairs whose scores cannot reach the int16
+// limit (min length * smax) run packed, two per group; the rest, and every
+// pair under MSA_INT32, in int32 cells.  Each class is ordered by passes, then
+// columns, longest first, so the pairs of a group and the groups of a warp
+// stay in step and the last warps have the least to do.
 int run_pairs(msa_ctx *ctx, const std::vector<int2> &pairs_in, const std::vector<int32_t> &dst_in,
               int32_t *d_out) {
   const int np = (int)pairs_in.size();
   if (np == 0) return MSA_OK;
-  std::vector<int32_t> order(np);
-  std::iota(order.begin(), order.end(), 0);
-  const int short_rows = pairs_rows(8);
-  auto before = [&](int x, int y) {
-    const int ax = ctx->len_sorted[pairs_in[x].x] > short_rows;
-    const int ay = ctx->len_sorted[pairs_in[y].x] > short_rows;
-    if (ax != ay) return ax < ay;
-    const int lx = ctx->len_sorted[pairs_in[x].y], ly = ctx->len_sorted[pairs_in[y].y];
-    return lx < ly;
-  };
-  // (self pairs of the sorted set arrive in order already)
-  if (!std::is_sorted(order.begin(), order.end(), before))
-    std::stable_sort(order.begin(), order.end(), before);
+  const int32_t *len = ctx->len_sorted.data();
+  const bool can_pack = ctx->precision != MSA_INT32 && ctx->smin + ctx->o >= 0 && pairs_packed_fits(ctx->K);
+  const long long limit = sat_thresh(ctx);
+  const int smax = std::max(ctx->smax, 0);
+  auto packs = [&](int shorter) { return can_pack && (long long)shorter * smax <= limit; };
+  // classes: packed in 32, 16 and 8 lanes -- the narrowest group that holds the
+  // rows in one pass: a call with 60,000 pairs of 50-2,000 residues took 4.2 ms
+  // with 32 lanes for all, 7.5 with 8 (a 2,000-residue pair's 16
+  // passes outlast the rest), 3.7 so --, int32 in 32 and 8; key: class,
+  // then passes and columns descending (radix sort by the columns, then by
+  // class and passes)
+  constexpr int kClasses = 5, kCols = MSA_MAX_LEN + 1, kTop = kClasses << 10;
+  static const int class_g[kClasses] = {32, 16, 8, 32, 8};
+  const int rows8 = pairs_rows(8), rows16 = pairs_rows(16);
   std::vector<int2> pr(np);
-  std::vector<int32_t> dst(np);
-  int n_short = 0;
+  std::vector<int32_t> hi(np), cols(np), ord(np), tmp(np);
+  std::vector<int32_t> count(std::max(kCols, kTop) + 1, 0);
+  int n_class[kClasses] = {};
   for (int x = 0; x < np; ++x) {
-    pr[x] = pairs_in[order[x]];
-    dst[x] = dst_in[order[x]];
-    if (ctx->len_sorted[pr[x].x] <= short_rows) ++n_short;
+    int2 p = pairs_in[x];
+    if (len[p.x] > len[p.y]) std::swap(p.x, p.y);
+    pr[x] = p;
+    const int La = len[p.x];
+    const int cls = packs(La) ? (La > rows16 ? 0 : La > rows8 ? 1 : 2) : (La > rows8 ? 3 : 4);
+    hi[x] = (cls << 10) + 1023 - (La + 511) / 512;
+    cols[x] = MSA_MAX_LEN - len[p.y];
+    ++n_class[cls];
+    ++count[cols[x] + 1];
+  }
+  for (int c = 1; c <= kCols; ++c) count[c] += count[c - 1];
+  for (int x = 0; x < np; ++x) tmp[count[cols[x]]++] = x;
+  std::fill(count.begin(), count.end(), 0);
+  for (int x = 0; x < np; ++x) ++count[hi[x] + 1];
+  for (int c = 1; c <= kTop; ++c) count[c] += count[c - 1];
+  for (int y = 0; y < np; ++y) ord[count[hi[tmp[y]]]++] = tmp[y];
+  std::vector<int2> sorted(np);
+  for (int y = 0; y < np; ++y) {
+    sorted[y] = pr[ord[y]];
+    tmp[y] = dst_in[ord[y]];
   }
   TRY(ensure(ctx, ctx->pairs, sizeof(int2) * np));
   TRY(ensure(ctx, ctx->pair_dst, sizeof(int32_t) * np));
-  CK(cudaMemcpyAsync(ctx->pairs.p, pr.data(), sizeof(int2) * np, cudaMemcpyHostToDevice, ctx->st));
-  CK(cudaMemcpyAsync(ctx->pair_dst.p, dst.data(), sizeof(int32_t) * np, cudaMemcpyHostToDevice,
-                     ctx->st));
+  CK(cudaMemcpyAsync(ctx->pairs.p, sorted.data(), sizeof(int2) * np, cudaMemcpyHostToDevice, ctx->st));
+  CK(cudaMemcpyAsync(ctx->pair_dst.p, tmp.data(), sizeof(int32_t) * np, cudaMemcpyHostToDevice, ctx->st));
   const SeqSet ss = seqset(ctx);
   const Scoring sc = scoring(ctx);
-  for (int part = 0; part < 2; ++part) {
-    const int G = part == 0 ? 8 : 32;
-    const int b = part == 0 ? 0 : n_short, e = part == 0 ? n_short : np;
-    if (e <= b) continue;
-    const int grid = pairs_grid(G);
-    const size_t scr = (size_t)grid * (256 / G) * 2 * ctx->maxlen * sizeof(int2);
-    TRY(ensure(ctx, ctx->scratch, scr));
-    CK(cudaMemsetAsync(ctx->dcounter, 0, sizeof(unsigned long long), ctx->st));
+  // one launch per class, on the context's stream and the two private ones
+  // in turn, so a class's last long pairs overlap the next class; each has
+  // its own counter and boundary rows
+  int used = 0, grids[kClasses] = {};
+  size_t rows_off[kClasses + 1] = {};
+  for (int cls = 0; cls < kClasses; ++cls) {
+    const int G = class_g[cls], NG = 256 / G, units = cls < 3 ? (n_class[cls] + 1) / 2 : n_class[cls];
+    if (units > 0) {
+      grids[cls] = std::min(pairs_grid(G, cls < 3, ctx->K), (units + NG - 1) / NG);
+      ++used;
+    }
+    // (packed classes 1 and 2 hold their rows in one pass)
+    rows_off[cls + 1] = rows_off[cls] + (cls == 1 || cls == 2 || cls == 4 ? 0 : (size_t)grids[cls] * NG * 2 * ctx->maxlen);
+  }
+  TRY(ensure(ctx, ctx->scratch, sizeof(int2) * rows_off[kClasses]));
+  TRY(ensure(ctx, ctx->counters, sizeof(unsigned long long) * kClasses));
+  CK(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long) * kClasses, ctx->st));
+  const cudaStream_t lanes[3] = {ctx->st, ctx->cap_st, ctx->cap_st2};
+  if (used > 1) {
+    CK(cudaEventRecord(ctx->cap_fork, ctx->st));
+    for (int k = 1; k < std::min(used, 3); ++k) CK(cudaStreamWaitEvent(lanes[k], ctx->cap_fork, 0));
+  }
+  cudaError_t err = cudaSuccess;
+  for (int cls = 0, b = 0, k = 0; cls < kClasses; b += n_class[cls], ++cls) {
+    if (n_class[cls] == 0) continue;
     PairJob job;
     job.pairs = P<int2>(ctx->pairs) + b;
     job.dst = P<int32_t>(ctx->pair_dst) + b;
     job.out = d_out;
-    job.npairs = e - b;
-    job.counter = ctx->dcounter;
-    job.scratch = P<int2>(ctx->scratch);
+    job.npairs = n_class[cls];
+    job.counter = P<unsigned long long>(ctx->counters) + cls;
+    job.scratch = P<int2>(ctx->scratch) + rows_off[cls];
     job.scratch_cols = ctx->maxlen;
-    CK((++ctx->launches, launch_pairs)(G, ss, sc, job, grid, ctx->st));
+    if (err == cudaSuccess)
+      err = (++ctx->launches, launch_pairs)(class_g[cls], cls < 3, ss, sc, job, grids[cls], lanes[k++ % 3]);
   }
+  if (used > 1)  // the context's stream goes on when all of them are done
+    for (int k = 1; k < std::min(used, 3); ++k) {
+      CK(cudaEventRecord(ctx->cap_join, lanes[k]));
+      CK(cudaStreamWaitEvent(ctx->st, ctx->cap_join, 0));
+    }
+  CK(err);
   return MSA_OK;
 }
 
@@ -259,7 +307,7 @@ int choose_variant(msa_ctx *ctx, int Lq, int Ls_est, bool packed) {
 // int16 lanes need every biased score s + o >= 0 (the lane-local add) and,
 // under MSA_AUTO, an a-priori bound on any local score of a sequence of
 // length Lq that stays below the overflow guard.
-int sat_thresh(msa_ctx *ctx) { return ctx->sat_limit - ctx->smax - ctx->o; }
+static int sat_thresh(msa_ctx *ctx) { return ctx->sat_limit - ctx->smax - ctx->o; }
 
 // int16 lanes hold every value of the alignment to a center of length Lc:
 // H <= Lc * smax, and the biased P = H + s + o never passes Lc * smax + smax + o.

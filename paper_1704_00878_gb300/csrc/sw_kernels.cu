@@ -28,8 +28,9 @@
 
 namespace {
 
-// One pass of G*R rows, score only.  prof points at the pass's row 0 and
-// holds s(query_i, r) + o (>= 0; padding rows hold 0, i.e. a score of -o).
+// One pass of G*R rows, score only.  profA (and profB, the second int16
+// lane's) points at the pass's row 0 and holds s(query_i, r) + o (>= 0; padding
+// rows hold 0, i.e. a score of -o).
 // The cell update works with E* = E + o and F* = F + o:
 //   P  = Hdiag + (s + o)          one 32-bit add: never carries across the
 //                                 int16 lanes because every lane stays >= 0
@@ -40,7 +41,8 @@ namespace {
 // the matrix, H = 0, F* = 0 (F = -o)).  scr_out: where the last lane stores
 // its bottom row (nullptr for the last pass).  Returns the lane's best H.
 template <int G, int R, bool PACK>
-__device__ __forceinline__ int wave_pass(const int8_t *__restrict__ prof, int stride,
+__device__ __forceinline__ int wave_pass(const int8_t *__restrict__ profA,
+                                         const int8_t *__restrict__ profB, int stride,
                                          const uint8_t *__restrict__ rA, int LA,
                                          const uint8_t *__restrict__ rB, int LB, int Lw, int t,
                                          int base_lane, int padc, int o, int e,
@@ -67,7 +69,7 @@ __device__ __forceinline__ int wave_pass(const int8_t *__restrict__ prof, int st
     if (0 < Lw) sv0 = scr_in[0];
     if (1 < Lw) sv1 = scr_in[1];
   }
-  const int8_t *pb = prof + t * R;
+  const int8_t *pbA = profA + t * R, *pbB = profB + t * R;
   const int steps = Lw + G - 1;
 
 #pragma unroll 4
@@ -89,8 +91,8 @@ __device__ __forceinline__ int wave_pass(const int8_t *__restrict__ prof, int st
     }
     resv = rin;
     ProfRow<R> pa, pq;
-    pa.load(pb + (int)(resv & 0xffu) * stride);
-    if constexpr (PACK) pq.load(pb + (int)(resv >> 8) * stride);
+    pa.load(pbA + (int)(resv & 0xffu) * stride);
+    if constexpr (PACK) pq.load(pbB + (int)(resv >> 8) * stride);
 
     int hdiag = htop_prev;
     htop_prev = hin;
@@ -180,7 +182,7 @@ k_center(SeqSet ss, Scoring sc, CenterJob job) {
       for (int p = 0; p < np; ++p) {
         const int2 *sin = p > 0 ? scr + (size_t)((p - 1) & 1) * job.scratch_cols : nullptr;
         int2 *sout = p + 1 < np ? scr + (size_t)(p & 1) * job.scratch_cols : nullptr;
-        const int b = wave_pass<G, R, PACK>(smem + p * G * R, stride, rA, LA, rB, LB, Lw, t,
+        const int b = wave_pass<G, R, PACK>(smem + p * G * R, smem + p * G * R, stride, rA, LA, rB, LB, Lw, t,
                                             base_lane, padc, sc.o, sc.e, sin, sout);
         best = Cell<PACK>::vmax(best, b);
         __syncwarp();
@@ -588,7 +590,7 @@ __global__ void __launch_bounds__(256) k_pairs(SeqSet ss, Scoring sc, PairJob jo
       if (Lw > 0) {
         const int2 *sin = p > 0 ? scr + (size_t)((p - 1) & 1) * job.scratch_cols : nullptr;
         int2 *sout = p + 1 < np ? scr + (size_t)(p & 1) * job.scratch_cols : nullptr;
-        best = max(best, wave_pass<G, R, false>(prof, SR, rb, Lb, nullptr, 0, Lw, t, base_lane,
+        best = max(best, wave_pass<G, R, false>(prof, prof, SR, rb, Lb, nullptr, 0, Lw, t, base_lane,
                                                 padc, sc.o, sc.e, sin, sout));
       }
       __syncwarp();
@@ -597,6 +599,104 @@ __global__ void __launch_bounds__(256) k_pairs(SeqSet ss, Scoring sc, PairJob jo
     for (int off = G / 2; off > 0; off >>= 1)
       best = max(best, __shfl_xor_sync(MSA_FULL_MASK, best, off));
     if (valid && t == 0) job.out[job.dst[pi]] = best;
+  }
+}
+
+// The pair list in packed cells: each group carries two pairs, neighbours in
+// the list (the host sorts it by passes and columns), in the int16 lanes of
+// every register, each with its own profile (the host lists a pair here only
+// when no score of it can reach the lanes' limit).  The profile of a pass is
+// built four rows by four letters at a time: four words of the biased matrix
+// and eight byte permutations give four profile words.
+// Integer (DPX) bound: a register's two cells cost the pipe 9 slots of DPX and
+// 2 of byte unpacking where the int32 form spends them on one cell, and narrow
+// groups (8 lanes, 128 rows per pass) leave less of a short query's pass empty
+// than 512 rows: 60,000 pairs of 50-2,000 residues took 9.2 ms in int32 cells
+// with 32 lanes, 3.0 ms so (8 warps per SM: the two profiles fill shared memory).
+template <int G>
+__global__ void __launch_bounds__(256, 1) k_pairs2(SeqSet ss, Scoring sc, PairJob job) {
+  constexpr int R = kPairsR, NT = 256, NG = NT / G, SR = G * R, GPW = 32 / G;
+  extern __shared__ __align__(16) int8_t smem[];
+  __shared__ uint32_t sMw[(MSA_MAX_ALPHABET + 1) * (MSA_MAX_ALPHABET / 4)];
+  const int K = sc.K, KW = (K + 3) / 4;  // words of a matrix row
+  // the biased matrix, letter K (padding) all zero
+  for (int i = threadIdx.x; i < (K + 1) * KW; i += NT) {
+    const int a = i / KW, r0 = 4 * (i - a * KW);
+    uint32_t v = 0;
+    for (int u = 0; u < 4; ++u)
+      if (a < K && r0 + u < K) v |= (uint32_t)(uint8_t)(sc.M[a * K + r0 + u] + sc.o) << (8 * u);
+    sMw[i] = v;
+  }
+  __syncthreads();
+  const int g = threadIdx.x / G, t = threadIdx.x % G, lane = threadIdx.x & 31;
+  const int base_lane = lane - t;
+  int8_t *prof[2];
+  prof[0] = smem + (size_t)g * 2 * (K + 1) * SR;
+  prof[1] = prof[0] + (size_t)(K + 1) * SR;
+  int2 *scr = job.scratch + ((size_t)blockIdx.x * NG + g) * 2 * job.scratch_cols;
+  // the padding letter's row scores -o everywhere
+  for (int i = t; i < SR / 4; i += G)
+    for (int l = 0; l < 2; ++l) reinterpret_cast<uint32_t *>(prof[l] + K * SR)[i] = 0u;
+  const int nunit = (job.npairs + 1) / 2;
+  for (;;) {
+    int base = 0;
+    if (lane == 0) base = (int)atomicAdd(job.counter, (unsigned long long)GPW);
+    base = __shfl_sync(MSA_FULL_MASK, base, 0);
+    if (base >= nunit) break;
+    const int pi = 2 * (base + lane / G);
+    int La[2] = {0, 0}, Lb[2] = {0, 0};
+    const uint8_t *ra[2] = {ss.res, ss.res}, *rb[2] = {ss.res, ss.res};
+#pragma unroll
+    for (int l = 0; l < 2; ++l)
+      if (pi + l < job.npairs) {
+        const int2 pr = job.pairs[pi + l];
+        La[l] = ss.len[pr.x];
+        Lb[l] = ss.len[pr.y];
+        ra[l] = ss.res + ss.pstart[pr.x];
+        rb[l] = ss.res + ss.pstart[pr.y];
+      }
+    const int Lw = __reduce_max_sync(MSA_FULL_MASK, max(Lb[0], Lb[1]));
+    const int np = __reduce_max_sync(MSA_FULL_MASK, (max(La[0], La[1]) + SR - 1) / SR);
+    int best = 0;
+    for (int p = 0; p < np; ++p) {
+      __syncwarp();
+#pragma unroll
+      for (int l = 0; l < 2; ++l)
+        for (int i = t; i < SR / 4; i += G) {
+          const int q0 = p * SR + 4 * i;
+          int c[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) c[u] = q0 + u < La[l] ? (int)ra[l][q0 + u] * KW : K * KW;
+          uint32_t *dst = reinterpret_cast<uint32_t *>(prof[l]) + i;
+          for (int rw = 0; rw < KW; ++rw) {
+            // a 4 x 4 byte transpose: rows' words of letters -> letters' words of rows
+            const uint32_t w0 = sMw[c[0] + rw], w1 = sMw[c[1] + rw], w2 = sMw[c[2] + rw], w3 = sMw[c[3] + rw];
+            const uint32_t a0 = __byte_perm(w0, w1, 0x5140), a1 = __byte_perm(w2, w3, 0x5140);
+            const uint32_t b0 = __byte_perm(w0, w1, 0x7362), b1 = __byte_perm(w2, w3, 0x7362);
+            const int r = 4 * rw;
+            dst[r * (SR / 4)] = __byte_perm(a0, a1, 0x5410);
+            if (r + 1 < K) dst[(r + 1) * (SR / 4)] = __byte_perm(a0, a1, 0x7632);
+            if (r + 2 < K) dst[(r + 2) * (SR / 4)] = __byte_perm(b0, b1, 0x5410);
+            if (r + 3 < K) dst[(r + 3) * (SR / 4)] = __byte_perm(b0, b1, 0x7632);
+          }
+        }
+      __syncwarp();
+      if (Lw > 0) {
+        const int2 *sin = p > 0 ? scr + (size_t)((p - 1) & 1) * job.scratch_cols : nullptr;
+        int2 *sout = p + 1 < np ? scr + (size_t)(p & 1) * job.scratch_cols : nullptr;
+        const int b = wave_pass<G, R, true>(prof[0], prof[1], SR, rb[0], Lb[0], rb[1], Lb[1], Lw, t,
+                                            base_lane, K, sc.o, sc.e, sin, sout);
+        best = Cell<true>::vmax(best, b);
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int off = G / 2; off > 0; off >>= 1)
+      best = Cell<true>::vmax(best, __shfl_xor_sync(MSA_FULL_MASK, best, off));
+    if (t == 0) {
+      if (pi < job.npairs) job.out[job.dst[pi]] = Cell<true>::lane0(best);
+      if (pi + 1 < job.npairs) job.out[job.dst[pi + 1]] = Cell<true>::lane1(best);
+    }
   }
 }
 
@@ -940,23 +1040,28 @@ cudaError_t launch_center(int variant, const SeqSet &ss, const Scoring &sc, cons
 }
 
 typedef void (*pairs_fn)(SeqSet, Scoring, PairJob);
-static pairs_fn pairs_kernel(int G) {
+static pairs_fn pairs_kernel(int G, bool packed) {
+  if (packed) return G == 8 ? k_pairs2<8> : G == 16 ? k_pairs2<16> : G == 32 ? k_pairs2<32> : nullptr;
   return G == 8 ? k_pairs<8> : (G == 32 ? k_pairs<32> : nullptr);
 }
 int pairs_rows(int G) { return G * kPairsR; }
-static int pairs_smem(int G, int K) { return (256 / G) * (K + 1) * G * kPairsR; }
+// 256 threads hold 256 * kPairsR query rows whatever the width, twice when packed
+static int pairs_smem(int K, bool packed) { return (packed ? 2 : 1) * 256 * kPairsR * (K + 1); }
 
-int pairs_grid(int G) {
-  pairs_fn fn = pairs_kernel(G);
+// packed cells fit the shared memory for this alphabet
+bool pairs_packed_fits(int K) { return pairs_smem(K, true) <= 216 * 1024; }
+
+int pairs_grid(int G, bool packed, int K) {
+  pairs_fn fn = pairs_kernel(G, packed);
   if (!fn) return 0;
-  return occupancy_grid((const void *)fn, 256, pairs_smem(G, MSA_MAX_ALPHABET));
+  return occupancy_grid((const void *)fn, 256, pairs_smem(packed ? K : MSA_MAX_ALPHABET, packed));
 }
 
-cudaError_t launch_pairs(int G, const SeqSet &ss, const Scoring &sc, const PairJob &job,
+cudaError_t launch_pairs(int G, bool packed, const SeqSet &ss, const Scoring &sc, const PairJob &job,
                          int grid, cudaStream_t st) {
-  pairs_fn fn = pairs_kernel(G);
+  pairs_fn fn = pairs_kernel(G, packed);
   if (!fn) return cudaErrorInvalidValue;
-  const int smem = pairs_smem(G, sc.K);
+  const int smem = pairs_smem(sc.K, packed);
   if (smem > 40 * 1024)  // static shared memory counts too
     cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   fn<<<grid, 256, smem, st>>>(ss, sc, job);
@@ -1136,7 +1241,7 @@ __global__ void __launch_bounds__(256) k_pairs_noalloc(NoallocArgs a) {
       __syncwarp();
       const int2 *sin = p > 0 ? scr + (size_t)((p - 1) & 1) * a.scratch_cols : nullptr;
       int2 *sout = p + 1 < np ? scr + (size_t)(p & 1) * a.scratch_cols : nullptr;
-      best = max(best, wave_pass<G, R, false>(prof, SR, rb, Lb, nullptr, 0, Lb, t, 0, padc, a.o,
+      best = max(best, wave_pass<G, R, false>(prof, prof, SR, rb, Lb, nullptr, 0, Lb, t, 0, padc, a.o,
                                               a.e, sin, sout));
       __syncwarp();
     }

@@ -41,7 +41,7 @@ struct CenterJob {
 // Query pairs one stream of the paired center kernel may stack.
 constexpr int kMaxSeg = 32;
 
-// Arbitrary pair list (int32 cells).
+// Arbitrary pair list.
 struct PairJob {
   const int2 *pairs;              // (a, b) sorted indices; a = rows (query), b = columns
   const int32_t *dst;             // output slot of each listed pair
@@ -82,10 +82,13 @@ cudaError_t launch_center(int variant, const SeqSet &ss, const Scoring &sc, cons
 cudaError_t center_allow_smem(int variant, int smem);
 int center_grid(int variant, int smem);
 
-cudaError_t launch_pairs(int G, const SeqSet &ss, const Scoring &sc, const PairJob &job,
+// packed: two pairs per group in int16 lanes (G 8, 16 or 32; the caller checks
+// that no score can reach their limit), else int32 cells (G 8 or 32)
+cudaError_t launch_pairs(int G, bool packed, const SeqSet &ss, const Scoring &sc, const PairJob &job,
                          int grid, cudaStream_t st);
-int pairs_grid(int G);
+int pairs_grid(int G, bool packed, int K);
 int pairs_rows(int G);
+bool pairs_packed_fits(int K);
 
 // G = threads per subject group (1, 2, 4, 8, 16 or 32; codes_group picks 8-32 from the
 // center length and the subject lengths); 16 center rows per thread.  packed: each group carries two
