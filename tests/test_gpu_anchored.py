@@ -70,3 +70,43 @@ def test_proteins_with_short_segments():
         _check(b, h, prob, 5, 4, letters, offsets)
         with pytest.raises(b.MSAError):
             b.msa_align_anchored(h, 5, 13)          # 13 x 5 bits > 64
+
+
+@pytest.mark.parametrize("k", [4, 8, 10, 16])
+def test_stretch_sizes_and_repeated_segments(k):
+    """Unmatched stretches of every shape the aligners divide (one lane: 8 and
+    16 center residues x 24; the warp: up to 80 a side), several in one
+    sequence, beside centers with repeated segments (many matches per segment
+    and position, chains decided by the tie rules)."""
+    b = binding()
+    alph, M = dna_matrix(2, -3)
+    rng = np.random.default_rng(100 + k)
+    bases = np.frombuffer(b"ACGT", np.uint8)
+    rnd = lambda n: bases[rng.integers(0, 4, n)]  # noqa: E731
+    for repeats in (False, True):
+        center = rnd(63 * k)
+        if repeats:
+            unit = center[:2 * k].copy()
+            for at in (6, 14, 15, 30, 31, 32, 50):
+                center[at * k:at * k + 2 * k] = unit[:center.size - at * k][:2 * k]
+        seqs = [center]
+        for lc, lx in [(1, 1), (1, 7), (1, 24), (1, 25), (2, 3), (2, 16), (2, 24), (2, 30), (3, 20),
+                       (0, 1), (0, 33), (1, 0), (4, 40), (5, 79), (6, 80), (6, 81)]:
+            lc = min(lc, 80 // k) if lc else 0
+            parts = [center[:10 * k]]
+            for at in (10, 24, 40):
+                parts += [rnd(lx), center[(at + lc) * k:(at + 14 if at < 40 else 63) * k if at != 24 else 40 * k]]
+            seqs.append(np.concatenate(parts))
+        for rate in (0.02, 0.1, 0.2):
+            for _ in range(6):
+                s = center.copy()
+                hit = rng.random(s.size) < rate
+                s[hit] = rnd(int(hit.sum()))
+                cut = int(rng.integers(1, s.size - 1))
+                seqs.append(np.concatenate([s[:cut], rnd(int(rng.integers(0, 30))), s[cut + int(rng.integers(0, 30)):]]))
+        seqs.append(np.tile(center[:2 * k], 12))
+        letters, offsets = pack_sequences(seqs)
+        prob = oracle_problem(letters, offsets, alph, M, 5, 2)
+        with make_ctx(alph, M, 5, 2) as h:
+            b.msa_load(h, letters, offsets)
+            _check(b, h, prob, 0, k, letters, offsets)
