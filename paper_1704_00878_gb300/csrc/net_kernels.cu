@@ -13,14 +13,43 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
-__global__ void k_colsum(int cout, const bf16 *__restrict__ dy, float *__restrict__ db, int T,
-                         int chunk) {
-  const int c = threadIdx.x;
-  if (c >= cout) return;
+__device__ __forceinline__ void unpack8(const uint4 &u, float (&v)[8]) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162 *>(&w[i]);
+    v[2 * i] = __low2float(p);
+    v[2 * i + 1] = __high2float(p);
+  }
+}
+
+// Column sums of `chunk` rows per CTA: a thread takes 8 channels (one 16-byte
+// load) of every (256 * 8 / COUT)-th row, four loads in flight, and the CTA's
+// partial sums meet in shared memory.  HBM / L2 bound: 160,000 rows x 128
+// channels (41 MB) 14 us with one 2-byte load per thread and row, 12.7 us so.
+template <int COUT>
+__global__ void __launch_bounds__(256) k_colsum(const bf16 *__restrict__ dy, float *__restrict__ db,
+                                                int T, int chunk) {
+  constexpr int LANES = COUT / 8, ROWS = 256 / LANES;  // threads per row, rows per pass
+  __shared__ float part[ROWS][COUT];
+  const int c = (threadIdx.x % LANES) * 8, rr = threadIdx.x / LANES;
   const int r0 = blockIdx.x * chunk, r1 = min(T, r0 + chunk);
-  float s = 0.f;
-  for (int r = r0; r < r1; ++r) s += __bfloat162float(dy[(size_t)r * cout + c]);
-  if (s != 0.f) atomicAdd(db + c, s);
+  float s[8] = {};
+#pragma unroll 4
+  for (int r = r0 + rr; r < r1; r += ROWS) {
+    float v[8];
+    unpack8(__ldg(reinterpret_cast<const uint4 *>(dy + (size_t)r * COUT + c)), v);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] += v[i];
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) part[rr][c + i] = s[i];
+  __syncthreads();
+  if (threadIdx.x >= COUT) return;
+  float t = 0.f;
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) t += part[r][threadIdx.x];
+  if (t != 0.f) atomicAdd(db + threadIdx.x, t);
 }
 
 __global__ void k_fill_rows(Batch b) {
@@ -54,54 +83,69 @@ __global__ void k_onehot(Batch b, const uint8_t *__restrict__ res, const int64_t
 // sum_t P_t W4_t + len b4 with the window sums P_t = sum_r a3[r + t - 4]
 // (rows outside the sequence are zero).  P_0 covers rows base - 4 ..
 // base + len - 5 and P_{t+1} = P_t - a3[base - 4 + t] + a3[base + len - 4 + t].
-// One 128-thread block per sequence: each warp sums every fourth row of P_0
-// (four channels per lane), warp 0 adds the partial sums and slides the
-// window; the nine sums are written as rows 9 s .. 9 s + 8 of pw (bf16),
-// the input of the output convolution.
-__device__ __forceinline__ void load4(const bf16 *p, float (&v)[4]) {
-  const uint2 u = *reinterpret_cast<const uint2 *>(p);
-  const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162 *>(&u.x);
-  const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162 *>(&u.y);
-  v[0] = __low2float(lo);
-  v[1] = __high2float(lo);
-  v[2] = __low2float(hi);
-  v[3] = __high2float(hi);
+// One 256-thread block per sequence: a warp sums every fourth row of P_0 for
+// half of the channels (two per lane), warps 0 and 4 add the partial sums and
+// slide the window; the nine sums are written as rows 9 s .. 9 s + 8 of pw
+// (bf16), the input of the output convolution.  A warp has 32 rows in flight,
+// added in order: a long sequence is a chain of loads whose latency bounds the
+// launch (440 sequences of up to 2,000 rows from cold L2: 54 us with four rows
+// in flight and four channels per lane, 24 us so).
+__device__ __forceinline__ float2 unpack2(uint32_t u) {
+  const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162 *>(&u);
+  return make_float2(__low2float(p), __high2float(p));
 }
 
-__global__ void k_window_sums(Batch b, const bf16 *__restrict__ a3, bf16 *__restrict__ pw) {
+__global__ void __launch_bounds__(256) k_window_sums(Batch b, const bf16 *__restrict__ a3,
+                                                     bf16 *__restrict__ pw) {
   __shared__ float part[4][WD];
   const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (s >= b.nseq) return;
   const int base = b.base[s], L = b.len[s];
-  const bf16 *row0 = a3 + (size_t)(base - HALF) * WD + 4 * lane;  // row base - 4
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-  for (int i = warp; i < L; i += 4) {
-    float v[4];
-    load4(row0 + (size_t)i * WD, v);
+  const int ch = 64 * (warp >> 2) + 2 * lane;          // this lane's channels
+  const bf16 *row0 = a3 + (size_t)(base - HALF) * WD;  // row base - 4
+  auto at = [&](int i) { return reinterpret_cast<const uint32_t *>(row0 + (size_t)i * WD + ch); };
+  float a0 = 0.f, a1 = 0.f;
+  constexpr int FLY = 32;
+  int i = warp & 3;
+  for (; i + 4 * (FLY - 1) < L; i += 4 * FLY) {
+    uint32_t u[FLY];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[c] += v[c];
+    for (int k = 0; k < FLY; ++k) u[k] = __ldg(at(i + 4 * k));
+#pragma unroll
+    for (int k = 0; k < FLY; ++k) {
+      const float2 v = unpack2(u[k]);
+      a0 += v.x;
+      a1 += v.y;
+    }
   }
+#pragma unroll 8
+  for (; i < L; i += 4) {
+    const float2 v = unpack2(__ldg(at(i)));
+    a0 += v.x;
+    a1 += v.y;
+  }
+  part[warp & 3][ch] = a0;
+  part[warp & 3][ch + 1] = a1;
+  // the rows that enter and leave the window as it slides
+  uint32_t out[TAPS - 1], in[TAPS - 1];
+  if ((warp & 3) == 0) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) part[warp][4 * lane + c] = acc[c];
+    for (int t = 0; t < TAPS - 1; ++t) {
+      out[t] = __ldg(at(t));
+      in[t] = __ldg(at(L + t));
+    }
+  }
   __syncthreads();
-  if (warp != 0) return;
-  float p[4];
+  if ((warp & 3) != 0) return;
+  float p0 = part[0][ch] + part[1][ch] + part[2][ch] + part[3][ch];
+  float p1 = part[0][ch + 1] + part[1][ch + 1] + part[2][ch + 1] + part[3][ch + 1];
 #pragma unroll
-  for (int c = 0; c < 4; ++c)
-    p[c] = part[0][4 * lane + c] + part[1][4 * lane + c] + part[2][4 * lane + c] + part[3][4 * lane + c];
   for (int t = 0; t < TAPS; ++t) {
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(p[0], p[1]), hi = __floats2bfloat162_rn(p[2], p[3]);
-    uint2 u;
-    u.x = *reinterpret_cast<const uint32_t *>(&lo);
-    u.y = *reinterpret_cast<const uint32_t *>(&hi);
-    *reinterpret_cast<uint2 *>(pw + ((size_t)TAPS * s + t) * WD + 4 * lane) = u;
+    *reinterpret_cast<__nv_bfloat162 *>(pw + ((size_t)TAPS * s + t) * WD + ch) = __floats2bfloat162_rn(p0, p1);
     if (t + 1 < TAPS) {
-      float out[4], in[4];
-      load4(row0 + (size_t)t * WD, out);
-      load4(row0 + (size_t)(L + t) * WD, in);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) p[c] += in[c] - out[c];
+      const float2 o = unpack2(out[t]), n = unpack2(in[t]);
+      p0 += n.x - o.x;
+      p1 += n.y - o.y;
     }
   }
 }
@@ -140,14 +184,23 @@ __global__ void k_pair_loss(const int2 *__restrict__ pairs, const float *__restr
   atomicAdd(demb + (size_t)b * DIM + lane + 32, -g * d1);
 }
 
+// Eight channels per thread, one 16-byte store (HBM bound by its 128 bytes per
+// row; 160,000 rows 35 us with a 2-byte store per thread, 7.9 us so).
 __global__ void k_pool_backward(Batch b, const float *__restrict__ demb, bf16 *__restrict__ dy4) {
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)b.T * DIM) return;
-  const int r = (int)(idx / DIM), c = (int)(idx - (size_t)r * DIM);
+  if (idx >= (size_t)b.T * (DIM / 8)) return;
+  const int r = (int)(idx / (DIM / 8)), c = 8 * (int)(idx % (DIM / 8));
   const int s = b.rowseq[r];
-  float v = 0.f;
-  if (s >= 0) v = demb[(size_t)s * DIM + c] * rsqrtf((float)b.len[s]);
-  dy4[idx] = __float2bfloat16(v);
+  uint4 out = make_uint4(0u, 0u, 0u, 0u);
+  if (s >= 0) {
+    const float k = rsqrtf((float)b.len[s]);
+    const float4 lo = *reinterpret_cast<const float4 *>(demb + (size_t)s * DIM + c);
+    const float4 hi = *reinterpret_cast<const float4 *>(demb + (size_t)s * DIM + c + 4);
+    const __nv_bfloat162 p[4] = {__floats2bfloat162_rn(lo.x * k, lo.y * k), __floats2bfloat162_rn(lo.z * k, lo.w * k),
+                                 __floats2bfloat162_rn(hi.x * k, hi.y * k), __floats2bfloat162_rn(hi.z * k, hi.w * k)};
+    out = *reinterpret_cast<const uint4 *>(p);
+  }
+  *reinterpret_cast<uint4 *>(dy4 + (size_t)r * DIM + c) = out;
 }
 
 __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
@@ -245,14 +298,17 @@ cudaError_t onehot(const Batch &b, const uint8_t *res, const int64_t *pstart, bf
 
 cudaError_t colsum(int cout, const bf16 *dy, float *db, int T, cudaStream_t st) {
   if (T <= 0) return cudaSuccess;
-  const int chunk = 128;  // short serial sums, many CTAs
-  k_colsum<<<(T + chunk - 1) / chunk, cout, 0, st>>>(cout, dy, db, T, chunk);
+  const int chunk = 512;  // short serial sums, a few CTAs per SM
+  const int blocks = (T + chunk - 1) / chunk;
+  if (cout == WD) k_colsum<WD><<<blocks, 256, 0, st>>>(dy, db, T, chunk);
+  else if (cout == DIM) k_colsum<DIM><<<blocks, 256, 0, st>>>(dy, db, T, chunk);
+  else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
 cudaError_t window_sums(const Batch &b, const bf16 *a3, bf16 *pw, cudaStream_t st) {
   if (b.nseq <= 0) return cudaSuccess;
-  k_window_sums<<<b.nseq, 128, 0, st>>>(b, a3, pw);
+  k_window_sums<<<b.nseq, 256, 0, st>>>(b, a3, pw);
   return cudaGetLastError();
 }
 
@@ -272,7 +328,7 @@ cudaError_t pair_loss(const int2 *pairs, const float *targets, int npairs, const
 }
 
 cudaError_t pool_backward(const Batch &b, const float *demb, bf16 *dy4, cudaStream_t st) {
-  const size_t total = (size_t)b.T * DIM;
+  const size_t total = (size_t)b.T * (DIM / 8);
   k_pool_backward<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(b, demb, dy4);
   return cudaGetLastError();
 }

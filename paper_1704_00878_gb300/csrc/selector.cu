@@ -28,6 +28,14 @@ struct Selector {
   DevBuf seq, base, len, rowseq, x0, a1, a2, a3, pw, yw, emb, demb, dy4, dz3, dz2, dz1;
   DevBuf bpairs, btargets, loss, small, allemb, dist;
   DevBuf vstart, vlen, vself;  // a reference/candidate view of the loaded set
+  // host side of a batch: the copies to the device read these until `staged`
+  std::vector<int32_t> h_seq, h_base, h_len;
+  std::vector<int2> h_pairs;
+  std::vector<float> h_targets;
+  cudaEvent_t staged = nullptr;
+  // batch-local number of a sequence: h_slot[k] where h_stamp[k] == stamp
+  std::vector<int32_t> h_slot, h_stamp;
+  int32_t stamp = 0;
 };
 
 namespace {
@@ -111,7 +119,9 @@ int set_params(msa_ctx *ctx, Selector *s, const float *host) {
 // its one-hot input.
 int build_batch(msa_ctx *ctx, Selector *s, const std::vector<int32_t> &seqs, net::Batch &b) {
   const int ns = (int)seqs.size();
-  std::vector<int32_t> base(ns), len(ns);
+  std::vector<int32_t> &base = s->h_base, &len = s->h_len;
+  base.resize(ns);
+  len.resize(ns);
   int64_t row = net::HALF;
   for (int i = 0; i < ns; ++i) {
     base[i] = (int32_t)row;
@@ -142,9 +152,15 @@ int build_batch(msa_ctx *ctx, Selector *s, const std::vector<int32_t> &seqs, net
   b.rowseq = P<int32_t>(s->rowseq);
   CK((++ctx->launches, net::fill_rows)(b, ctx->st));
   CK((++ctx->launches, net::onehot)(b, P<uint8_t>(ctx->res), P<int64_t>(ctx->d_pstart), P<bf16>(s->x0), ctx->st));
-  // the stream orders the small host arrays' copies before their use; keep
-  // them alive until then
-  CK(cudaStreamSynchronize(ctx->st));
+  // (no wait: the host arrays stay as they are until `staged`)
+  CK(cudaEventRecord(s->staged, ctx->st));
+  return MSA_OK;
+}
+
+// Before a batch's host arrays are written again: their last copies are done.
+int reuse_staging(msa_ctx *ctx, Selector *s) {
+  if (!s->staged) CK(cudaEventCreateWithFlags(&s->staged, cudaEventDisableTiming));
+  CK(cudaEventSynchronize(s->staged));
   return MSA_OK;
 }
 
@@ -212,29 +228,38 @@ int forward_backward(msa_ctx *ctx, Selector *s, const net::Batch &b, int npairs)
 // Batch of pairs (input indices) -> unique batch sequences and local pairs.
 int stage_pairs(msa_ctx *ctx, Selector *s, const int64_t *pairs, const float *targets, int64_t np,
                 net::Batch &b) {
-  std::unordered_map<int32_t, int32_t> local;
-  std::vector<int32_t> seqs;
-  std::vector<int2> lp(np);
+  TRY(reuse_staging(ctx, s));
+  if ((int)s->h_stamp.size() != ctx->n || s->stamp == INT32_MAX) {
+    s->h_stamp.assign(ctx->n, 0);
+    s->h_slot.resize(ctx->n);
+    s->stamp = 0;
+  }
+  const int32_t stamp = ++s->stamp;
+  std::vector<int32_t> &seqs = s->h_seq;
+  std::vector<int2> &lp = s->h_pairs;
+  seqs.clear();
+  lp.resize(np);
   for (int64_t x = 0; x < np; ++x) {
     int32_t ids[2];
     for (int h = 0; h < 2; ++h) {
       const int64_t t = pairs[2 * x + h];
       if (t < 0 || t >= ctx->n) return fail(ctx, MSA_EINVAL, "pair index out of range");
       const int32_t k = ctx->inv[t];
-      auto it = local.find(k);
-      if (it == local.end()) {
-        it = local.emplace(k, (int32_t)seqs.size()).first;
+      if (s->h_stamp[k] != stamp) {
+        s->h_stamp[k] = stamp;
+        s->h_slot[k] = (int32_t)seqs.size();
         seqs.push_back(k);
       }
-      ids[h] = it->second;
+      ids[h] = s->h_slot[k];
     }
     lp[x] = make_int2(ids[0], ids[1]);
   }
+  s->h_targets.assign(targets, targets + np);
   TRY(ensure(ctx, s->bpairs, sizeof(int2) * np));
   TRY(ensure(ctx, s->btargets, sizeof(float) * np));
   CK(cudaMemcpyAsync(s->bpairs.p, lp.data(), sizeof(int2) * np, cudaMemcpyHostToDevice, ctx->st));
-  CK(cudaMemcpyAsync(s->btargets.p, targets, sizeof(float) * np, cudaMemcpyHostToDevice, ctx->st));
-  return build_batch(ctx, s, seqs, b);  // synchronises before the host vectors go away
+  CK(cudaMemcpyAsync(s->btargets.p, s->h_targets.data(), sizeof(float) * np, cudaMemcpyHostToDevice, ctx->st));
+  return build_batch(ctx, s, seqs, b);
 }
 
 // The exact center's distance of a pair in units of 2^-16 (the kernels' sums
@@ -287,7 +312,9 @@ int embed_all(msa_ctx *ctx, Selector *s) {
   const int64_t max_rows = (int64_t)1 << 23;  // ~1.1 KB of activations per row
   int k = 0;
   while (k < n) {
-    std::vector<int32_t> seqs;
+    TRY(reuse_staging(ctx, s));
+    std::vector<int32_t> &seqs = s->h_seq;
+    seqs.clear();
     int64_t rows = net::HALF;
     while (k < n && (seqs.empty() || rows + ctx->len_sorted[k] + net::HALF <= max_rows)) {
       rows += ctx->len_sorted[k] + net::HALF;
@@ -312,6 +339,10 @@ void selector_free(msa_ctx *ctx, Selector *s) {
                     &s->dz2, &s->dz1, &s->bpairs, &s->btargets, &s->loss, &s->small, &s->allemb,
                     &s->dist, &s->vstart, &s->vlen, &s->vself};
   for (DevBuf *b : bufs) release(ctx, *b);
+  if (s->staged) {
+    cudaEventSynchronize(s->staged);  // the copies that read the host arrays
+    cudaEventDestroy(s->staged);
+  }
   delete s;
 }
 

@@ -603,11 +603,21 @@ k_conv_tc2(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
     const int q = warp & 3, hh = (warp - 2) >> 2;
     for (int it = 0, tile = first; tile < ntiles; tile += stride, ++it) {
       const int b = it & 1, k = it >> 1;
-      if (!mbar_wait_cl(bar(B_CFULL + b), (uint32_t)(k & 1), spins)) { ok = false; break; }
-      tc_fence_after();
       const int r = tile * PAIR_TBM + (int)rank * TBM + q * 32 + lane;
       const bool inb = r < T;
+      const int cb = hh * HC;  // first channel of this warp
+      // what the epilogue reads from memory, in flight while the tile's MMAs run
+      // (data gradients of 160,000 rows, 128 -> 128 channels 49 -> 40 us and
+      // 64 -> 128 channels 38 -> 29 us against loads after the wait)
       const bool valid = inb && (rowseq == nullptr || rowseq[r] >= 0);
+      [[maybe_unused]] uint4 mask[MODE == 2 ? NCH : 1];
+      if constexpr (MODE == 2) {
+        const uint4 *pv = reinterpret_cast<const uint4 *>(prev + (size_t)r * COUT + cb);
+#pragma unroll
+        for (int jc = 0; jc < NCH; ++jc) mask[jc] = inb ? __ldg(pv + jc) : make_uint4(0u, 0u, 0u, 0u);
+      }
+      if (!mbar_wait_cl(bar(B_CFULL + b), (uint32_t)(k & 1), spins)) { ok = false; break; }
+      tc_fence_after();
       // this warp's slice into registers (one load, one wait), then the
       // accumulator goes back to the issuer before any store
       float v[HC];
@@ -618,9 +628,7 @@ k_conv_tc2(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster_relaxed(peer_addr(bar(B_CEMPTY + b), 0));
       if (!inb) continue;
-      const int cb = hh * HC;  // first channel of this warp
       uint4 *dst = reinterpret_cast<uint4 *>(static_cast<unsigned char *>(y) + ((size_t)r * COUT + cb) * OUTB);
-      const uint4 *pv = MODE == 2 ? reinterpret_cast<const uint4 *>(prev + (size_t)r * COUT + cb) : nullptr;
 #pragma unroll
       for (int jc = 0; jc < NCH; ++jc) {
         if constexpr (MODE == 1) {
@@ -634,7 +642,7 @@ k_conv_tc2(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
         } else {
           const int e = 8 * jc;
           uint4 pm = make_uint4(0u, 0u, 0u, 0u);
-          if constexpr (MODE == 2) pm = pv[jc];
+          if constexpr (MODE == 2) pm = mask[jc];
           [[maybe_unused]] const uint32_t pw[4] = {pm.x, pm.y, pm.z, pm.w};
           uint32_t w[4];
 #pragma unroll

@@ -247,3 +247,35 @@ def test_refined_over_references_is_the_sampled_row_sum(k):
     assert c in set(order[:k + 2].tolist())
     for q in order[:k - 2]:
         assert orow[q] > orow[c] or (orow[q] == orow[c] and q >= c)
+
+
+@pytest.mark.parametrize("lengths", [
+    tuple(range(1, 13)) + (31, 33),                  # shorter than the nine taps, one loop tail
+    (124, 125, 127, 128, 129, 131, 253, 256, 260),   # 32 rows in flight per warp: 128 a round
+    (508, 1, 500, 4, 511, 513, 1024),                # rows around the 512 of a column sum
+])
+def test_odd_lengths_embeddings_and_gradients(lengths):
+    """Window sums, column sums and the pooling's gradient at the edges of
+    their loops, with the bounds of the whole-tensor comparison above."""
+    b = binding()
+    from seqgen import blosum62, pack_sequences
+    rng = np.random.default_rng(sum(lengths))
+    alph, M = blosum62()
+    pool = np.frombuffer(b"ARNDCQEGHILKMFPSTWYV", dtype=np.uint8)
+    letters, offsets = pack_sequences([rng.choice(pool, size=L) for L in lengths])
+    prob = oracle_problem(letters, offsets, alph, M, 11, 1)
+    seqs = [prob.seq(i) for i in range(prob.n)]
+    pairs = np.array([(i, (i + prob.n // 2) % prob.n) for i in range(prob.n)])
+    targets = rng.uniform(0.2, 0.9, size=len(pairs)).astype(np.float32)
+    with make_ctx(alph, M, 11, 1) as h:
+        b.msa_load(h, letters, offsets)
+        b.msa_selector_init(h, seed=17)
+        params = net.unflatten(b.msa_selector_params(h).astype(np.float64))
+        emb = b.msa_selector_embed(h)
+        # twice: the second batch reuses the first one's staging
+        loss, grad = b.msa_selector_grad(h, pairs[:3], targets[:3])
+        loss, grad = b.msa_selector_grad(h, pairs, targets)
+    check_embeddings(emb, net.embed_all(params, seqs))
+    oloss, og = net.loss_and_grad(params, seqs, pairs, targets.astype(np.float64))
+    assert abs(loss - oloss) <= LOSS_TOL * abs(oloss)
+    assert rel_err(grad, net.flatten(og)) < GRAD_TOL
