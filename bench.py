@@ -61,7 +61,8 @@ TREE_PEAK_TCPS = 152 * 128 * 2.07e9 / (9 / 4) / 1e12
 # (two queries per int16x2 register?, lanes per group, query rows per lane, packed)
 CENTER_VARIANTS = [(1, 8, 12, 1), (1, 8, 20, 1), (1, 8, 28, 1), (1, 16, 12, 1), (1, 16, 20, 1),
                    (1, 16, 28, 1), (1, 32, 12, 1), (1, 32, 20, 1), (1, 32, 28, 1), (0, 32, 16, 1),
-                   (0, 32, 24, 1), (0, 8, 16, 0), (0, 16, 16, 0), (0, 32, 16, 0)]
+                   (0, 32, 24, 1), (0, 8, 16, 0), (0, 16, 16, 0), (0, 32, 16, 0), (1, 16, 16, 1),
+                   (1, 16, 24, 1)]
 BUCKET_EDGES = [1, 48, 80, 112, 144, 176, 208, 256, 320, 384, 448, 512, 640, 768, 896, 1024, 1280,
                 1536, 2048, 3072, 4096, 8193]
 

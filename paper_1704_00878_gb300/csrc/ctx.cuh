@@ -22,6 +22,7 @@ enum Stage {
 
 struct Selector;  // the learned center selector (selector.cu)
 constexpr int kMaxTreeRows = 65536;  // rows of a neighbour-joining tree
+constexpr int kCenterLanes = 8;      // branches of the center graph
 void selector_free(msa_ctx *ctx, Selector *s);
 
 }  // namespace msa_detail
@@ -61,8 +62,7 @@ struct msa_ctx {
   // center selection
   DevBuf pairsum, self, rowsum, prefix, qlist, ovf, ovf_scores, ovf_dst, part_val, part_idx,
       pairs, pair_dst, pair_out, counters, streams;
-  cudaStream_t cap_st = nullptr;  // private streams the center graph is captured on
-  cudaStream_t cap_st2 = nullptr;
+  cudaStream_t cap_lanes[msa_detail::kCenterLanes] = {};  // private streams the center graph is captured on
   cudaEvent_t cap_fork = nullptr, cap_join = nullptr;
   cudaGraphExec_t center_exec = nullptr;  // the last center graph and what it bakes in
   std::vector<int64_t> center_key;

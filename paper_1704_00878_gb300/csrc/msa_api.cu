@@ -178,7 +178,7 @@ int run_pairs(msa_ctx *ctx, const std::vector<int2> &pairs_in, const std::vector
   TRY(ensure(ctx, ctx->scratch, sizeof(int2) * rows_off[kClasses]));
   TRY(ensure(ctx, ctx->counters, sizeof(unsigned long long) * kClasses));
   CK(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long) * kClasses, ctx->st));
-  const cudaStream_t lanes[3] = {ctx->st, ctx->cap_st, ctx->cap_st2};
+  const cudaStream_t lanes[3] = {ctx->st, ctx->cap_lanes[0], ctx->cap_lanes[1]};
   if (used > 1) {
     CK(cudaEventRecord(ctx->cap_fork, ctx->st));
     for (int k = 1; k < std::min(used, 3); ++k) CK(cudaStreamWaitEvent(lanes[k], ctx->cap_fork, 0));
@@ -453,7 +453,9 @@ ClassPlan plan_class(msa_ctx *ctx, int mode, int nq_list, const CenterClass &cc,
   const int rows = cv.G * cv.R;
   pl.npass = (maxrows + rows - 1) / rows;
   pl.smem = center_smem_bytes(cc.variant, ctx->K, pl.npass * rows);
-  pl.grid = center_grid(cc.variant, pl.smem);
+  // no more CTAs than items: those that would find the list empty only delay
+  // the CTAs of the classes beside this one
+  pl.grid = (int)std::min<int64_t>(center_grid(cc.variant, pl.smem), std::max<int64_t>(pl.n_items, 1));
   return pl;
 }
 
@@ -485,7 +487,7 @@ CenterJob class_job(msa_ctx *ctx, int mode, const ClassPlan &pl, int sub_off, in
 }
 
 // Upload the plans' prefixes and size the scratch rows of multi-pass
-// classes (all classes run in stream order, so they share one scratch).
+// classes (those of a lane run in stream order, so they share one scratch).
 int stage_plans(msa_ctx *ctx, const std::vector<ClassPlan> &plans,
                 const std::vector<int64_t> &prefix_all, const std::vector<int2> &streams) {
   TRY(ensure(ctx, ctx->streams, sizeof(int2) * std::max<size_t>(streams.size(), 1)));
@@ -497,7 +499,7 @@ int stage_plans(msa_ctx *ctx, const std::vector<ClassPlan> &plans,
     if (pl.npass > 1)
       scratch = std::max(scratch, (size_t)pl.grid * (kCenterThreads / kCenterVariants[pl.cc.variant].G) *
                                       2 * ctx->maxlen * sizeof(int2));
-  // the graph runs its classes on two streams: one boundary-row area each
+  // the graph runs its multi-pass classes in two lanes: one boundary-row area each
   if (scratch) TRY(ensure(ctx, ctx->scratch, 2 * scratch));
   ctx->scratch_half = scratch / sizeof(int2);
   TRY(ensure(ctx, ctx->prefix, sizeof(int64_t) * prefix_all.size()));
@@ -547,18 +549,23 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
   unsigned long long *cnt = P<unsigned long long>(ctx->counters);
   // Everything the graph bakes in; a selection with the same key (the same
   // set and buffers, e.g. a repeated step) relaunches the cached graph.
-  // The classes run longest queries first, alternating between two streams
-  // (a fork and a join in the graph), so a class's tail of long items
-  // overlaps the next class instead of idling the GPU; each stream has its
-  // own boundary-row area.
+  // The classes run longest queries first, dealt out to the lanes of a fork
+  // and a join in the graph, so the CTAs that a class's last, long items leave
+  // free go to the classes after it.  Multi-pass classes take the first two
+  // lanes only, which have a boundary-row area each.  A set of a few hundred
+  // sequences is all tails: the all-pairs selection of 100 (200) proteins took
+  // 463 (505) us in two lanes and 234 (402) in eight.
   std::vector<CenterJob> jobs;
+  auto lane_of = [&](size_t c) {
+    const size_t order = plans.size() - 1 - c;  // launch position
+    return (int)(order % (plans[c].npass > 1 ? 2 : kCenterLanes));
+  };
   std::vector<int64_t> key = {mode, sub_off, sub_n, (int64_t)ss.res, (int64_t)ss.pstart,
                               (int64_t)ss.len, ss.n, (int64_t)sc.M, sc.K, sc.o, sc.e,
                               (int64_t)cnt, (int64_t)plans.size()};
   for (size_t c = 0; c < plans.size(); ++c) {
     CenterJob job = class_job(ctx, mode, plans[c], sub_off, sub_n, cnt + c, self);
-    const size_t order = plans.size() - 1 - c;  // launch position
-    if (order & 1) job.scratch += ctx->scratch_half;
+    if (lane_of(c) == 1) job.scratch += ctx->scratch_half;
     jobs.push_back(job);
     const int64_t f[] = {plans[c].cc.variant, plans[c].grid, plans[c].smem, job.mode,
                          (int64_t)job.qlist, job.nq, job.qb, job.qe, job.sub_off, job.sub_n,
@@ -575,24 +582,26 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
       ctx->center_exec = nullptr;
       ctx->center_key.clear();
     }
-    CK(cudaStreamBeginCapture(ctx->cap_st, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * plans.size(), ctx->cap_st);
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->cap_fork, ctx->cap_st);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->cap_st2, ctx->cap_fork, 0);
+    CK(cudaStreamBeginCapture(ctx->cap_lanes[0], cudaStreamCaptureModeThreadLocal));
+    cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * plans.size(), ctx->cap_lanes[0]);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->cap_fork, ctx->cap_lanes[0]);
+    const int lanes = (int)std::min<size_t>(plans.size(), kCenterLanes);
+    for (int k = 1; k < lanes && e == cudaSuccess; ++k)
+      e = cudaStreamWaitEvent(ctx->cap_lanes[k], ctx->cap_fork, 0);
     int failed = -1;
     for (size_t k = 0; k < plans.size() && e == cudaSuccess; ++k) {
       const size_t c = plans.size() - 1 - k;
       e = launch_center(plans[c].cc.variant, ss, sc, jobs[c], plans[c].grid,
-                        (k & 1) ? ctx->cap_st2 : ctx->cap_st, false);
+                        ctx->cap_lanes[lane_of(c)], false);
       if (e != cudaSuccess) failed = (int)c;
     }
-    {
-      const cudaError_t e2 = cudaEventRecord(ctx->cap_join, ctx->cap_st2);
-      const cudaError_t e3 = cudaStreamWaitEvent(ctx->cap_st, ctx->cap_join, 0);
+    for (int k = 1; k < lanes; ++k) {
+      const cudaError_t e2 = cudaEventRecord(ctx->cap_join, ctx->cap_lanes[k]);
+      const cudaError_t e3 = cudaStreamWaitEvent(ctx->cap_lanes[0], ctx->cap_join, 0);
       if (e == cudaSuccess) e = e2 != cudaSuccess ? e2 : e3;
     }
     cudaGraph_t graph = nullptr;
-    const cudaError_t e_end = cudaStreamEndCapture(ctx->cap_st, &graph);
+    const cudaError_t e_end = cudaStreamEndCapture(ctx->cap_lanes[0], &graph);
     if (failed >= 0) {
       if (graph) cudaGraphDestroy(graph);
       const ClassPlan &pl = plans[failed];
@@ -676,9 +685,21 @@ int run_center(msa_ctx *ctx, int mode, const std::vector<int32_t> &qsorted, cons
   // within one pass (a stack over several passes pays boundary rows the
   // model does not see).
   int64_t items_single = 0;
-  for (int p = p_begin; p < p_end; ++p) items_single += (int64_t)(mode == 0 ? n - 2 * p : n) / 8;
+  double groups = 0;  // alignments of a query pair with a subject
+  for (int p = p_begin; p < p_end; ++p) {
+    items_single += (int64_t)(mode == 0 ? n - 2 * p : n) / 8;
+    groups += partners(2 * p);
+  }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->dev);
+  // A set too small to give every scheduler eight warps in all runs at the rate
+  // of its dependent steps, not of their instructions: a shape's cost per cell
+  // grows as its warps get fewer, which turns short lists to wider groups of
+  // lanes.  100 DNA sequences of 3,000 against 100 references: 7.95 ms without
+  // the rule, 3.75 with it (5.4 with a line at two warps, 3.77 at four); 200
+  // such: 10.9, 4.77, 11.0, 5.5; 200 proteins of 350: 8.8, 6.0 (8.8 at four, 4.2
+  // at twelve, which loses on 400 DNA); from 500 proteins on both are within 2 %.
+  auto fill = [&](int G) { return std::min(1.0, groups * G / 32 / (8.0 * 4 * std::max(sms, 1))); };
   const bool stack = mode != 2 && items_single >= 16 * 2 * 3 * (int64_t)std::max(sms, 1);
   for (int p = p_begin; p < p_end;) {
     int bv = -1, bm = 0;
@@ -704,7 +725,7 @@ int run_center(msa_ctx *ctx, int mode, const std::vector<int32_t> &qsorted, cons
         real += (double)qlen[xa] * partner_cells(xa) + (xb < x1 ? (double)qlen[xb] * partner_cells(xb) : 0.0);
         const int np = (rows + GR - 1) / GR;
         const double cost = (double)np * GR * (1.0 + 3.0 / cv.R) *
-                            (partner_cells(2 * p) + partners(2 * p) * (cv.G - 1 + (np > 1 ? 48 : 0))) / corr;
+                            (partner_cells(2 * p) + partners(2 * p) * (cv.G - 1 + (np > 1 ? 48 : 0))) / (corr * fill(cv.G));
         if (cost / real < bcost) { bcost = cost / real; bv = v; bm = q - p + 1; }
       }
     }
@@ -1215,8 +1236,7 @@ int msa_create(msa_ctx **out, const msa_params *p, void *cuda_stream) {
     CK(cudaMalloc(&ctx->dSymLut, 256));
     CK(cudaMemcpy(ctx->dSymLut, sym, 256, cudaMemcpyHostToDevice));
     CK(cudaMalloc(&ctx->dcounter, sizeof(unsigned long long)));
-    CK(cudaStreamCreateWithFlags(&ctx->cap_st, cudaStreamNonBlocking));
-    CK(cudaStreamCreateWithFlags(&ctx->cap_st2, cudaStreamNonBlocking));
+    for (cudaStream_t &lane : ctx->cap_lanes) CK(cudaStreamCreateWithFlags(&lane, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&ctx->cap_fork, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ctx->cap_join, cudaEventDisableTiming));
     CK(cudaMalloc(&ctx->derr, 2 * sizeof(unsigned)));
@@ -1258,8 +1278,8 @@ void msa_destroy(msa_ctx *ctx) {
   if (ctx->center_exec) cudaGraphExecDestroy(ctx->center_exec);
   if (ctx->align_exec) cudaGraphExecDestroy(ctx->align_exec);
   for (cudaEvent_t ev : ctx->align_ev) cudaEventDestroy(ev);
-  if (ctx->cap_st) cudaStreamDestroy(ctx->cap_st);
-  if (ctx->cap_st2) cudaStreamDestroy(ctx->cap_st2);
+  for (cudaStream_t lane : ctx->cap_lanes)
+    if (lane) cudaStreamDestroy(lane);
   if (ctx->cap_fork) cudaEventDestroy(ctx->cap_fork);
   if (ctx->cap_join) cudaEventDestroy(ctx->cap_join);
   cudaFree(ctx->derr);
@@ -1662,7 +1682,7 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
       ctx->align_exec = nullptr;
       ctx->align_key.clear();
     }
-    CK(cudaStreamBeginCapture(ctx->cap_st, cudaStreamCaptureModeThreadLocal));
+    CK(cudaStreamBeginCapture(ctx->cap_lanes[0], cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     for (int bi = 0; bi < nb && e == cudaSuccess; ++bi) {
       const int sb = batches[bi].first, se = batches[bi].second;
@@ -1677,21 +1697,21 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
       job.counter = ctx->dcounter;
       job.scratch = P<int2>(ctx->scratch);
       job.scratch_cols = ctx->maxlen;
-      e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi], ctx->cap_st, cudaEventRecordExternal);
-      if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dcounter, 0, sizeof(unsigned long long), ctx->cap_st);
+      e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi], ctx->cap_lanes[0], cudaEventRecordExternal);
+      if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dcounter, 0, sizeof(unsigned long long), ctx->cap_lanes[0]);
       // offsets inside the batch are relative to the batch start
-      if (e == cudaSuccess) e = launch_codes(G, packed, ss, sc, job, grid, ctx->cap_st, false, cta);
-      if (e == cudaSuccess) e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi + 1], ctx->cap_st, cudaEventRecordExternal);
+      if (e == cudaSuccess) e = launch_codes(G, packed, ss, sc, job, grid, ctx->cap_lanes[0], false, cta);
+      if (e == cudaSuccess) e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi + 1], ctx->cap_lanes[0], cudaEventRecordExternal);
       if (e == cudaSuccess)
         e = launch_traceback(P<uint8_t>(ctx->codes), P<int64_t>(ctx->code_off) + sb,
                              P<unsigned long long>(ctx->best) + sb, sb, se, P<int32_t>(ctx->d_len),
                              P<int32_t>(ctx->d_perm), ss.res, ss.pstart, kc, sc.M, sc.K, sc.o, sc.e,
                              Lc, G, P<uint16_t>(ctx->ins), P<uint8_t>(ctx->occ), P<int32_t>(ctx->seg),
-                             P<int32_t>(ctx->score), ctx->derr, ctx->cap_st);
-      if (e == cudaSuccess) e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi + 2], ctx->cap_st, cudaEventRecordExternal);
+                             P<int32_t>(ctx->score), ctx->derr, ctx->cap_lanes[0]);
+      if (e == cudaSuccess) e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi + 2], ctx->cap_lanes[0], cudaEventRecordExternal);
     }
     cudaGraph_t graph = nullptr;
-    const cudaError_t e_end = cudaStreamEndCapture(ctx->cap_st, &graph);
+    const cudaError_t e_end = cudaStreamEndCapture(ctx->cap_lanes[0], &graph);
     if (e == cudaSuccess) e = e_end;
     cudaGraphExec_t exec = nullptr;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);

@@ -227,10 +227,13 @@ k_center(SeqSet ss, Scoring sc, CenterJob job) {
 // subject, so the profile can be stored pre-packed: prof[r*stride + i] =
 // (s(qA_i, r) + o) | (s(qB_i, r) + o) << 16, and P = Hdiag + prof is a single
 // add with no unpacking.  Lane t reads R words (R/4 16-byte loads) at word
-// offset t*R; with R/4 odd the eight lanes of a load phase hit eight
-// different 16-byte bank groups whatever residues they read.
+// offset t*pitch, pitch = R or R + 4 so that pitch/4 is odd: the eight lanes of
+// a load phase hit eight different 16-byte bank groups whatever residues they
+// read.
 // IN / OUT: the pass reads the row above from scr_in / writes its bottom row
 // to scr_out (compile-time, so a single-pass query carries no test for them).
+__host__ __device__ constexpr int center_pitch(int R) { return (R / 4) % 2 ? R : R + 4; }
+
 template <int G, int R, bool IN, bool OUT>
 __device__ __forceinline__ int wave_pass_pp(const uint32_t *__restrict__ prof, int stride,
                                             const uint8_t *__restrict__ rs, int Ls, int Lw, int t,
@@ -238,7 +241,7 @@ __device__ __forceinline__ int wave_pass_pp(const uint32_t *__restrict__ prof, i
                                             const int2 *__restrict__ scr_in,
                                             int2 *__restrict__ scr_out) {
   using C = Cell<true>;
-  static_assert(R % 4 == 0 && (R / 4) % 2 == 1, "R/4 must be odd");
+  static_assert(R % 4 == 0, "16-byte profile loads");
   const int negO = C::splat(-o), negE = C::splat(-e);
   const uint32_t pc = (uint32_t)padc;
   int H[R], E[R];
@@ -252,7 +255,7 @@ __device__ __forceinline__ int wave_pass_pp(const uint32_t *__restrict__ prof, i
     if (0 < Lw) sv0 = scr_in[0];
     if (1 < Lw) sv1 = scr_in[1];
   }
-  const uint32_t *pb = prof + t * R;
+  const uint32_t *pb = prof + t * center_pitch(R);
   const int steps = Lw + G - 1;
 #pragma unroll 4
   for (int k = 0; k < steps; ++k) {
@@ -325,7 +328,10 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
   __shared__ unsigned long long s_qsum[kMaxSeg][2];
   constexpr int NT = kCenterThreads, NG = NT / G;
   const int K = sc.K, padc = K, o = sc.o;
-  const int stride = dround_up(job.npass * G * R, 32);
+  constexpr int PITCH = center_pitch(R);
+  const int stride = dround_up(job.npass * G * PITCH, 32);  // of a letter's row
+  // word of query row i (rows of a lane are consecutive, lanes PITCH apart)
+  auto word_of_row = [](int i) { return PITCH == R ? i : i + (i / R) * (PITCH - R); };
   // after the profile: the segment of every R-row block, then the best score
   // of every segment per group (two int16 lanes kept as two ints)
   int *s_blk = reinterpret_cast<int *>(smem32 + (K + 1) * stride);
@@ -367,7 +373,7 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
           if (i < LqA) a = (uint32_t)(sM[ra[i] * K + r] + o);
           if (i < LqB) b = (uint32_t)(sM[rb[i] * K + r] + o);
         }
-        smem32[r * stride + i] = a | (b << 16);
+        smem32[r * stride + word_of_row(i)] = a | (b << 16);
       }
       __syncthreads();
       const int s0 = (job.mode == 0 ? xa : job.sub_off) + (int)(item - job.prefix[lo]) * NG;
@@ -382,7 +388,7 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
         for (int p = 0; p < np; ++p) {
           const int2 *sin = p > 0 ? scr + (size_t)((p - 1) & 1) * job.scratch_cols : nullptr;
           int2 *sout = p + 1 < np ? scr + (size_t)(p & 1) * job.scratch_cols : nullptr;
-          const uint32_t *pp = smem32 + p * G * R;
+          const uint32_t *pp = smem32 + p * G * PITCH;
           int b;
           if (np == 1)
             b = wave_pass_pp<G, R, false, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, sout);
@@ -474,7 +480,7 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
         if (li < s_len[k][0]) a = (uint32_t)(sM[s_res[k][0][li] * K + r] + o);
         if (li < s_len[k][1]) b = (uint32_t)(sM[s_res[k][1][li] * K + r] + o);
       }
-      smem32[r * stride + i] = a | (b << 16);
+      smem32[r * stride + word_of_row(i)] = a | (b << 16);
     }
     __syncthreads();
 
@@ -490,7 +496,7 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
       for (int p = 0; p < np; ++p) {
         const int2 *sin = p > 0 ? scr + (size_t)((p - 1) & 1) * job.scratch_cols : nullptr;
         int2 *sout = p + 1 < np ? scr + (size_t)(p & 1) * job.scratch_cols : nullptr;
-        const uint32_t *pp = smem32 + p * G * R;
+        const uint32_t *pp = smem32 + p * G * PITCH;
         const int blk = p * G + t, kseg = s_blk[blk];
         const bool top = kseg >= 0 && blk * R == s_start[kseg];
         int b;
@@ -949,17 +955,19 @@ __global__ void __launch_bounds__(NT, 1) k_codes2(SeqSet ss, Scoring sc, CodesJo
 // Kernel variants of center selection.  Paired-query variants (k_center2)
 // carry two queries in the int16 lanes; single-query variants (k_center) carry
 // two subjects (packed) or one (int32).  Every shape keeps the profile loads
-// free of shared-memory bank conflicts.
+// free of shared-memory bank conflicts.  The 16- and 24-row shapes close the
+// gaps between 224 and 320 and between 320 and 448 rows: the all-pairs center
+// of 10,000 proteins (median 350) took 1,390 ms without them, 1,351 with.
 const CenterVariant kCenterVariants[] = {
     {1, 8, 12, true},  {1, 8, 20, true},  {1, 8, 28, true},  {1, 16, 12, true},
     {1, 16, 20, true}, {1, 16, 28, true}, {1, 32, 12, true}, {1, 32, 20, true},
     {1, 32, 28, true}, {0, 32, 16, true}, {0, 32, 24, true}, {0, 8, 16, false},
-    {0, 16, 16, false}, {0, 32, 16, false}};
+    {0, 16, 16, false}, {0, 32, 16, false}, {1, 16, 16, true}, {1, 16, 24, true}};
 const int kNumCenterVariants = sizeof(kCenterVariants) / sizeof(kCenterVariants[0]);
 
 int center_profile_bytes(int variant, int K, int rows_alloc) {
   const CenterVariant &v = kCenterVariants[variant];
-  if (v.paired) return (K + 1) * round_up_int(rows_alloc, 32) * 4;
+  if (v.paired) return (K + 1) * round_up_int(rows_alloc / v.R * center_pitch(v.R), 32) * 4;
   return (K + 1) * round_up_int(rows_alloc, MSA_PROF_ALIGN);
 }
 
@@ -969,7 +977,7 @@ int center_smem_bytes(int variant, int K, int rows_alloc) {
   const CenterVariant &v = kCenterVariants[variant];
   int b = center_profile_bytes(variant, K, rows_alloc);
   if (v.paired)
-    b += round_up_int(round_up_int(rows_alloc, 32) / v.R + 1, 4) * 4 +
+    b += round_up_int(round_up_int(rows_alloc / v.R * center_pitch(v.R), 32) / v.R + 1, 4) * 4 +
          (kCenterThreads / v.G) * kMaxSeg * 8;
   return b;
 }
@@ -992,6 +1000,8 @@ static center_fn center_kernel(int variant) {
     case 11: return k_center<8, 16, false>;
     case 12: return k_center<16, 16, false>;
     case 13: return k_center<32, 16, false>;
+    case 14: return k_center2<16, 16>;
+    case 15: return k_center2<16, 24>;
     default: return nullptr;
   }
 }
