@@ -23,6 +23,7 @@ enum Stage {
 struct Selector;  // the learned center selector (selector.cu)
 constexpr int kMaxTreeRows = 65536;  // rows of a neighbour-joining tree
 constexpr int kCenterLanes = 8;      // branches of the center graph
+constexpr int kDerrWords = 4;        // msa_ctx::derr
 void selector_free(msa_ctx *ctx, Selector *s);
 
 }  // namespace msa_detail
@@ -84,7 +85,7 @@ struct msa_ctx {
 
   // small device scalars
   unsigned long long *dcounter = nullptr;
-  unsigned *derr = nullptr;     // derr[0] error bits, derr[1] overflow count
+  unsigned *derr = nullptr;     // [0] error bits, [1] overflow count, [2] subjects that resemble the center
   long long *dsmall = nullptr;  // [0] total, [1] argmin val, [2] argmin idx, [3] width, [4] sp
   DevBuf scratch;
   size_t scratch_half = 0;  // int2 offset of the second stream's boundary rows (center graph)

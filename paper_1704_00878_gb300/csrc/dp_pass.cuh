@@ -123,6 +123,10 @@ struct HalfRows {
   int rowsA, rowsB;
 };
 
+// scr_in holds the row above for in_cols columns; past them it reads as zeros.
+// col0: the column of the subjects that the pass's first column is (a caller
+// that starts inside the subjects hands in pointers and lengths from there on,
+// so col0 only moves the best cell's column).
 template <int G, int MODE = kFull>
 __device__ __forceinline__ void codes_pass2(const int8_t *__restrict__ profA,
                                             const int8_t *__restrict__ profB, int stride,
@@ -130,9 +134,9 @@ __device__ __forceinline__ void codes_pass2(const int8_t *__restrict__ profA,
                                             const uint8_t *__restrict__ rB, int LB, int Lw, int t,
                                             int base_lane, int blk, int nblkA, int nblkB, int padc,
                                             int o, int e, const int2 *__restrict__ scr_in,
-                                            int2 *__restrict__ scr_out,
+                                            int in_cols, int2 *__restrict__ scr_out,
                                             uint2 *__restrict__ coutA, uint2 *__restrict__ coutB,
-                                            const HalfRows &hr,
+                                            const HalfRows &hr, int col0,
                                             int (&bv)[2], int (&bi)[2], int (&bj)[2]) {
   constexpr int R = kCodesR;
   constexpr bool CODES = MODE == kFull || MODE == kBox;
@@ -161,8 +165,8 @@ __device__ __forceinline__ void codes_pass2(const int8_t *__restrict__ profA,
   uint32_t cur = fetch(t), nxt = fetch(G + t);
   int2 sv0 = make_int2(0, 0), sv1 = make_int2(0, 0);
   if (scr_in != nullptr) {
-    if (0 < Lw) sv0 = scr_in[0];
-    if (1 < Lw) sv1 = scr_in[1];
+    if (0 < in_cols) sv0 = scr_in[0];
+    if (1 < in_cols) sv1 = scr_in[1];
   }
   const int8_t *pbA = profA + t * R;
   const int8_t *pbB = OWN_ROWS ? profB + t * R : pbA;
@@ -182,10 +186,10 @@ __device__ __forceinline__ void codes_pass2(const int8_t *__restrict__ profA,
     }
     const int2 sv = sv0;
     sv0 = sv1;
-    if (scr_in != nullptr && k + 2 < Lw) sv1 = scr_in[k + 2];
+    if (scr_in != nullptr && k + 2 < in_cols) sv1 = scr_in[k + 2];
     if (t == 0) {
       rin = r0;
-      const bool above = scr_in != nullptr && k < Lw;
+      const bool above = scr_in != nullptr && k < in_cols;
       hin = above ? (uint32_t)sv.x : 0u;
       fin = above ? (uint32_t)sv.y : 0u;
     }
@@ -268,8 +272,8 @@ __device__ __forceinline__ void codes_pass2(const int8_t *__restrict__ profA,
   for (int r = 0; r < R; ++r) {
     const int va = C::lane0((int)rb[r]), vb = C::lane1((int)rb[r]);
     if constexpr (!OWN_ROWS) {
-      if (va > bv[0]) { bv[0] = va; bi[0] = blk * R + r + 1; bj[0] = (int)(rj[r] & 0xffffu) + 1; }
-      if (vb > bv[1]) { bv[1] = vb; bi[1] = blk * R + r + 1; bj[1] = (int)(rj[r] >> 16) + 1; }
+      if (va > bv[0]) { bv[0] = va; bi[0] = blk * R + r + 1; bj[0] = col0 + (int)(rj[r] & 0xffffu) + 1; }
+      if (vb > bv[1]) { bv[1] = vb; bi[1] = blk * R + r + 1; bj[1] = col0 + (int)(rj[r] >> 16) + 1; }
       continue;
     }
     const int row = blk * R + r + 1;

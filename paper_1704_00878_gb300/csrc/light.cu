@@ -125,9 +125,9 @@ __global__ void __launch_bounds__(NT, 1) k_light(SeqSet ss, Scoring sc, LightJob
         hr.mB[w] = mb;
       }
       codes_pass2<G, MODE>(pA, pB, stride, rA, LA, rB, LB, Lw, t, base_lane, blk, nblkA, nblkB,
-                           padc, sc.o, sc.e, sin, sout,
+                           padc, sc.o, sc.e, sin, Lw, sout,
                            cA ? cA + (size_t)blk * code_row_words(LA, G) : nullptr,
-                           cB ? cB + (size_t)blk * code_row_words(LB, G) : nullptr, hr, bv, bi, bj);
+                           cB ? cB + (size_t)blk * code_row_words(LB, G) : nullptr, hr, 0, bv, bi, bj);
       __syncwarp();
     }
 #pragma unroll

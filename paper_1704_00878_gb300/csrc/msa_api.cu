@@ -1132,7 +1132,7 @@ static int align_light(msa_ctx *ctx, int kc, int Lc) {
         pe - pb, P<int32_t>(ctx->d_len), P<int32_t>(ctx->d_perm), ss.res, ss.pstart, kc, sc.M, sc.K,
         sc.o, sc.e, Lc, G3, P<uint16_t>(ctx->ins), P<uint8_t>(ctx->occ), P<int32_t>(ctx->seg),
         P<int32_t>(ctx->score), ctx->derr, ctx->st, P<int32_t>(ctx->light_order) + pb,
-        P<int4>(ctx->light_win) + pb, P<unsigned long long>(ctx->light_keys) + pb));
+        P<int4>(ctx->light_win) + pb, P<unsigned long long>(ctx->light_keys) + pb, nullptr, 0u, 0));
     CK(cudaEventRecord(ctx->align_ev[3 * bi + 2], ctx->st));
   }
   CK(cudaStreamSynchronize(ctx->st));
@@ -1239,7 +1239,7 @@ int msa_create(msa_ctx **out, const msa_params *p, void *cuda_stream) {
     for (cudaStream_t &lane : ctx->cap_lanes) CK(cudaStreamCreateWithFlags(&lane, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&ctx->cap_fork, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ctx->cap_join, cudaEventDisableTiming));
-    CK(cudaMalloc(&ctx->derr, 2 * sizeof(unsigned)));
+    CK(cudaMalloc(&ctx->derr, kDerrWords * sizeof(unsigned)));
     CK(cudaMemset(ctx->derr, 0, 2 * sizeof(unsigned)));
     CK(cudaMalloc(&ctx->dsmall, 8 * sizeof(long long)));
     for (auto &ev : ctx->ev) CK(cudaEventCreate(&ev));
@@ -1568,7 +1568,7 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
   TRY(ensure(ctx, ctx->score, sizeof(int32_t) * n));
   CK(cudaMemsetAsync(ctx->ins.p, 0, sizeof(uint16_t) * row * n, ctx->st));
   CK(cudaMemsetAsync(ctx->occ.p, 0, row * n, ctx->st));
-  CK(cudaMemsetAsync(ctx->derr, 0, 2 * sizeof(unsigned), ctx->st));
+  CK(cudaMemsetAsync(ctx->derr, 0, kDerrWords * sizeof(unsigned), ctx->st));
   ctx->light_used = false;
   if (ctx->align_mode == MSA_ALIGN_BOX && packed) {
     int64_t matrix_cells = 0;
@@ -1654,8 +1654,28 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
   const int smem = codes_smem_bytes(ctx->K, npass * G * R);
   const int cta = align_cta(ctx, G, packed);
   const int grid = codes_grid(G, packed, smem, cta);
-  if (npass > 1)
-    TRY(ensure(ctx, ctx->scratch, (size_t)grid * (codes_threads(packed, cta) / G) * 2 * ctx->maxlen * sizeof(int2)));
+  // Similar subjects: decided on the device, so both fills are in the graph and
+  // one of them returns at once.  The vote and the idle launch cost about 10 us,
+  // so only from 8e9 cells on (3 ms), and only where a subject may match most of
+  // the center (a short one leaves no column out) and there are several passes.
+  const int Gs = ctx->align_group_fixed ? G : near_group(G, n);
+  const int near_npass = (Lc + Gs * R - 1) / (Gs * R), near_smem = codes_smem_bytes(ctx->K, near_npass * Gs * R);
+  bool near = packed && Gs >= 8 && near_npass > 1 && Lc >= 256 && ctx->smax > 0 &&
+                    (cells >= (int64_t)8e9 || ctx->align_group_fixed) && 2 * ctx->residues >= (int64_t)n * Lc;
+  const int ngrid = near ? near_grid(Gs, near_smem) : 0;
+  const size_t boundary = 2 * (size_t)ctx->maxlen * sizeof(int2);  // rows of a group
+  const size_t fscratch = npass > 1 ? (size_t)grid * (codes_threads(packed, cta) / G) * boundary : 0;
+  const size_t nscratch = (size_t)ngrid * (kCodes2Threads / Gs) * boundary;
+  // narrower groups want more boundary rows; where there is no room for them
+  // the full fill runs alone
+  if (near && nscratch > std::max(fscratch, ctx->scratch.cap) &&
+      (ctx->dev_limit || ensure(ctx, ctx->scratch, nscratch) != MSA_OK)) {
+    near = false;
+    cudaGetLastError();
+  }
+  if (fscratch) TRY(ensure(ctx, ctx->scratch, fscratch));
+  if (near && nscratch > ctx->scratch.cap) near = false;
+  unsigned *similar = near ? ctx->derr + 2 : nullptr;
   float ms_dp = 0.f, ms_tb = 0.f;
   // All batches as one CUDA graph (captured on the context's private stream,
   // launched on its stream, cached while the key holds): per batch the fill
@@ -1672,9 +1692,11 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
                               (int64_t)ctx->codes.p, (int64_t)ctx->code_off.p, (int64_t)ctx->best.p,
                               (int64_t)ctx->ins.p, (int64_t)ctx->occ.p, (int64_t)ctx->seg.p,
                               (int64_t)ctx->score.p, (int64_t)ctx->scratch.p, (int64_t)ctx->derr,
-                              (int64_t)ctx->dcounter, (int64_t)ctx->d_perm.p, ctx->maxlen};
+                              (int64_t)ctx->dcounter, (int64_t)ctx->d_perm.p, ctx->maxlen,
+                              near, Gs, ngrid, ctx->smax};
   for (auto [sb, se] : batches) { key.push_back(sb); key.push_back(se); }
   CK(codes_allow_smem(G, packed, smem, cta));
+  if (near) CK(near_allow_smem(Gs, near_smem));
   if (!ctx->align_exec || key != ctx->align_key) {
     if (ctx->align_exec) {
       CK(cudaStreamSynchronize(ctx->st));
@@ -1700,14 +1722,23 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
       e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi], ctx->cap_lanes[0], cudaEventRecordExternal);
       if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dcounter, 0, sizeof(unsigned long long), ctx->cap_lanes[0]);
       // offsets inside the batch are relative to the batch start
+      job.similar = similar;
+      job.similar_min = kSimilarSample / 2;
+      if (near && bi == 0 && e == cudaSuccess) e = launch_similar(ss, kc, similar, ctx->cap_lanes[0]);
       if (e == cudaSuccess) e = launch_codes(G, packed, ss, sc, job, grid, ctx->cap_lanes[0], false, cta);
+      if (near && e == cudaSuccess) {
+        job.npass = near_npass;
+        job.smax = ctx->smax;
+        e = launch_codes_near(Gs, ss, sc, job, ngrid, ctx->cap_lanes[0]);
+      }
       if (e == cudaSuccess) e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi + 1], ctx->cap_lanes[0], cudaEventRecordExternal);
       if (e == cudaSuccess)
         e = launch_traceback(P<uint8_t>(ctx->codes), P<int64_t>(ctx->code_off) + sb,
                              P<unsigned long long>(ctx->best) + sb, sb, se, P<int32_t>(ctx->d_len),
                              P<int32_t>(ctx->d_perm), ss.res, ss.pstart, kc, sc.M, sc.K, sc.o, sc.e,
                              Lc, G, P<uint16_t>(ctx->ins), P<uint8_t>(ctx->occ), P<int32_t>(ctx->seg),
-                             P<int32_t>(ctx->score), ctx->derr, ctx->cap_lanes[0]);
+                             P<int32_t>(ctx->score), ctx->derr, ctx->cap_lanes[0], nullptr, nullptr,
+                             nullptr, similar, kSimilarSample / 2, Gs);
       if (e == cudaSuccess) e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi + 2], ctx->cap_lanes[0], cudaEventRecordExternal);
     }
     cudaGraph_t graph = nullptr;
@@ -1720,7 +1751,7 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
     ctx->align_exec = exec;
     ctx->align_key = key;
   }
-  ctx->launches += 2 * nb;
+  ctx->launches += 2 * nb + (near ? nb + 1 : 0);
   stage_begin(ctx, ST_ALIGN);
   CK(cudaGraphLaunch(ctx->align_exec, ctx->st));
   stage_end(ctx, ST_ALIGN);

@@ -111,8 +111,10 @@ __global__ void k_traceback(const uint8_t *__restrict__ codes, const int64_t *__
                             int32_t *__restrict__ seg, int32_t *__restrict__ score,
                             unsigned *err, const int32_t *__restrict__ list,
                             const int4 *__restrict__ box,
-                            const unsigned long long *__restrict__ box_best) {
+                            const unsigned long long *__restrict__ box_best,
+                            const unsigned *__restrict__ similar, unsigned similar_min, int Gs) {
   __shared__ int8_t sM[MSA_MAX_ALPHABET * MSA_MAX_ALPHABET];
+  if (similar && *similar >= similar_min) G = Gs;  // codes of the bounded fill
   for (int i = threadIdx.x; i < K * K; i += blockDim.x) sM[i] = M[i];
   __syncthreads();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -492,14 +494,16 @@ cudaError_t launch_traceback(const uint8_t *codes, const int64_t *code_off,
                              const int8_t *M, int K, int o, int e, int Lc, int G,
                              uint16_t *ins, uint8_t *occ, int32_t *seg, int32_t *score,
                              unsigned *err, cudaStream_t st, const int32_t *list, const int4 *box,
-                             const unsigned long long *box_best) {
+                             const unsigned long long *box_best, const unsigned *similar,
+                             unsigned similar_min, int Gs) {
   const int cnt = se - sb;
   if (cnt <= 0) return cudaSuccess;
   const int threads = 128;
   k_traceback<<<(cnt + threads - 1) / threads, threads, 0, st>>>(codes, code_off, best, sb, se, len,
                                                                  perm, res, pstart, center, M, K, o,
                                                                  e, Lc, G, ins, occ, seg, score, err,
-                                                                 list, box, box_best);
+                                                                 list, box, box_best, similar,
+                                                                 similar_min, Gs);
   return cudaGetLastError();
 }
 

@@ -30,7 +30,8 @@ cudaError_t launch_traceback(const uint8_t *codes, const int64_t *code_off,
                              uint16_t *ins, uint8_t *occ, int32_t *seg, int32_t *score,
                              unsigned *err, cudaStream_t st, const int32_t *list = nullptr,
                              const int4 *box = nullptr,
-                             const unsigned long long *box_best = nullptr);
+                             const unsigned long long *box_best = nullptr,
+                             const unsigned *similar = nullptr, unsigned similar_min = 0, int Gs = 0);
 
 cudaError_t launch_colmax(const uint16_t *ins, int n, int Lc, int32_t *G, cudaStream_t st);
 cudaError_t launch_scan(const int32_t *G, int Lc, int32_t *off, int64_t *width, cudaStream_t st);

@@ -881,6 +881,7 @@ __global__ void __launch_bounds__(256) k_codes(SeqSet ss, Scoring sc, CodesJob j
 // once per lane.
 template <int G, int NT>
 __global__ void __launch_bounds__(NT, 1) k_codes2(SeqSet ss, Scoring sc, CodesJob job) {
+  if (job.similar && *job.similar >= job.similar_min) return;  // k_codes_near fills these
   constexpr int R = kCodesR, NG = NT / G, GPW = 32 / G;
   extern __shared__ __align__(16) int8_t smem[];
   __shared__ int8_t sM[MSA_MAX_ALPHABET * MSA_MAX_ALPHABET];
@@ -925,10 +926,10 @@ __global__ void __launch_bounds__(NT, 1) k_codes2(SeqSet ss, Scoring sc, CodesJo
       int2 *sout = p + 1 < job.npass ? scr + (size_t)(p & 1) * job.scratch_cols : nullptr;
       const int blk = p * G + t;
       codes_pass2<G, kFull>(smem + p * G * R, smem + p * G * R, stride, rA, LA, rB, LB, Lw, t,
-                            base_lane, blk, nblk, nblk, padc, sc.o, sc.e, sin, sout,
+                            base_lane, blk, nblk, nblk, padc, sc.o, sc.e, sin, Lw, sout,
                             cA ? cA + (size_t)blk * code_row_words(LA, G) : nullptr,
-                            cB ? cB + (size_t)blk * code_row_words(LB, G) : nullptr, HalfRows{}, bv,
-                            bi, bj);
+                            cB ? cB + (size_t)blk * code_row_words(LB, G) : nullptr, HalfRows{}, 0,
+                            bv, bi, bj);
       __syncwarp();
     }
 #pragma unroll
@@ -946,6 +947,189 @@ __global__ void __launch_bounds__(NT, 1) k_codes2(SeqSet ss, Scoring sc, CodesJo
       if (t == 0 && (s2 == 0 ? valid : hasb)) job.best[ks - job.sb] = best_key(v, bi2, bj2);
     }
   }
+}
+
+// ------------------------------------------------------------ similar subjects
+// A path that pairs m residues scores at most smax m, and from the cell (i, j)
+// on it pairs at most min(Lc - 1 - i, Ls - 1 - j) more.  So once a subject's best
+// score is known to be at least v, a pass of rows [r0, r1) needs only the columns
+// that a path of score v can reach:
+//   from the left   the first column of the row above with H + smax min(Lc - r0,
+//                   Ls - 1 - column) >= v; or, while a path of v could still begin
+//                   below that row, diagonal -(Lc - ceil(v / smax)),
+//   to the right    diagonal Ls - r0 - ceil((v - top) / smax), top the best H of
+//                   those columns (0 in the first pass): further right the rest
+//                   of the subject is too short.
+// Cells outside read as zeros and the cells inside as lower bounds of themselves,
+// exact (values, ties and codes) wherever a path of score v runs.  v is a guess:
+// smax min(Lc, Ls) less the share that the warp's previous subjects fell short
+// by and a fifth more, at its first item a quarter.  A score of at least v proves
+// the columns; a subject that falls short runs again with its score as v, and
+// past a share of 45 % every column is filled.  Integer bound as k_codes2, in
+// fewer columns.  Alignment of DNA sequences that differ in 4 % of their residues:
+// 20,000 of 1,500 21.7 ms with every column, 16.1 with the diagonals alone, 11.0
+// so; 60,000 63.1 -> 28.6 ms, 10,000 of 2,900 48.7 -> 22.6 ms.
+template <int G>
+__global__ void __launch_bounds__(256, 1) k_codes_near(SeqSet ss, Scoring sc, CodesJob job) {
+  if (*job.similar < job.similar_min) return;  // k_codes2 has filled every column
+  constexpr int R = kCodesR, NT = 256, NG = NT / G, GPW = 32 / G;
+  constexpr int kFirstShare = 256, kMaxShare = 376, kEvery = 1024;  // of 1024
+  extern __shared__ __align__(16) int8_t smem[];
+  __shared__ int8_t sM[MSA_MAX_ALPHABET * MSA_MAX_ALPHABET];
+  const int K = sc.K, padc = K, smax = job.smax;
+  const int rows = job.npass * G * R;
+  const int stride = dround_up(rows, MSA_PROF_ALIGN);
+  for (int i = threadIdx.x; i < K * K; i += NT) sM[i] = sc.M[i];
+  __syncthreads();
+  const int Lc = ss.len[job.center];
+  const uint8_t *rc = ss.res + ss.pstart[job.center];
+  for (int idx = threadIdx.x; idx < (K + 1) * rows; idx += NT) {
+    const int r = idx / rows, i = idx - r * rows;
+    int v = 0;  // padding: score -o
+    if (r < K && i < Lc) v = sM[rc[i] * K + r] + sc.o;
+    smem[r * stride + i] = (int8_t)v;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, t = threadIdx.x % G, g = threadIdx.x / G;
+  const int base_lane = lane - t;
+  const int nblk = (Lc + R - 1) / R;
+  int2 *scr = job.scratch + ((size_t)blockIdx.x * NG + g) * 2 * job.scratch_cols;
+  const int nsub = job.se - job.sb, nitem = (nsub + 1) / 2;
+  int share = kFirstShare;
+  for (;;) {
+    int x0 = 0;
+    if (lane == 0) x0 = (int)atomicAdd(job.counter, (unsigned long long)GPW);
+    x0 = __shfl_sync(MSA_FULL_MASK, x0, 0);
+    if (x0 >= nitem) break;
+    const int x = x0 + lane / G;
+    const bool valid = x < nitem;
+    const int k[2] = {job.se - 1 - 2 * (valid ? x : 0), job.se - 2 - 2 * (valid ? x : 0)};  // longest first
+    const bool has[2] = {valid, valid && k[1] >= job.sb};
+    int Ls[2], full[2], guess[2];  // full: the score of a perfect match
+    const uint8_t *rs[2];
+    uint2 *codes[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      Ls[s] = has[s] ? ss.len[k[s]] : 0;
+      rs[s] = has[s] ? ss.res + ss.pstart[k[s]] : ss.res;
+      codes[s] = has[s] ? reinterpret_cast<uint2 *>(job.codes + job.code_off[k[s] - job.sb]) : nullptr;
+      full[s] = smax * min(Lc, Ls[s]);
+      guess[s] = share < kEvery ? full[s] - full[s] * share / 1024 : 0;
+    }
+    const int Lw = __reduce_max_sync(MSA_FULL_MASK, max(Ls[0], Ls[1]));
+    int bv[2], bi[2], bj[2];
+    for (;;) {
+      int first[2] = {0, 0}, top[2] = {0, 0};  // of the row above: first column and best H that may lead to v
+      int above = 0;                           // and the end of its columns
+#pragma unroll
+      for (int s = 0; s < 2; ++s) bv[s] = bi[s] = bj[s] = 0;
+      for (int p = 0; p < job.npass; ++p) {
+        const int2 *sin = p > 0 ? scr + (size_t)((p - 1) & 1) * job.scratch_cols : nullptr;
+        int2 *sout = p + 1 < job.npass ? scr + (size_t)(p & 1) * job.scratch_cols : nullptr;
+        const int blk = p * G + t, r0 = p * G * R, r1 = min(Lc, r0 + G * R);
+        int c0 = Lw, c1 = 0;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          if (!has[s]) continue;
+          const int need = guess[s] - top[s];
+          const int begin = smax * (Lc - r0) < guess[s] ? first[s] : r0 - (Lc - (guess[s] + smax - 1) / smax);
+          const int diag = need > 0 ? Ls[s] - r0 - (need + smax - 1) / smax : Ls[s];
+          c0 = min(c0, max(0, begin) & ~3);  // code words are stored by fours
+          c1 = max(c1, min(Ls[s], r1 + diag));
+        }
+        c0 = __reduce_min_sync(MSA_FULL_MASK, c0);
+        c1 = __reduce_max_sync(MSA_FULL_MASK, c1);
+        if (c1 > c0)
+          codes_pass2<G, kFull>(smem + p * G * R, smem + p * G * R, stride, rs[0] + c0, Ls[0] - c0,
+                                rs[1] + c0, Ls[1] - c0, c1 - c0, t, base_lane, blk, nblk, nblk, padc,
+                                sc.o, sc.e, sin ? sin + c0 : nullptr, above - c0, sout ? sout + c0 : nullptr,
+                                codes[0] ? codes[0] + (size_t)blk * code_row_words(Ls[0], G) + c0 : nullptr,
+                                codes[1] ? codes[1] + (size_t)blk * code_row_words(Ls[1], G) + c0 : nullptr,
+                                HalfRows{}, c0, bv, bi, bj);
+        above = c1;
+        __syncwarp();
+        if (!sout) continue;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) { first[s] = Lw; top[s] = -1; }
+        for (int j = c0 + t; j < c1; j += G) {
+          const int h = sout[j].x;
+#pragma unroll
+          for (int s = 0; s < 2; ++s) {
+            const int hv = s ? Cell<true>::lane1(h) : Cell<true>::lane0(h);
+            const int left = min(Lc - r1, Ls[s] - 1 - j);
+            if (left >= 0 && hv + smax * left >= guess[s]) {
+              first[s] = min(first[s], j);
+              top[s] = max(top[s], hv);
+            }
+          }
+        }
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1)
+#pragma unroll
+          for (int s = 0; s < 2; ++s) {
+            first[s] = min(first[s], __shfl_xor_sync(MSA_FULL_MASK, first[s], off));
+            top[s] = max(top[s], __shfl_xor_sync(MSA_FULL_MASK, top[s], off));
+          }
+      }
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) {
+          const int ov = __shfl_xor_sync(MSA_FULL_MASK, bv[s], off);
+          const int oi = __shfl_xor_sync(MSA_FULL_MASK, bi[s], off);
+          const int oj = __shfl_xor_sync(MSA_FULL_MASK, bj[s], off);
+          const bool take = ov > bv[s] || (ov == bv[s] && (oi < bi[s] || (oi == bi[s] && oj < bj[s])));
+          if (take) { bv[s] = ov; bi[s] = oi; bj[s] = oj; }
+        }
+      if (!__any_sync(MSA_FULL_MASK, bv[0] < guess[0] || bv[1] < guess[1])) break;
+      // (more columns find no less, so the second fill is the last)
+#pragma unroll
+      for (int s = 0; s < 2; ++s) guess[s] = min(guess[s], bv[s]);
+    }
+    // the next guess (a score of 15 bits and 1/1024 stay within an int)
+    int far = 0;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      if (full[s] > 0) far = max(far, (full[s] - bv[s]) * 1024 / full[s]);
+      if (t == 0 && has[s]) job.best[k[s] - job.sb] = best_key(bv[s], bi[s], bj[s]);
+    }
+    far = __reduce_max_sync(MSA_FULL_MASK, far);
+    share = far > kMaxShare ? kEvery : far + far / 5 + 8;
+  }
+}
+
+// Whether the subjects resemble the center: of kSimilarSample subjects spread
+// over the set, how many share at least 12 of 32 words of 12 residues with it
+// (residues that differ in 8 % or more share fewer).  A CTA per subject, a word
+// per lane, a quarter of the center per warp: about 3 us.
+constexpr int kWordLen = 12, kWordBits = 5;
+
+__global__ void __launch_bounds__(128) k_similar(SeqSet ss, int center, unsigned *similar) {
+  __shared__ unsigned s_found[4];
+  const int k = (int)((long long)blockIdx.x * ss.n / gridDim.x), Ls = ss.len[k], Lc = ss.len[center];
+  if (Ls < 4 * kWordLen) return;
+  const uint8_t *rs = ss.res + ss.pstart[k], *rc = ss.res + ss.pstart[center];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned long long mask = (1ull << (kWordLen * kWordBits)) - 1;
+  unsigned long long mine = 0, key = 0;
+  const int at = lane * (Ls - kWordLen) / 31;
+  for (int u = 0; u < kWordLen; ++u) mine = (mine << kWordBits) | (__ldg(rs + at + u) & 31u);
+  // this warp's words end in [a, b)
+  const int a = max(kWordLen - 1, warp * Lc / 4), b = (warp + 1) * Lc / 4;
+  bool found = false;
+  for (int i0 = a - (kWordLen - 1); i0 < b; i0 += 32) {
+    const uint32_t c = i0 + lane < b ? (uint32_t)__ldg(rc + i0 + lane) & 31u : 0u;
+    const int m = min(32, b - i0);
+#pragma unroll 8
+    for (int u = 0; u < m; ++u) {
+      key = ((key << kWordBits) | __shfl_sync(MSA_FULL_MASK, c, u)) & mask;
+      found |= key == mine && i0 + u >= a;
+    }
+  }
+  const unsigned votes = __ballot_sync(MSA_FULL_MASK, found);
+  if (lane == 0) s_found[warp] = votes;
+  __syncthreads();
+  if (threadIdx.x == 0 && __popc(s_found[0] | s_found[1] | s_found[2] | s_found[3]) >= 12) atomicAdd(similar, 1u);
 }
 
 }  // namespace
@@ -1132,6 +1316,44 @@ int codes_group(int Lc, bool packed, int K, int64_t n, double mean_len, int max_
     if (G == 32 || est < best) { best = est; best_g = G; }
   }
   return best_g;
+}
+
+static codes_fn near_kernel(int G) {
+  return G == 8 ? k_codes_near<8> : G == 16 ? k_codes_near<16> : G == 32 ? k_codes_near<32> : (codes_fn) nullptr;
+}
+
+int near_group(int G, int64_t n) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  for (int g = 8; g < G; g *= 2)
+    if (n / 2 / (32 / g) >= 4 * (int64_t)sms * (kCodes2Threads / 32)) return g;
+  return G;
+}
+
+int near_grid(int G, int smem) {
+  codes_fn fn = near_kernel(G);
+  return fn ? occupancy_grid((const void *)fn, kCodes2Threads, smem) : 0;
+}
+
+cudaError_t near_allow_smem(int G, int smem) {
+  codes_fn fn = near_kernel(G);
+  if (!fn) return cudaErrorInvalidValue;
+  if (smem <= 40 * 1024) return cudaSuccess;  // static shared memory counts too
+  return cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
+
+cudaError_t launch_codes_near(int G, const SeqSet &ss, const Scoring &sc, const CodesJob &job, int grid,
+                              cudaStream_t st) {
+  codes_fn fn = near_kernel(G);
+  if (!fn) return cudaErrorInvalidValue;
+  fn<<<grid, kCodes2Threads, codes_smem_bytes(sc.K, job.npass * G * kCodesR), st>>>(ss, sc, job);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_similar(const SeqSet &ss, int center, unsigned *similar, cudaStream_t st) {
+  k_similar<<<kSimilarSample, 128, 0, st>>>(ss, center, similar);
+  return cudaGetLastError();
 }
 
 cudaError_t codes_allow_smem(int G, bool packed, int smem, int threads) {

@@ -1,0 +1,91 @@
+"""Alignment of similar sequences, where the fill leaves out columns that no
+best path can reach: against the oracle with shifts, long indels, repeats (tied
+and off-diagonal paths) and unrelated subjects among similar ones, and against
+the int32 kernels (which fill every column) over several subjects per warp."""
+import numpy as np
+import pytest
+
+import oracle
+from seqgen import blosum62, dna_matrix, pack_sequences
+from tests._gpu import binding, make_ctx, oracle_problem
+
+pytestmark = pytest.mark.gpu
+
+
+def mutate(rng, s, p, pool):
+    s = s.copy()
+    hit = rng.random(s.size) < p
+    s[hit] = rng.choice(pool, size=int(hit.sum()))
+    return s
+
+
+def variants(rng, center, pool):
+    """Subjects of every kind a window can meet, similar ones first."""
+    L = center.size
+    seqs = [mutate(rng, center, p, pool) for p in (0.0, 0.0, 0.01, 0.03, 0.05, 0.08, 0.15)]
+    for k in (3, 20, 90, 250):
+        seqs.append(mutate(rng, np.concatenate([center[:L // 2], center[L // 2 + k:]]), 0.02, pool))
+        seqs.append(mutate(rng, np.concatenate([center[:L // 3], rng.choice(pool, size=k), center[L // 3:]]), 0.02, pool))
+        seqs.append(mutate(rng, center[k:], 0.02, pool))
+        seqs.append(mutate(rng, center[:L - k], 0.02, pool))
+        seqs.append(np.concatenate([rng.choice(pool, size=k), center, rng.choice(pool, size=2 * k)]))
+    # a segment repeated, moved to the other end, and halves swapped
+    seqs.append(np.concatenate([center[:200], center[:200], center]))
+    seqs.append(np.concatenate([center[-150:], center]))
+    seqs.append(np.concatenate([center[L // 2:], center[:L // 2]]))
+    seqs.append(np.tile(center[:60], 12))
+    seqs.append(rng.choice(pool, size=L))
+    seqs.append(rng.choice(pool, size=70))
+    seqs.append(center[100:140])
+    return seqs
+
+
+@pytest.mark.parametrize("kind, o, e", [("dna", 5, 2), ("dna", 2, 1), ("dna", 3, 3), ("protein", 11, 1)])
+@pytest.mark.parametrize("lanes", [8, 16, 32])
+def test_similar_subjects_match_the_oracle(kind, o, e, lanes):
+    b = binding()
+    rng = np.random.default_rng(o * 100 + lanes)
+    alph, M = blosum62() if kind == "protein" else dna_matrix()
+    pool = np.frombuffer(("ARNDCQEGHILKMFPSTWYV" if kind == "protein" else "ACGT").encode(), np.uint8)
+    half = rng.choice(pool, size=330)
+    for center in (rng.choice(pool, size=700), np.concatenate([half, mutate(rng, half, 0.03, pool)])):
+        letters, offsets = pack_sequences([center] + variants(rng, center, pool))
+        prob = oracle_problem(letters, offsets, alph, M, o, e)
+        oseg, oins, oocc, _, _, _ = oracle.msa(prob, 0)
+        with make_ctx(alph, M, o, e) as h:
+            b.msa_load(h, letters, offsets)
+            b.msa_set_align_group(h, lanes)
+            b.msa_align_to_center(h, 0)
+            seg, ins, occ = b.msa_alignment_info(h)
+        assert (seg == oseg).all()
+        assert (ins == oins).all() and (occ == oocc).all()
+
+
+@pytest.mark.parametrize("odd_every", [0, 13, 2, 1])
+def test_several_subjects_per_warp_match_full_columns(odd_every):
+    """Guesses that come from a warp's previous subjects, too high ones
+    included: subjects that are unrelated or half as long at a rate (too many of
+    them, and every column is filled)."""
+    b = binding()
+    rng = np.random.default_rng(odd_every)
+    alph, M = dna_matrix()
+    pool = np.frombuffer(b"ACGT", np.uint8)
+    center = rng.choice(pool, size=300)
+    seqs = [center]
+    for x in range(24000):
+        if odd_every and x % odd_every == 0:
+            seqs.append(rng.choice(pool, size=int(rng.integers(60, 310))) if x & 1 else center[:int(rng.integers(100, 200))])
+            continue
+        s = mutate(rng, center, (0.0, 0.02, 0.06)[x % 3], pool)
+        a, k = int(rng.integers(0, 30)), int(rng.integers(30, 270))
+        seqs.append(np.concatenate([s[a:k], s[k + int(rng.integers(0, 6)):]]))
+    letters, offsets = pack_sequences(seqs)
+    got = []
+    for precision in (b.MSA_AUTO, b.MSA_INT32):
+        with make_ctx(alph, M, 5, 2, precision=precision) as h:
+            b.msa_load(h, letters, offsets)
+            b.msa_set_align_group(h, 8)
+            b.msa_align_to_center(h, 0)
+            got.append(b.msa_alignment_info(h))
+    for x, y in zip(*got):
+        assert (x == y).all()
