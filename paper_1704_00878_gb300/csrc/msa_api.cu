@@ -409,6 +409,8 @@ struct CenterClass {
 struct ClassPlan {
   CenterClass cc;
   int nq_list, npass, smem, grid;
+  // a class with a bounded twin (k_center_near) for similar sequences, the twin
+  enum Role { kAlone, kFull, kNear } role = kAlone;
   size_t prefix_off;  // into the concatenated prefix of all planned classes
   int64_t n_items;
 };
@@ -539,13 +541,24 @@ int launch_class(msa_ctx *ctx, int mode, int nq_list, const CenterClass &cc,
 // single submission with no host round trip between buckets.  The graph is
 // captured on the context's private capture stream and launched on its
 // stream (which may be the legacy default stream).
+// near: classes whose plan says so get the full and the bounded kernel, and a
+// vote at the graph's start decides on the device which of the two works.
 int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, int sub_off,
-                 int sub_n, const SeqSet &ss, const int32_t *self) {
+                 int sub_n, const SeqSet &ss, const int32_t *self, int nq) {
   const Scoring sc = scoring(ctx);
   std::vector<int> top(kNumCenterVariants, 0);
-  for (const ClassPlan &pl : plans) top[pl.cc.variant] = std::max(top[pl.cc.variant], pl.smem);
-  for (int v = 0; v < kNumCenterVariants; ++v)
+  std::vector<int> top_near(kNumCenterVariants, 0);
+  int num_near = 0;
+  for (const ClassPlan &pl : plans) {
+    int &most = (pl.role == ClassPlan::kNear ? top_near : top)[pl.cc.variant];
+    most = std::max(most, pl.smem);
+    if (pl.role == ClassPlan::kNear) ++num_near;
+  }
+  for (int v = 0; v < kNumCenterVariants; ++v) {
     if (top[v] > 0) CK(center_allow_smem(v, top[v]));
+    if (top_near[v] > 0) CK(center_allow_smem(v, top_near[v], true));
+  }
+  unsigned *similar = ctx->derr + 2;
   unsigned long long *cnt = P<unsigned long long>(ctx->counters);
   // Everything the graph bakes in; a selection with the same key (the same
   // set and buffers, e.g. a repeated step) relaunches the cached graph.
@@ -562,9 +575,14 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
   };
   std::vector<int64_t> key = {mode, sub_off, sub_n, (int64_t)ss.res, (int64_t)ss.pstart,
                               (int64_t)ss.len, ss.n, (int64_t)sc.M, sc.K, sc.o, sc.e,
-                              (int64_t)cnt, (int64_t)plans.size()};
+                              (int64_t)cnt, (int64_t)plans.size(), nq, (int64_t)similar};
   for (size_t c = 0; c < plans.size(); ++c) {
     CenterJob job = class_job(ctx, mode, plans[c], sub_off, sub_n, cnt + c, self);
+    if (plans[c].role != ClassPlan::kAlone) {
+      job.similar = similar;
+      job.similar_min = kSimilarSample / 2;
+      job.smax = ctx->smax;
+    }
     if (lane_of(c) == 1) job.scratch += ctx->scratch_half;
     jobs.push_back(job);
     const int64_t f[] = {plans[c].cc.variant, plans[c].grid, plans[c].smem, job.mode,
@@ -572,7 +590,7 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
                          (int64_t)job.prefix, job.n_items, job.npass, (int64_t)job.counter,
                          (int64_t)job.pairsum, (int64_t)job.self, job.sat_thresh,
                          (int64_t)job.ovf, (int64_t)job.ovf_count, job.ovf_cap, (int64_t)job.err,
-                         (int64_t)job.scratch, job.scratch_cols, (int64_t)job.streams};
+                         (int64_t)job.scratch, job.scratch_cols, (int64_t)job.streams, plans[c].role, job.smax};
     key.insert(key.end(), f, f + sizeof(f) / sizeof(f[0]));
   }
   if (!ctx->center_exec || key != ctx->center_key) {
@@ -584,6 +602,12 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
     }
     CK(cudaStreamBeginCapture(ctx->cap_lanes[0], cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * plans.size(), ctx->cap_lanes[0]);
+    if (num_near > 0 && e == cudaSuccess) {
+      e = cudaMemsetAsync(similar, 0, sizeof(unsigned), ctx->cap_lanes[0]);
+      if (e == cudaSuccess)
+        e = launch_similar(ss, sub_n, mode == 0 ? nullptr : P<int32_t>(ctx->qlist), 0, nq, similar,
+                           ctx->cap_lanes[0]);
+    }
     if (e == cudaSuccess) e = cudaEventRecord(ctx->cap_fork, ctx->cap_lanes[0]);
     const int lanes = (int)std::min<size_t>(plans.size(), kCenterLanes);
     for (int k = 1; k < lanes && e == cudaSuccess; ++k)
@@ -592,7 +616,7 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
     for (size_t k = 0; k < plans.size() && e == cudaSuccess; ++k) {
       const size_t c = plans.size() - 1 - k;
       e = launch_center(plans[c].cc.variant, ss, sc, jobs[c], plans[c].grid,
-                        ctx->cap_lanes[lane_of(c)], false);
+                        ctx->cap_lanes[lane_of(c)], false, plans[c].role == ClassPlan::kNear);
       if (e != cudaSuccess) failed = (int)c;
     }
     for (int k = 1; k < lanes; ++k) {
@@ -616,7 +640,7 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
     ctx->center_exec = exec;
     ctx->center_key = key;
   }
-  ctx->launches += (int64_t)plans.size();
+  ctx->launches += (int64_t)plans.size() + (num_near > 0);
   stage_begin(ctx, ST_CENTER_K);
   CK(cudaGraphLaunch(ctx->center_exec, ctx->st));
   stage_end(ctx, ST_CENTER_K);
@@ -760,26 +784,59 @@ int run_center(msa_ctx *ctx, int mode, const std::vector<int32_t> &qsorted, cons
     ctx->cells[0] = 0;
     return MSA_OK;
   }
+  int64_t center_cells = 0;
+  if (mode == 0) {  // pairs q < s
+    for (int x = q_begin; x < q_end; ++x) center_cells += (int64_t)lens[x] * suffix[x + 1];
+  } else {
+    for (int q : qsorted) center_cells += (int64_t)lens[q] * suffix[0];
+  }
+  // One bounded kernel for all multi-pass pairs: passes of few rows leave out more,
+  // and one class has one tail.  3,000 (1,000) DNA sequences of 1,500 against 100
+  // references: 51.7 (18.9) ms in the full kernel's own shapes, one class each,
+  // 47.7 (17.8) in one of 8 lanes x 20 rows; short lists take 16 x 16 (500 against
+  // 60 references 8.1 ms, 9.3 in 8 x 20).
+  // The vote and the idle launches cost about 10 us: from 2e10 cells on (3 ms).
+  // Cells near the int16 limit (which the precision setting may allow), profiles
+  // beyond shared memory and a device memory limit (the narrower groups want more
+  // boundary rows) keep the full kernel.
+  const int near_variant = fill(8) < 1.0 ? 14 : 1;
+  const int longest = p_end > p_begin ? qlen[std::min(2 * p_end, x1) - 1] : 0;
+  const bool may_near = center_cells >= (int64_t)2e10 && longest > 0 && ctx->smax > 0 && !ctx->dev_limit &&
+                        (long long)longest * ctx->smax <= sat_thresh(ctx) &&
+                        variant_fits(ctx, near_variant, longest);
+  std::vector<CenterClass> twins;
   std::vector<ClassPlan> plans;
   std::vector<int64_t> prefix_all;
   for (const CenterClass &cc : classes) {
     // a paired class may not pair across the packed / int32 boundary
     const int nq_list = kCenterVariants[cc.variant].paired ? x1 : nq;
     plans.push_back(plan_class(ctx, mode, nq_list, cc, qlen, n, prefix_all, streams));
+    ClassPlan &pl = plans.back();
+    bool near = may_near && kCenterVariants[cc.variant].paired && pl.npass > 1;
+    for (int u = cc.ub; near && u < cc.ue; ++u) near = streams[u].y == 1;
+    if (!near) continue;
+    pl.role = ClassPlan::kFull;
+    if (!twins.empty() && twins.back().ue == cc.ub) twins.back().ue = cc.ue;
+    else twins.push_back({near_variant, cc.ub, cc.ue});
   }
-  TRY(stage_plans(ctx, plans, prefix_all, streams));
+  for (const CenterClass &cc : twins) {  // (last: the launch order is from the back)
+    plans.push_back(plan_class(ctx, mode, x1, cc, qlen, n, prefix_all, streams));
+    plans.back().role = ClassPlan::kNear;
+  }
+  int rc = stage_plans(ctx, plans, prefix_all, streams);
+  if (rc != MSA_OK && !twins.empty()) {  // no room for the twins' boundary rows
+    cudaGetLastError();
+    plans.resize(plans.size() - twins.size());
+    for (ClassPlan &pl : plans) pl.role = ClassPlan::kAlone;
+    rc = stage_plans(ctx, plans, prefix_all, streams);
+  }
+  TRY(rc);
   const int32_t *self = view ? view->self : P<int32_t>(ctx->self);
-  TRY(launch_plans(ctx, mode, plans, 0, n, ss, self));
+  TRY(launch_plans(ctx, mode, plans, 0, n, ss, self, nq));
   CK(cudaStreamSynchronize(ctx->st));
   stage_collect(ctx, ST_CENTER_K);
   const float center_ms = ctx->stage_ms[ST_CENTER_K];
-  int64_t cells = 0;
-  if (mode == 0) {  // pairs q < s
-    for (int x = q_begin; x < q_end; ++x) cells += (int64_t)lens[x] * suffix[x + 1];
-  } else {
-    for (int q : qsorted) cells += (int64_t)lens[q] * suffix[0];
-  }
-  ctx->cells[0] = cells;
+  ctx->cells[0] = center_cells;
   ctx->stage_ms[ST_CENTER_K] = center_ms;
 
   // pairs whose packed lanes may have overflowed: recompute in int32
@@ -1726,7 +1783,7 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
       // offsets inside the batch are relative to the batch start
       job.similar = similar;
       job.similar_min = kSimilarSample / 2;
-      if (near && bi == 0 && e == cudaSuccess) e = launch_similar(ss, kc, similar, ctx->cap_lanes[0]);
+      if (near && bi == 0 && e == cudaSuccess) e = launch_similar(ss, n, nullptr, kc, 1, similar, ctx->cap_lanes[0]);
       if (e == cudaSuccess) e = launch_codes(G, packed, ss, sc, job, grid, ctx->cap_lanes[0], false, cta);
       if (near && e == cudaSuccess) {
         job.npass = near_npass;

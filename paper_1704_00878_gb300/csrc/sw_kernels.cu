@@ -230,15 +230,16 @@ k_center(SeqSet ss, Scoring sc, CenterJob job) {
 // offset t*pitch, pitch = R or R + 4 so that pitch/4 is odd: the eight lanes of
 // a load phase hit eight different 16-byte bank groups whatever residues they
 // read.
-// IN / OUT: the pass reads the row above from scr_in / writes its bottom row
-// to scr_out (compile-time, so a single-pass query carries no test for them).
+// IN / OUT: the pass reads the row above from scr_in (in_cols columns of it,
+// zeros beyond) / writes its bottom row to scr_out (compile-time, so a
+// single-pass query carries no test for them).
 __host__ __device__ constexpr int center_pitch(int R) { return (R / 4) % 2 ? R : R + 4; }
 
 template <int G, int R, bool IN, bool OUT>
 __device__ __forceinline__ int wave_pass_pp(const uint32_t *__restrict__ prof, int stride,
                                             const uint8_t *__restrict__ rs, int Ls, int Lw, int t,
                                             int base_lane, int padc, int o, int e, bool top,
-                                            const int2 *__restrict__ scr_in,
+                                            const int2 *__restrict__ scr_in, int in_cols,
                                             int2 *__restrict__ scr_out) {
   using C = Cell<true>;
   static_assert(R % 4 == 0, "16-byte profile loads");
@@ -252,8 +253,8 @@ __device__ __forceinline__ int wave_pass_pp(const uint32_t *__restrict__ prof, i
   uint32_t cur = residue_at(rs, Ls, t, pc), nxt = residue_at(rs, Ls, G + t, pc);
   int2 sv0 = make_int2(0, 0), sv1 = make_int2(0, 0);
   if (IN) {
-    if (0 < Lw) sv0 = scr_in[0];
-    if (1 < Lw) sv1 = scr_in[1];
+    if (0 < in_cols) sv0 = scr_in[0];
+    if (1 < in_cols) sv1 = scr_in[1];
   }
   const uint32_t *pb = prof + t * center_pitch(R);
   const int steps = Lw + G - 1;
@@ -268,11 +269,11 @@ __device__ __forceinline__ int wave_pass_pp(const uint32_t *__restrict__ prof, i
     const int2 sv = sv0;
     if (IN) {
       sv0 = sv1;
-      if (k + 2 < Lw) sv1 = scr_in[k + 2];
+      if (k + 2 < in_cols) sv1 = scr_in[k + 2];
     }
     if (t == 0) {
       rin = r0;
-      const bool above = IN && k < Lw;
+      const bool above = IN && k < in_cols;
       hin = above ? sv.x : 0;
       fin = above ? sv.y : 0;
     }
@@ -314,12 +315,35 @@ __device__ __forceinline__ int wave_pass_pp(const uint32_t *__restrict__ prof, i
   return best;
 }
 
+// The sums of a query pair's two scores (int16 lanes) with subject s.
+__device__ __forceinline__ void center_sums(const CenterJob &job, int best, int qA, int qB, int s,
+                                            unsigned long long *qsum) {
+#pragma unroll
+  for (int l = 0; l < 2; ++l) {
+    const int q = l ? qB : qA;
+    if (q < 0) continue;
+    // (s, q) with s < q is counted by the earlier query; d(q, q) = 0
+    if (job.mode == 0 && s <= q) continue;
+    const int S = l ? Cell<true>::lane1(best) : Cell<true>::lane0(best);
+    if (S > job.sat_thresh) {
+      const unsigned slot = atomicAdd(job.ovf_count, 1u);
+      if (slot < (unsigned)job.ovf_cap) job.ovf[slot] = make_int2(q, s);
+      else atomicOr(job.err, MSA_DERR_OVERFLOW);
+      continue;
+    }
+    const unsigned long long sim = center_sim(S, job.self[q], job.self[s]);
+    if (job.mode != 2) atomicAdd(&job.pairsum[s], sim);
+    if (job.mode != 1) atomicAdd(&qsum[l], sim);
+  }
+}
+
 // Work item = (query pair p, block of NG consecutive subjects, one per group).
 // three CTAs per SM for the 12-row variants (their registers fit 85 per
 // thread without spilling); two otherwise
 template <int G, int R>
 __global__ void __launch_bounds__(kCenterThreads, R <= 12 ? 3 : 2)
 k_center2(SeqSet ss, Scoring sc, CenterJob job) {
+  if (job.similar && *job.similar >= job.similar_min) return;  // k_center_near scores these
   extern __shared__ __align__(16) uint32_t smem32[];
   __shared__ int8_t sM[MSA_MAX_ALPHABET * MSA_MAX_ALPHABET];
   __shared__ long long s_item;
@@ -391,13 +415,13 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
           const uint32_t *pp = smem32 + p * G * PITCH;
           int b;
           if (np == 1)
-            b = wave_pass_pp<G, R, false, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, sout);
+            b = wave_pass_pp<G, R, false, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, Lw, sout);
           else if (p == 0)
-            b = wave_pass_pp<G, R, false, true>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, sout);
+            b = wave_pass_pp<G, R, false, true>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, Lw, sout);
           else if (p + 1 == np)
-            b = wave_pass_pp<G, R, true, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, sout);
+            b = wave_pass_pp<G, R, true, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, Lw, sout);
           else
-            b = wave_pass_pp<G, R, true, true>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, sout);
+            b = wave_pass_pp<G, R, true, true>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, false, sin, Lw, sout);
           best = Cell<true>::vmax(best, b);
           __syncwarp();
         }
@@ -406,29 +430,7 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
       for (int off = G / 2; off > 0; off >>= 1)
         best = Cell<true>::vmax(best, __shfl_xor_sync(MSA_FULL_MASK, best, off));
       if (t == 0 && valid) {
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          const int q = l ? qB : qA;
-          if (q < 0) continue;
-          // (s, q) with s < q is counted by the earlier query; d(q, q) = 0
-          if (job.mode == 0 && s <= q) continue;
-          const int S = l ? Cell<true>::lane1(best) : Cell<true>::lane0(best);
-          if (S > job.sat_thresh) {
-            const unsigned slot = atomicAdd(job.ovf_count, 1u);
-            if (slot < (unsigned)job.ovf_cap) job.ovf[slot] = make_int2(q, s);
-            else atomicOr(job.err, MSA_DERR_OVERFLOW);
-            continue;
-          }
-          const unsigned long long sim = center_sim(S, job.self[q], job.self[s]);
-          if (job.mode == 0) {
-            atomicAdd(&job.pairsum[s], sim);
-            atomicAdd(&s_qsum[0][l], sim);
-          } else if (job.mode == 1) {
-            atomicAdd(&job.pairsum[s], sim);
-          } else {
-            atomicAdd(&s_qsum[0][l], sim);
-          }
-        }
+        center_sums(job, best, qA, qB, s, s_qsum[0]);
       }
       __syncthreads();
       if (threadIdx.x == 0 && job.mode != 1) {
@@ -501,13 +503,13 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
         const bool top = kseg >= 0 && blk * R == s_start[kseg];
         int b;
         if (np == 1)
-          b = wave_pass_pp<G, R, false, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, top, sin, sout);
+          b = wave_pass_pp<G, R, false, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, top, sin, Lw, sout);
         else if (p == 0)
-          b = wave_pass_pp<G, R, false, true>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, top, sin, sout);
+          b = wave_pass_pp<G, R, false, true>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, top, sin, Lw, sout);
         else if (p + 1 == np)
-          b = wave_pass_pp<G, R, true, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, top, sin, sout);
+          b = wave_pass_pp<G, R, true, false>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, top, sin, Lw, sout);
         else
-          b = wave_pass_pp<G, R, true, true>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, top, sin, sout);
+          b = wave_pass_pp<G, R, true, true>(pp, stride, rs, Ls, Lw, t, base_lane, padc, o, sc.e, top, sin, Lw, sout);
         if (kseg >= 0) {
           atomicMax(&gbest[2 * kseg], Cell<true>::lane0(b));
           atomicMax(&gbest[2 * kseg + 1], Cell<true>::lane1(b));
@@ -550,6 +552,187 @@ k_center2(SeqSet ss, Scoring sc, CenterJob job) {
     if (job.mode != 1 && threadIdx.x < 2 * m) {
       const int k = threadIdx.x >> 1, l = threadIdx.x & 1;
       if (s_q[k][l] >= 0 && s_qsum[k][l]) atomicAdd(&job.pairsum[s_q[k][l]], s_qsum[k][l]);
+    }
+  }
+}
+
+// ------------------------------------------------------------ similar sequences
+// A path that pairs m residues scores at most smax m, and from the cell (i, j) of
+// Lq rows and Ls columns on it pairs at most min(Lq - 1 - i, Ls - 1 - j) more.  So
+// once a pair's score is known to be at least v, a pass of rows [r0, r1) needs
+// only the columns that a path of score v can reach:
+//   from the left   the first column of the row above with H + smax min(Lq - r0,
+//                   Ls - 1 - column) >= v; or, while a path of v could still begin
+//                   below that row, diagonal -(Lq - ceil(v / smax)),
+//   to the right    diagonal Ls - r0 - ceil((v - top) / smax), top the best H of
+//                   those columns (0 in the first pass): further right the rest
+//                   of the subject is too short.
+// Cells outside read as zeros and the cells inside as lower bounds of themselves,
+// exact (values, ties and codes) wherever a path of score v runs.  v is a guess:
+// smax min(Lq, Ls) less the share (of 1024) that the warp's previous pairs fell
+// short by and a fifth more, at its first item a quarter.  A score of at least v
+// proves the columns; a pair that falls short runs again with its score as v (more
+// columns find no less, so that fill is the last), and past a share of 45 % every
+// column is filled.
+constexpr int kNearFirst = 256, kNearMost = 376, kNearAll = 1024;
+
+// Widens [c0, c1) by the columns of rows [r0, r1) (c0 a multiple of 4: code words
+// are stored by fours).
+__device__ __forceinline__ void near_columns(int smax, int Lq, int Ls, int guess, int r0, int r1, int first,
+                                             int top, int &c0, int &c1) {
+  if (r0 >= Lq || Ls <= 0) return;
+  const int need = guess - top;
+  const int begin = smax * (Lq - r0) < guess ? first : r0 - (Lq - (guess + smax - 1) / smax);
+  const int diag = need > 0 ? Ls - r0 - (need + smax - 1) / smax : Ls;
+  c0 = min(c0, max(0, begin) & ~3);
+  c1 = max(c1, min(Ls, r1 + diag));
+}
+
+// The bottom row of a pass: of each int16 lane its first column and best H from
+// which the rows left and the columns left can make up the guess.
+template <int G>
+__device__ __forceinline__ void near_row(const int2 *row, int c0, int c1, int t, int Lw, int smax, int rowsA,
+                                         int rowsB, int LA, int LB, const int (&guess)[2], int (&first)[2],
+                                         int (&top)[2]) {
+  const int rows[2] = {rowsA, rowsB}, Ls[2] = {LA, LB};
+#pragma unroll
+  for (int l = 0; l < 2; ++l) { first[l] = Lw; top[l] = -1; }
+  for (int j = c0 + t; j < c1; j += G) {
+    const int h = row[j].x;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      const int hv = l ? Cell<true>::lane1(h) : Cell<true>::lane0(h);
+      const int left = min(rows[l], Ls[l] - 1 - j);
+      if (left >= 0 && hv + smax * left >= guess[l]) {
+        first[l] = min(first[l], j);
+        top[l] = max(top[l], hv);
+      }
+    }
+  }
+#pragma unroll
+  for (int off = G / 2; off > 0; off >>= 1)
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      first[l] = min(first[l], __shfl_xor_sync(MSA_FULL_MASK, first[l], off));
+      top[l] = max(top[l], __shfl_xor_sync(MSA_FULL_MASK, top[l], off));
+    }
+}
+
+// The warp's next share (a score of 15 bits and 1/1024 stay within an int).
+__device__ __forceinline__ int near_share(const int (&full)[2], int vA, int vB) {
+  int far = 0;
+  if (full[0] > 0) far = (full[0] - vA) * 1024 / full[0];
+  if (full[1] > 0) far = max(far, (full[1] - vB) * 1024 / full[1]);
+  far = __reduce_max_sync(MSA_FULL_MASK, far);
+  return far > kNearMost ? kNearAll : far + far / 5 + 8;
+}
+
+// The same items for similar sequences (streams of one pair each, passes of
+// fewer rows than the queries): a pass fills only the columns from which a path
+// of score v can still pass, v a guess that the score then proves -- the bounds
+// and the guess as at k_codes_near, each lane's with its own query's length.
+// Integer bound as k_center2, in fewer columns.  DNA sequences that differ in 4 %
+// of their residues, 100 references: 3,000 of 1,500 100.7 ms with every column,
+// 47.7 so; 1,000 39.9 -> 17.8; 3,000 of 2,400 258 -> 138.
+template <int G, int R>
+__global__ void __launch_bounds__(kCenterThreads, R <= 12 ? 3 : 2)
+k_center_near(SeqSet ss, Scoring sc, CenterJob job) {
+  if (*job.similar < job.similar_min) return;  // k_center2 has scored them
+  extern __shared__ __align__(16) uint32_t smem32[];
+  __shared__ int8_t sM[MSA_MAX_ALPHABET * MSA_MAX_ALPHABET];
+  __shared__ long long s_item;
+  __shared__ unsigned long long s_qsum[2];
+  constexpr int NT = kCenterThreads, NG = NT / G, PITCH = center_pitch(R);
+  const int K = sc.K, padc = K, o = sc.o, smax = job.smax;
+  const int stride = dround_up(job.npass * G * PITCH, 32);  // of a letter's row
+  for (int i = threadIdx.x; i < K * K; i += NT) sM[i] = sc.M[i];
+  const int g = threadIdx.x / G, t = threadIdx.x % G;
+  const int base_lane = (threadIdx.x & 31) - t;
+  int2 *scr = job.scratch + ((size_t)blockIdx.x * NG + g) * 2 * job.scratch_cols;
+  int share = kNearFirst;
+  for (;;) {
+    if (threadIdx.x == 0) s_item = (long long)atomicAdd(job.counter, 1ull);
+    __syncthreads();
+    long long item = s_item;
+    if (item >= job.n_items) break;
+    item = job.n_items - 1 - item;  // longest queries first
+    int lo = 0, hi = job.qe - job.qb - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (job.prefix[mid] <= item) lo = mid; else hi = mid - 1;
+    }
+    const int xa = 2 * job.streams[job.qb + lo].x, xb = xa + 1;
+    const int qA = job.mode == 0 ? xa : job.qlist[xa];
+    const int qB = xb < job.nq ? (job.mode == 0 ? xb : job.qlist[xb]) : -1;
+    const int Lq[2] = {ss.len[qA], qB >= 0 ? ss.len[qB] : 0};
+    const int np = (max(Lq[0], Lq[1]) + G * R - 1) / (G * R);
+    {
+      const uint8_t *ra = ss.res + ss.pstart[qA];
+      const uint8_t *rb = ss.res + ss.pstart[qB >= 0 ? qB : qA];
+      const int prow = np * G * R;
+      if (threadIdx.x < 2) s_qsum[threadIdx.x] = 0ull;
+      for (int idx = threadIdx.x; idx < (K + 1) * prow; idx += NT) {
+        const int r = idx / prow, i = idx - r * prow;
+        uint32_t a = 0, b = 0;  // padding: score -o
+        if (r < K) {
+          if (i < Lq[0]) a = (uint32_t)(sM[ra[i] * K + r] + o);
+          if (i < Lq[1]) b = (uint32_t)(sM[rb[i] * K + r] + o);
+        }
+        smem32[r * stride + (PITCH == R ? i : i + (i / R) * (PITCH - R))] = a | (b << 16);
+      }
+    }
+    __syncthreads();
+    const int s0 = (job.mode == 0 ? xa : job.sub_off) + (int)(item - job.prefix[lo]) * NG;
+    const int send = job.mode == 0 ? ss.n : job.sub_off + job.sub_n;
+    const int s = s0 + g;
+    const bool valid = s < send;
+    const int Ls = valid ? ss.len[s] : 0;
+    const uint8_t *rs = ss.res + (valid ? ss.pstart[s] : 0);
+    const int Lw = __reduce_max_sync(MSA_FULL_MASK, Ls);
+    int best = 0;
+    if (Lw > 0) {
+      int full[2], guess[2];
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        full[l] = smax * min(Lq[l], Ls);
+        guess[l] = share < kNearAll ? full[l] - full[l] * share / 1024 : 0;
+      }
+      for (;;) {
+        int first[2] = {0, 0}, top[2] = {0, 0}, above = 0;
+        best = 0;
+        for (int p = 0; p < np; ++p) {
+          const int2 *sin = scr + (size_t)((p + 1) & 1) * job.scratch_cols;
+          int2 *sout = scr + (size_t)(p & 1) * job.scratch_cols;
+          const int r0 = p * G * R, r1 = r0 + G * R;
+          int c0 = Lw, c1 = 0;
+#pragma unroll
+          for (int l = 0; l < 2; ++l) near_columns(smax, Lq[l], Ls, guess[l], r0, r1, first[l], top[l], c0, c1);
+          c0 = __reduce_min_sync(MSA_FULL_MASK, c0);
+          c1 = __reduce_max_sync(MSA_FULL_MASK, c1);
+          if (c1 > c0)
+            best = Cell<true>::vmax(
+                best, wave_pass_pp<G, R, true, true>(smem32 + p * G * PITCH, stride, rs + c0, Ls - c0, c1 - c0,
+                                                     t, base_lane, padc, o, sc.e, false, sin + c0, above - c0,
+                                                     sout + c0));
+          above = c1;
+          __syncwarp();
+          if (p + 1 < np) near_row<G>(sout, c0, c1, t, Lw, smax, Lq[0] - r1, Lq[1] - r1, Ls, Ls, guess, first, top);
+        }
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1)
+          best = Cell<true>::vmax(best, __shfl_xor_sync(MSA_FULL_MASK, best, off));
+        const int v[2] = {Cell<true>::lane0(best), Cell<true>::lane1(best)};
+        if (!__any_sync(MSA_FULL_MASK, v[0] < guess[0] || v[1] < guess[1])) break;
+        guess[0] = min(guess[0], v[0]);
+        guess[1] = min(guess[1], v[1]);
+      }
+      share = near_share(full, Cell<true>::lane0(best), Cell<true>::lane1(best));
+    }
+    if (t == 0 && valid) center_sums(job, best, qA, qB, s, s_qsum);
+    __syncthreads();
+    if (threadIdx.x == 0 && job.mode != 1) {
+      if (s_qsum[0]) atomicAdd(&job.pairsum[qA], s_qsum[0]);
+      if (qB >= 0 && s_qsum[1]) atomicAdd(&job.pairsum[qB], s_qsum[1]);
     }
   }
 }
@@ -949,31 +1132,15 @@ __global__ void __launch_bounds__(NT, 1) k_codes2(SeqSet ss, Scoring sc, CodesJo
   }
 }
 
-// ------------------------------------------------------------ similar subjects
-// A path that pairs m residues scores at most smax m, and from the cell (i, j)
-// on it pairs at most min(Lc - 1 - i, Ls - 1 - j) more.  So once a subject's best
-// score is known to be at least v, a pass of rows [r0, r1) needs only the columns
-// that a path of score v can reach:
-//   from the left   the first column of the row above with H + smax min(Lc - r0,
-//                   Ls - 1 - column) >= v; or, while a path of v could still begin
-//                   below that row, diagonal -(Lc - ceil(v / smax)),
-//   to the right    diagonal Ls - r0 - ceil((v - top) / smax), top the best H of
-//                   those columns (0 in the first pass): further right the rest
-//                   of the subject is too short.
-// Cells outside read as zeros and the cells inside as lower bounds of themselves,
-// exact (values, ties and codes) wherever a path of score v runs.  v is a guess:
-// smax min(Lc, Ls) less the share that the warp's previous subjects fell short
-// by and a fifth more, at its first item a quarter.  A score of at least v proves
-// the columns; a subject that falls short runs again with its score as v, and
-// past a share of 45 % every column is filled.  Integer bound as k_codes2, in
-// fewer columns.  Alignment of DNA sequences that differ in 4 % of their residues:
-// 20,000 of 1,500 21.7 ms with every column, 16.1 with the diagonals alone, 11.0
-// so; 60,000 63.1 -> 28.6 ms, 10,000 of 2,900 48.7 -> 22.6 ms.
+// Similar subjects: k_codes2's items in the columns that a best path can reach
+// (bounds and guess: near_columns).  Integer bound as k_codes2, in fewer columns.
+// Alignment of DNA sequences that differ in 4 % of their residues: 20,000 of 1,500
+// 21.7 ms with every column, 16.1 with the diagonals alone, 11.0 so; 60,000 63.1 ->
+// 28.6 ms, 10,000 of 2,900 48.7 -> 22.6 ms.
 template <int G>
 __global__ void __launch_bounds__(256, 1) k_codes_near(SeqSet ss, Scoring sc, CodesJob job) {
   if (*job.similar < job.similar_min) return;  // k_codes2 has filled every column
   constexpr int R = kCodesR, NT = 256, NG = NT / G, GPW = 32 / G;
-  constexpr int kFirstShare = 256, kMaxShare = 376, kEvery = 1024;  // of 1024
   extern __shared__ __align__(16) int8_t smem[];
   __shared__ int8_t sM[MSA_MAX_ALPHABET * MSA_MAX_ALPHABET];
   const int K = sc.K, padc = K, smax = job.smax;
@@ -995,7 +1162,7 @@ __global__ void __launch_bounds__(256, 1) k_codes_near(SeqSet ss, Scoring sc, Co
   const int nblk = (Lc + R - 1) / R;
   int2 *scr = job.scratch + ((size_t)blockIdx.x * NG + g) * 2 * job.scratch_cols;
   const int nsub = job.se - job.sb, nitem = (nsub + 1) / 2;
-  int share = kFirstShare;
+  int share = kNearFirst;
   for (;;) {
     int x0 = 0;
     if (lane == 0) x0 = (int)atomicAdd(job.counter, (unsigned long long)GPW);
@@ -1014,7 +1181,7 @@ __global__ void __launch_bounds__(256, 1) k_codes_near(SeqSet ss, Scoring sc, Co
       rs[s] = has[s] ? ss.res + ss.pstart[k[s]] : ss.res;
       codes[s] = has[s] ? reinterpret_cast<uint2 *>(job.codes + job.code_off[k[s] - job.sb]) : nullptr;
       full[s] = smax * min(Lc, Ls[s]);
-      guess[s] = share < kEvery ? full[s] - full[s] * share / 1024 : 0;
+      guess[s] = share < kNearAll ? full[s] - full[s] * share / 1024 : 0;
     }
     const int Lw = __reduce_max_sync(MSA_FULL_MASK, max(Ls[0], Ls[1]));
     int bv[2], bi[2], bj[2];
@@ -1029,14 +1196,7 @@ __global__ void __launch_bounds__(256, 1) k_codes_near(SeqSet ss, Scoring sc, Co
         const int blk = p * G + t, r0 = p * G * R, r1 = min(Lc, r0 + G * R);
         int c0 = Lw, c1 = 0;
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          if (!has[s]) continue;
-          const int need = guess[s] - top[s];
-          const int begin = smax * (Lc - r0) < guess[s] ? first[s] : r0 - (Lc - (guess[s] + smax - 1) / smax);
-          const int diag = need > 0 ? Ls[s] - r0 - (need + smax - 1) / smax : Ls[s];
-          c0 = min(c0, max(0, begin) & ~3);  // code words are stored by fours
-          c1 = max(c1, min(Ls[s], r1 + diag));
-        }
+        for (int s = 0; s < 2; ++s) near_columns(smax, Lc, Ls[s], guess[s], r0, r1, first[s], top[s], c0, c1);
         c0 = __reduce_min_sync(MSA_FULL_MASK, c0);
         c1 = __reduce_max_sync(MSA_FULL_MASK, c1);
         if (c1 > c0)
@@ -1048,28 +1208,7 @@ __global__ void __launch_bounds__(256, 1) k_codes_near(SeqSet ss, Scoring sc, Co
                                 HalfRows{}, c0, bv, bi, bj);
         above = c1;
         __syncwarp();
-        if (!sout) continue;
-#pragma unroll
-        for (int s = 0; s < 2; ++s) { first[s] = Lw; top[s] = -1; }
-        for (int j = c0 + t; j < c1; j += G) {
-          const int h = sout[j].x;
-#pragma unroll
-          for (int s = 0; s < 2; ++s) {
-            const int hv = s ? Cell<true>::lane1(h) : Cell<true>::lane0(h);
-            const int left = min(Lc - r1, Ls[s] - 1 - j);
-            if (left >= 0 && hv + smax * left >= guess[s]) {
-              first[s] = min(first[s], j);
-              top[s] = max(top[s], hv);
-            }
-          }
-        }
-#pragma unroll
-        for (int off = G / 2; off > 0; off >>= 1)
-#pragma unroll
-          for (int s = 0; s < 2; ++s) {
-            first[s] = min(first[s], __shfl_xor_sync(MSA_FULL_MASK, first[s], off));
-            top[s] = max(top[s], __shfl_xor_sync(MSA_FULL_MASK, top[s], off));
-          }
+        if (sout) near_row<G>(sout, c0, c1, t, Lw, smax, Lc - r1, Lc - r1, Ls[0], Ls[1], guess, first, top);
       }
 #pragma unroll
       for (int s = 0; s < 2; ++s)
@@ -1086,29 +1225,27 @@ __global__ void __launch_bounds__(256, 1) k_codes_near(SeqSet ss, Scoring sc, Co
 #pragma unroll
       for (int s = 0; s < 2; ++s) guess[s] = min(guess[s], bv[s]);
     }
-    // the next guess (a score of 15 bits and 1/1024 stay within an int)
-    int far = 0;
+    share = near_share(full, bv[0], bv[1]);
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      if (full[s] > 0) far = max(far, (full[s] - bv[s]) * 1024 / full[s]);
+    for (int s = 0; s < 2; ++s)
       if (t == 0 && has[s]) job.best[k[s] - job.sb] = best_key(bv[s], bi[s], bj[s]);
-    }
-    far = __reduce_max_sync(MSA_FULL_MASK, far);
-    share = far > kMaxShare ? kEvery : far + far / 5 + 8;
   }
 }
 
-// Whether the subjects resemble the center: of kSimilarSample subjects spread
-// over the set, how many share at least 12 of 32 words of 12 residues with it
+// Whether the subjects resemble the queries: of kSimilarSample subjects spread
+// over the set, how many share at least 12 of 32 words of 12 residues with a query
 // (residues that differ in 8 % or more share fewer).  A CTA per subject, a word
-// per lane, a quarter of the center per warp: about 3 us.
+// per lane, a quarter of the query per warp: about 3 us.
 constexpr int kWordLen = 12, kWordBits = 5;
 
-__global__ void __launch_bounds__(128) k_similar(SeqSet ss, int center, unsigned *similar) {
+__global__ void __launch_bounds__(128) k_similar(SeqSet ss, int nsub, const int32_t *qlist, int q0, int nq, unsigned *similar) {
   __shared__ unsigned s_found[4];
-  const int k = (int)((long long)blockIdx.x * ss.n / gridDim.x), Ls = ss.len[k], Lc = ss.len[center];
-  if (Ls < 4 * kWordLen) return;
-  const uint8_t *rs = ss.res + ss.pstart[k], *rc = ss.res + ss.pstart[center];
+  // (the queries in another order than the subjects)
+  const int k = (int)((long long)blockIdx.x * nsub / gridDim.x);
+  const int x = (int)((long long)((blockIdx.x * 37) % gridDim.x) * nq / gridDim.x);
+  const int q = qlist ? qlist[x] : q0 + x, Ls = ss.len[k], Lc = ss.len[q];
+  if (Ls < 4 * kWordLen || Lc < 4 * kWordLen) return;
+  const uint8_t *rs = ss.res + ss.pstart[k], *rc = ss.res + ss.pstart[q];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned long long mask = (1ull << (kWordLen * kWordBits)) - 1;
   unsigned long long mine = 0, key = 0;
@@ -1190,6 +1327,24 @@ static center_fn center_kernel(int variant) {
   }
 }
 
+// The paired variants' bounded form.
+static center_fn center_near_kernel(int variant) {
+  switch (variant) {
+    case 0: return k_center_near<8, 12>;
+    case 1: return k_center_near<8, 20>;
+    case 2: return k_center_near<8, 28>;
+    case 3: return k_center_near<16, 12>;
+    case 4: return k_center_near<16, 20>;
+    case 5: return k_center_near<16, 28>;
+    case 6: return k_center_near<32, 12>;
+    case 7: return k_center_near<32, 20>;
+    case 8: return k_center_near<32, 28>;
+    case 14: return k_center_near<16, 16>;
+    case 15: return k_center_near<16, 24>;
+    default: return nullptr;
+  }
+}
+
 static int sm_count() {
   int dev = 0, n = 0;
   cudaGetDevice(&dev);
@@ -1213,20 +1368,20 @@ int center_grid(int variant, int smem) {
 
 // (static shared memory counts against the 48 KB default too, so the limit
 // is raised whatever the dynamic size)
-cudaError_t center_allow_smem(int variant, int smem) {
-  center_fn fn = center_kernel(variant);
+cudaError_t center_allow_smem(int variant, int smem, bool near) {
+  center_fn fn = near ? center_near_kernel(variant) : center_kernel(variant);
   if (!fn) return cudaErrorInvalidValue;
   return cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 cudaError_t launch_center(int variant, const SeqSet &ss, const Scoring &sc, const CenterJob &job,
-                          int grid, cudaStream_t st, bool set_smem) {
-  center_fn fn = center_kernel(variant);
+                          int grid, cudaStream_t st, bool set_smem, bool near) {
+  center_fn fn = near ? center_near_kernel(variant) : center_kernel(variant);
   if (!fn) return cudaErrorInvalidValue;
   const CenterVariant &v = kCenterVariants[variant];
   const int smem = center_smem_bytes(variant, sc.K, job.npass * v.G * v.R);
   if (set_smem) {
-    const cudaError_t e = center_allow_smem(variant, smem);
+    const cudaError_t e = center_allow_smem(variant, smem, near);
     if (e != cudaSuccess) return e;
   }
   fn<<<grid, kCenterThreads, smem, st>>>(ss, sc, job);
@@ -1351,8 +1506,9 @@ cudaError_t launch_codes_near(int G, const SeqSet &ss, const Scoring &sc, const 
   return cudaGetLastError();
 }
 
-cudaError_t launch_similar(const SeqSet &ss, int center, unsigned *similar, cudaStream_t st) {
-  k_similar<<<kSimilarSample, 128, 0, st>>>(ss, center, similar);
+cudaError_t launch_similar(const SeqSet &ss, int nsub, const int32_t *qlist, int q0, int nq, unsigned *similar,
+                           cudaStream_t st) {
+  k_similar<<<kSimilarSample, 128, 0, st>>>(ss, nsub, qlist, q0, nq, similar);
   return cudaGetLastError();
 }
 

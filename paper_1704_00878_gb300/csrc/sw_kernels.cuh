@@ -36,6 +36,11 @@ struct CenterJob {
   // paired classes: the unit is a stream of consecutive query pairs stacked
   // in one row range, streams[u] = {first pair, pair count <= kMaxSeg}
   const int2 *streams;
+  // set: the full kernel does nothing where *similar >= similar_min, the bounded
+  // one (which needs smax, the matrix's largest score) where not
+  const unsigned *similar = nullptr;
+  unsigned similar_min = 0;
+  int smax = 0;
 };
 
 // Query pairs one stream of the paired center kernel may stack.
@@ -81,10 +86,11 @@ int center_smem_bytes(int variant, int K, int rows_alloc);
 int center_profile_bytes(int variant, int K, int rows_alloc);
 // set_smem = false: the caller has already raised the kernel's dynamic
 // shared-memory limit with center_allow_smem (required while a stream is
-// being captured into a graph).
+// being captured into a graph).  near: the bounded form (paired variants, units
+// of one pair each).
 cudaError_t launch_center(int variant, const SeqSet &ss, const Scoring &sc, const CenterJob &job,
-                          int grid, cudaStream_t st, bool set_smem = true);
-cudaError_t center_allow_smem(int variant, int smem);
+                          int grid, cudaStream_t st, bool set_smem = true, bool near = false);
+cudaError_t center_allow_smem(int variant, int smem, bool near = false);
 int center_grid(int variant, int smem);
 
 // packed: two pairs per group in int16 lanes (G 8, 16 or 32; the caller checks
@@ -110,7 +116,8 @@ int codes_grid(int G, bool packed, int smem, int threads = 256);
 int codes_threads(bool packed, int threads = 256);  // threads per CTA of the codes kernels
 // The packed fill of similar subjects without the columns that no best path
 // reaches (G 8, 16 or 32), and the vote that decides between the two: the number
-// of kSimilarSample subjects that resemble the center, added to *similar.
+// of kSimilarSample of the subjects [0, nsub) that resemble one of the nq queries
+// (qlist, or q0 on), added to *similar.
 // near_group: its lanes per subject where the full fill has G -- narrower groups
 // leave out more columns (a pass has fewer rows), and pay once every warp has
 // four items: with 8 / 16 / 32 lanes 60,000 of 1,500 residues 28.8 / 30.5 / 36.3
@@ -121,7 +128,8 @@ int near_grid(int G, int smem);
 cudaError_t near_allow_smem(int G, int smem);
 cudaError_t launch_codes_near(int G, const SeqSet &ss, const Scoring &sc, const CodesJob &job, int grid,
                               cudaStream_t st);
-cudaError_t launch_similar(const SeqSet &ss, int center, unsigned *similar, cudaStream_t st);
+cudaError_t launch_similar(const SeqSet &ss, int nsub, const int32_t *qlist, int q0, int nq, unsigned *similar,
+                           cudaStream_t st);
 int codes_group(int Lc, bool packed, int K, int64_t n, double mean_len, int max_len);
 constexpr int kCodesR = 16;
 // lanes per subject the alignment kernels come in: 1, 2, 4, 8, 16, 32

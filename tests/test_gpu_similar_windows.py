@@ -89,3 +89,39 @@ def test_several_subjects_per_warp_match_full_columns(odd_every):
             got.append(b.msa_alignment_info(h))
     for x, y in zip(*got):
         assert (x == y).all()
+
+
+@pytest.mark.parametrize("n, nref, length", [(1000, 30, 900), (2500, 25, 600), (260, 0, 900)])
+@pytest.mark.parametrize("odd_every", [0, 9, 2])
+def test_center_of_similar_sequences_matches_full_columns(n, nref, length, odd_every):
+    """Row sums of the bounded center kernel (every pair, and a sample of
+    references) against the int32 kernels, with unrelated, repeated and short
+    sequences among the similar ones; an odd number of references leaves one
+    lane of the last pair empty."""
+    b = binding()
+    rng = np.random.default_rng(n + odd_every)
+    alph, M = dna_matrix()
+    pool = np.frombuffer(b"ACGT", np.uint8)
+    center = rng.choice(pool, size=length)
+    seqs = []
+    for x in range(n):
+        if odd_every and x % odd_every == 0:
+            seqs.append((rng.choice(pool, size=int(rng.integers(50, length))), np.tile(center[:90], 7),
+                         center[:int(rng.integers(100, length))])[x % 3])
+            continue
+        s = mutate(rng, center, (0.0, 0.02, 0.06)[x % 3], pool)
+        a, k = int(rng.integers(0, length // 8)), int(rng.integers(length // 8, length))
+        seqs.append(np.concatenate([s[a:k], s[k + int(rng.integers(0, 40)):]]))
+    letters, offsets = pack_sequences(seqs)
+    refs = np.sort(rng.choice(n, size=max(nref - 1 + n % 2, 1), replace=False))
+    got = []
+    for precision in (b.MSA_AUTO, b.MSA_INT32):
+        with make_ctx(alph, M, 5, 2, precision=precision) as h:
+            b.msa_load(h, letters, offsets)
+            if nref:
+                c = b.msa_select_center(h, b.MSA_CENTER_EXACT_SAMPLED, refs=refs)
+            else:
+                c = b.msa_select_center(h, b.MSA_CENTER_EXACT)
+            got.append((c, b.msa_center_rowsums(h)))
+    assert got[0][0] == got[1][0]
+    assert (got[0][1] == got[1][1]).all()
