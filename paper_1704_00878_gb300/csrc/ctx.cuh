@@ -63,7 +63,7 @@ struct msa_ctx {
   // center selection
   DevBuf pairsum, self, rowsum, prefix, qlist, ovf, ovf_scores, ovf_dst, part_val, part_idx,
       pairs, pair_dst, pair_out, counters, streams;
-  cudaStream_t cap_lanes[msa_detail::kCenterLanes] = {};  // private streams the center graph is captured on
+  cudaStream_t cap_lanes[2] = {};  // private streams: the graphs are captured on the first
   cudaEvent_t cap_fork = nullptr, cap_join = nullptr;
   cudaGraphExec_t center_exec = nullptr;  // the last center graph and what it bakes in
   std::vector<int64_t> center_key;

@@ -608,21 +608,40 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
         e = launch_similar(ss, sub_n, mode == 0 ? nullptr : P<int32_t>(ctx->qlist), 0, nq, similar,
                            ctx->cap_lanes[0]);
     }
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->cap_fork, ctx->cap_lanes[0]);
-    const int lanes = (int)std::min<size_t>(plans.size(), kCenterLanes);
-    for (int k = 1; k < lanes && e == cudaSuccess; ++k)
-      e = cudaStreamWaitEvent(ctx->cap_lanes[k], ctx->cap_fork, 0);
+    // a branch per lane: one stream captures them all, its dependencies set to
+    // the lane's last node before each launch (a stream per lane cost 40 us each
+    // to create)
+    std::vector<cudaGraphNode_t> tail[kCenterLanes];
+    auto last_nodes = [&](std::vector<cudaGraphNode_t> &nodes) -> cudaError_t {
+      cudaStreamCaptureStatus status;
+      const cudaGraphNode_t *deps = nullptr;
+      size_t count = 0;
+      const cudaError_t r = cudaStreamGetCaptureInfo(ctx->cap_lanes[0], &status, nullptr, nullptr, &deps, nullptr, &count);
+      if (r == cudaSuccess) nodes.assign(deps, deps + count);
+      return r;
+    };
+    auto go_on_from = [&](std::vector<cudaGraphNode_t> &nodes) {
+      return cudaStreamUpdateCaptureDependencies(ctx->cap_lanes[0], nodes.data(), nullptr, nodes.size(),
+                                                 cudaStreamSetCaptureDependencies);
+    };
+    if (e == cudaSuccess) e = last_nodes(tail[0]);
+    for (int k = 1; k < kCenterLanes; ++k) tail[k] = tail[0];
     int failed = -1;
     for (size_t k = 0; k < plans.size() && e == cudaSuccess; ++k) {
       const size_t c = plans.size() - 1 - k;
-      e = launch_center(plans[c].cc.variant, ss, sc, jobs[c], plans[c].grid,
-                        ctx->cap_lanes[lane_of(c)], false, plans[c].role == ClassPlan::kNear);
+      std::vector<cudaGraphNode_t> &lane = tail[lane_of(c)];
+      if ((e = go_on_from(lane)) != cudaSuccess) break;
+      e = launch_center(plans[c].cc.variant, ss, sc, jobs[c], plans[c].grid, ctx->cap_lanes[0], false,
+                        plans[c].role == ClassPlan::kNear);
       if (e != cudaSuccess) failed = (int)c;
+      else e = last_nodes(lane);
     }
-    for (int k = 1; k < lanes; ++k) {
-      const cudaError_t e2 = cudaEventRecord(ctx->cap_join, ctx->cap_lanes[k]);
-      const cudaError_t e3 = cudaStreamWaitEvent(ctx->cap_lanes[0], ctx->cap_join, 0);
-      if (e == cudaSuccess) e = e2 != cudaSuccess ? e2 : e3;
+    if (e == cudaSuccess) {
+      std::vector<cudaGraphNode_t> all;
+      for (const auto &lane : tail) all.insert(all.end(), lane.begin(), lane.end());
+      std::sort(all.begin(), all.end());
+      all.erase(std::unique(all.begin(), all.end()), all.end());
+      e = go_on_from(all);
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t e_end = cudaStreamEndCapture(ctx->cap_lanes[0], &graph);
