@@ -73,3 +73,33 @@ def test_anchored_path_at_its_longest_sequences():
         with pytest.raises(b.MSAError) as ei:
             b.msa_align_anchored(h, 0, 8)
         assert ei.value.code == b.MSA_ERANGE
+
+
+ROWS_OF_6120 = """
+import numpy as np
+from seqgen import dna_matrix, pack_sequences
+from tests._gpu import binding, make_ctx
+b = binding()
+alph, M = dna_matrix()
+s = np.random.default_rng(1).choice(np.frombuffer(b"ACGT", np.uint8), size=6120)
+letters, offsets = pack_sequences([s, s, s[:5000]])
+with make_ctx(alph, M, 5, 2) as h:
+    b.msa_load(h, letters, offsets)
+    b.msa_align_to_center(h, 0)
+    rows, W = b.msa_merge_gaps(h)
+rows = np.asarray(rows).reshape(3, W)
+assert W == 6120 and (rows[0] == s).all() and (rows[1] == s).all()
+assert (rows[2] == np.concatenate([s[:5000], np.full(1120, ord("-"), np.uint8)])).all()
+"""
+
+
+def test_rows_whose_staging_fills_the_default_shared_memory():
+    """Eight rows of 6,113 to 6,128 columns take exactly the 48 KB that a kernel
+    gets by default, static shared memory not counted.  (In a process of its own:
+    wider rows raise the limit for good.)"""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", ROWS_OF_6120], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
