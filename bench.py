@@ -54,9 +54,10 @@ CODES_BYTES_PER_CELL = 0.5   # 4-bit traceback code per cell written to HBM
 # traffic grows with the cells, so a launch's traffic is this times its cells
 CODES_TRAFFIC_PER_CELL = (10.6e6 + 528.5e6) / 1.006925e9
 ALIGN_WORKLOAD, ALIGN_N = "short_peptides_1m", 200_000
-# distance kernel of the tree: 9 integer instructions per 32-bit word of both
-# rows (4 columns: xor, nonzero test, residue mask, two counter updates)
-TREE_PEAK_TCPS = 152 * 128 * 2.07e9 / (9 / 4) / 1e12
+# distance kernel of the tree: about 20 integer lane operations per 32 columns of
+# a row pair (one three-input operation per bit plane, two masks, the share of the
+# carry-save adds and counts)
+TREE_PEAK_TCPS = 152 * 128 * 2.07e9 / (20 / 32) / 1e12
 # the library's center kernel variants, in msa_autotune's column order:
 # (two queries per int16x2 register?, lanes per group, query rows per lane, packed)
 CENTER_VARIANTS = [(1, 8, 12, 1), (1, 8, 20, 1), (1, 8, 28, 1), (1, 16, 12, 1), (1, 16, 20, 1),
@@ -438,7 +439,8 @@ def tree_record(b, h, n, W, stream, peak_gbs, cpu_n=600):
                                    "peak": TREE_PEAK_TCPS, "unit": "T column pairs/s",
                                    "frac": col_pairs / (dist_ms * 1e-3) / 1e12 / TREE_PEAK_TCPS,
                                    "peak_source": "152 SMs x 128 integer lanes/clk x 2.07 GHz / "
-                                                  "9 instructions per 4 column pairs"},
+                                                  "20 operations per 32 column pairs"},
+            # what scanning the whole matrix at every join would read, over the time
             "nj_matrix_gbs": nj_bytes / (nj_ms * 1e-3) / 1e9, "hbm_peak_gbs": peak_gbs,
             "cpu_oracle_nj": {"rows": int(sub.shape[0]), "seconds": cpu_s,
                               "kind": "oracle", "cores": 1}}

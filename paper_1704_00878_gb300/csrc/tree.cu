@@ -8,8 +8,8 @@
 //
 // Neighbour joining: the matrix stays on the device (int32 -- every entry and
 // joined distance within 2^30, else ERANGE -- positions in ascending slot
-// order); one cooperative launch runs the joins until half of the positions
-// are left (k_nj_joins), then the matrix is packed to the active ones; the
+// order); one launch of a thread-block cluster runs the joins until half of the
+// positions are left (k_nj_joins), then the matrix is packed to the active ones; the
 // last few hundred positions run in one CTA.
 #include <algorithm>
 #include <climits>
