@@ -902,6 +902,8 @@ def run_ours(args):
                                       "cells (0.28 MB for one 1.57 ms launch on 2,000 "
                                       "proteins, profiles/k_center2_batched_uneven_10k.md)",
                       "peak_source": "152 SMs x 64 DPX lanes/clk x 2.07 GHz / 3 DPX ops per cell",
+                      "cells": "of whole matrices; similar sequences leave out columns that no "
+                               "best path reaches, which can put the rate past the peak",
                       "peak_measured": rate / OPS_PER_CELL / 1e9,
                       "dpx_ops_per_clk_sm_measured": per_clk}
                      if center_cells else
