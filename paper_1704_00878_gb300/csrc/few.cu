@@ -28,18 +28,14 @@
 
 #include "dp_pass.cuh"
 #include "few.cuh"
+#include "few_schedule.cuh"
 
 namespace {
 
 constexpr int kR = kFewRows;               // center rows per lane
 constexpr int kStrip = 32 * kR;            // rows of a warp's strip
-constexpr int kStep = 16;                  // steps between CTA barriers
-constexpr int kLag = 48;                   // steps a strip runs behind the one above: 31 + 16, rounded up
-constexpr int kRing = 64;                  // columns of the row between two strips
+constexpr int kStep = kFewStep, kLag = kFewLag, kRing = kFewRing;
 constexpr int kTileCols = 128, kTileSlots = kTileCols + 8;  // traceback window: columns, 16-byte aligned slots
-
-static_assert(kLag % kStep == 0 && kLag >= 31 + kStep, "a column must be complete a barrier before it is read");
-static_assert(kRing >= kLag - 31 + 2 * kStep, "ring");
 
 // a lane's state while its warp sweeps a strip
 struct FewLane {
@@ -88,17 +84,17 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_align_few(SeqSet ss, Scoring
     const uint8_t *rs = ss.res + ss.pstart[kx];
     for (int i = tid; i < L; i += NT) sres[i] = rs[i];
     const int row_slots = few_row_slots(L);
-    const int steps = (L + 31 + kStep - 1) / kStep * kStep;
-    const int period = max(steps, W * kLag);               // steps between a warp's strips
+    const int steps = few_steps(L), period = few_period(steps, W);
     const int rounds = (nstrip + W - 1) / W;
     const int total = (rounds - 1) * period + ((nstrip - 1) % W) * kLag + steps;
     __syncthreads();
     FewLane s;
     unsigned long long key = 0ull;
     for (int g = 0; g < total; g += kStep) {
-      const int rel = g - w * kLag;
-      const int q = rel >= 0 ? rel / period : -1, k0 = rel - q * period, strip = q * W + w;
-      if (q >= 0 && k0 < steps && strip < nstrip) {
+      int q = 0, k0 = 0;
+      const bool on = few_turn(g, w, period, q, k0);
+      const int strip = q * W + w;
+      if (on && k0 < steps && strip < nstrip) {
         if (k0 == 0) {
 #pragma unroll
           for (int r = 0; r < kR; ++r) { s.H[r] = 0; s.E[r] = 0; s.rb[r] = 0; s.rj[r] = 0; s.be[r] = 0; }
@@ -334,7 +330,7 @@ cudaError_t launch_align_few(const SeqSet &ss, const Scoring &sc, const FewJob &
 double few_cost(int Lc, int n, double mean_len, int grid, int sms) {
   const int W = few_warps(Lc), nstrip = (Lc + kStrip - 1) / kStrip, rounds = (nstrip + W - 1) / W;
   const double steps = mean_len + 31 + kStep / 2;
-  const double total = (rounds - 1) * std::max(steps, (double)W * kLag) + ((nstrip - 1) % W) * kLag + steps;
+  const double total = (rounds - 1) * std::max(steps + kStep, (double)W * kLag) + ((nstrip - 1) % W) * kLag + steps;
   const int ctas = std::max(1, std::min(n, grid));
   const double step = std::max(0.14, 0.088 * ctas * W / (4.0 * std::max(sms, 1)));
   const double walk = 4.0 + 0.02 * std::min((double)Lc, mean_len);

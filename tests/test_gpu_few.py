@@ -70,3 +70,18 @@ def test_few_subjects_long_gaps_ties_and_no_score(o, e):
     seqs.append(np.full(50, ord("T"), np.uint8))
     letters, offsets = pack_sequences(seqs)
     check(letters, offsets, alph, M, o, e, 0)
+
+
+@pytest.mark.parametrize("lc", [2305, 4200])
+def test_few_subjects_at_the_ring_s_wrap(lc):
+    """Centers of several rounds of strips against subjects of 64 q + 1
+    residues: the last column of a round and the first of the next share a
+    ring slot."""
+    rng = np.random.default_rng(lc)
+    alph, M = blosum62()
+    pool = np.frombuffer(b"ARNDCQEGHILKMFPSTWYV", np.uint8)
+    center = rng.choice(pool, size=lc)
+    seqs = [center] + [center[a:a + L] for L in (769, 833, 1025) for a in (0, 500, lc - L)]
+    seqs += [rng.choice(pool, size=L) for L in (769, 833, 1025)]
+    letters, offsets = pack_sequences(seqs)
+    check(letters, offsets, alph, M, 11, 1, 0)
