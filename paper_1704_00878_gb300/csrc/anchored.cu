@@ -919,7 +919,7 @@ extern "C" int msa_align_anchored(msa_ctx *ctx, int64_t center, int32_t k, int32
     job.counter = ctx->dcounter;
     auto fn = bits * k <= 32 ? k_anchored<uint32_t> : k_anchored<unsigned long long>;
     if (smem + kAnchStatic > 48 * 1024)
-      CK(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      CK(allow_smem((const void *)fn));
     int per_sm = 0, sms = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * warps, smem));
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->dev);

@@ -134,3 +134,22 @@ __host__ __device__ __forceinline__ size_t code_word(int i0, int j0, int L, int 
 
 static inline int round_up_int(int x, int m) { return (x + m - 1) / m * m; }
 static inline int64_t round_up_i64(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
+
+// Raises the dynamic shared memory that kernel fn may be launched with to all
+// that the device leaves beside its static part (*most, where given).  The
+// limit belongs to the kernel in the process and not to a context: set to one
+// call's size, another thread's smaller call could lower it before the first
+// one has launched.
+static inline cudaError_t allow_smem(const void *fn, int *most = nullptr) {
+  int dev = 0, all = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
+  if (e != cudaSuccess) return e;
+  all -= (int)a.sharedSizeBytes;
+  if (most) *most = all;
+  return a.maxDynamicSharedSizeBytes == all
+             ? cudaSuccess
+             : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, all);
+}

@@ -303,13 +303,14 @@ size_t few_slot_codes(int Lc, int maxlen) { return (size_t)((Lc + kR - 1) / kR) 
 
 int few_grid(int K, int Lc, int maxlen, int n) {
   const int smem = few_smem(K, Lc, maxlen);
-  int dev = 0, sms = 0, per_sm = 0;
+  int dev = 0, sms = 0, per_sm = 0, most = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaFuncSetAttribute((const void *)k_align_few, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+  if (allow_smem((const void *)k_align_few, &most) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
+  if (smem > most) return 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_align_few, 32 * few_warps(Lc), smem);
   return (int)std::min<int64_t>(n, (int64_t)per_sm * std::max(sms, 1));
 }

@@ -194,7 +194,7 @@ cudaError_t light_allow_smem(int G, int mode, int smem) {
   light_fn fn = light_kernel(G, mode);
   if (!fn) return cudaErrorInvalidValue;
   if (smem <= 40 * 1024) return cudaSuccess;  // static shared memory counts too
-  return cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return allow_smem((const void *)fn);
 }
 
 int light_grid(int G, int mode, int smem) {

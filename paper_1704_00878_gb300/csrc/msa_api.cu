@@ -546,17 +546,10 @@ int launch_class(msa_ctx *ctx, int mode, int nq_list, const CenterClass &cc,
 int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, int sub_off,
                  int sub_n, const SeqSet &ss, const int32_t *self, int nq) {
   const Scoring sc = scoring(ctx);
-  std::vector<int> top(kNumCenterVariants, 0);
-  std::vector<int> top_near(kNumCenterVariants, 0);
   int num_near = 0;
   for (const ClassPlan &pl : plans) {
-    int &most = (pl.role == ClassPlan::kNear ? top_near : top)[pl.cc.variant];
-    most = std::max(most, pl.smem);
+    CK(center_allow_smem(pl.cc.variant, pl.role == ClassPlan::kNear));
     if (pl.role == ClassPlan::kNear) ++num_near;
-  }
-  for (int v = 0; v < kNumCenterVariants; ++v) {
-    if (top[v] > 0) CK(center_allow_smem(v, top[v]));
-    if (top_near[v] > 0) CK(center_allow_smem(v, top_near[v], true));
   }
   unsigned *similar = ctx->derr + 2;
   unsigned long long *cnt = P<unsigned long long>(ctx->counters);

@@ -529,7 +529,7 @@ cudaError_t launch_rows(const uint8_t *res, const int64_t *pstart, const int32_t
     const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(8, (96 * 1024) / rowbytes));
     const int smem = warps * (int)rowbytes;
     if (smem > 40 * 1024)  // static shared memory counts too
-      cudaFuncSetAttribute((const void *)k_rows_staged, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      allow_smem((const void *)k_rows_staged);
     const int blocks = blocks_for((int64_t)n * 32, warps * 32, 8192);
     k_rows_staged<<<blocks, warps * 32, smem, st>>>(res, pstart, inv, ins, occ, off, n, Lc, W,
                                                     (int)rowbytes, letters, out);

@@ -1353,7 +1353,7 @@ static int sm_count() {
 }
 
 static int occupancy_grid(const void *fn, int threads, int smem) {
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  allow_smem(fn);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
   if (per_sm < 1) per_sm = 1;
@@ -1368,10 +1368,10 @@ int center_grid(int variant, int smem) {
 
 // (static shared memory counts against the 48 KB default too, so the limit
 // is raised whatever the dynamic size)
-cudaError_t center_allow_smem(int variant, int smem, bool near) {
+cudaError_t center_allow_smem(int variant, bool near) {
   center_fn fn = near ? center_near_kernel(variant) : center_kernel(variant);
   if (!fn) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return allow_smem((const void *)fn);
 }
 
 cudaError_t launch_center(int variant, const SeqSet &ss, const Scoring &sc, const CenterJob &job,
@@ -1381,7 +1381,7 @@ cudaError_t launch_center(int variant, const SeqSet &ss, const Scoring &sc, cons
   const CenterVariant &v = kCenterVariants[variant];
   const int smem = center_smem_bytes(variant, sc.K, job.npass * v.G * v.R);
   if (set_smem) {
-    const cudaError_t e = center_allow_smem(variant, smem, near);
+    const cudaError_t e = center_allow_smem(variant, near);
     if (e != cudaSuccess) return e;
   }
   fn<<<grid, kCenterThreads, smem, st>>>(ss, sc, job);
@@ -1412,7 +1412,7 @@ cudaError_t launch_pairs(int G, bool packed, const SeqSet &ss, const Scoring &sc
   if (!fn) return cudaErrorInvalidValue;
   const int smem = pairs_smem(sc.K, packed);
   if (smem > 40 * 1024)  // static shared memory counts too
-    cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    allow_smem((const void *)fn);
   fn<<<grid, 256, smem, st>>>(ss, sc, job);
   return cudaGetLastError();
 }
@@ -1495,7 +1495,7 @@ cudaError_t near_allow_smem(int G, int smem) {
   codes_fn fn = near_kernel(G);
   if (!fn) return cudaErrorInvalidValue;
   if (smem <= 40 * 1024) return cudaSuccess;  // static shared memory counts too
-  return cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return allow_smem((const void *)fn);
 }
 
 cudaError_t launch_codes_near(int G, const SeqSet &ss, const Scoring &sc, const CodesJob &job, int grid,
@@ -1516,7 +1516,7 @@ cudaError_t codes_allow_smem(int G, bool packed, int smem, int threads) {
   codes_fn fn = codes_kernel(G, packed, threads);
   if (!fn) return cudaErrorInvalidValue;
   if (smem <= 40 * 1024) return cudaSuccess;  // static shared memory counts too
-  return cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return allow_smem((const void *)fn);
 }
 
 cudaError_t launch_codes(int G, bool packed, const SeqSet &ss, const Scoring &sc, const CodesJob &job,
@@ -1685,10 +1685,7 @@ extern "C" int msa_pair_scores_noalloc(const uint8_t *residues, const int64_t *o
   const int np_max = (max_len + kNoallocG * kPairsR - 1) / (kNoallocG * kPairsR);
   const size_t per_cta = np_max > 1 ? (size_t)NG * 2 * max_len * sizeof(int2) : 0;
   const int smem = NG * (alphabet + 1) * kNoallocG * kPairsR;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute((const void *)k_pairs_noalloc,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return MSA_ECUDA;
+  if (smem > 48 * 1024 && allow_smem((const void *)k_pairs_noalloc) != cudaSuccess) return MSA_ECUDA;
   int per_sm = 0, sms = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairs_noalloc, 256, smem);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

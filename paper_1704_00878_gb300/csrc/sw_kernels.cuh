@@ -90,7 +90,7 @@ int center_profile_bytes(int variant, int K, int rows_alloc);
 // of one pair each).
 cudaError_t launch_center(int variant, const SeqSet &ss, const Scoring &sc, const CenterJob &job,
                           int grid, cudaStream_t st, bool set_smem = true, bool near = false);
-cudaError_t center_allow_smem(int variant, int smem, bool near = false);
+cudaError_t center_allow_smem(int variant, bool near = false);
 int center_grid(int variant, int smem);
 
 // packed: two pairs per group in int16 lanes (G 8, 16 or 32; the caller checks
