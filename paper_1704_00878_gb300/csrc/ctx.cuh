@@ -22,7 +22,6 @@ enum Stage {
 
 struct Selector;  // the learned center selector (selector.cu)
 constexpr int kMaxTreeRows = 65536;  // rows of a neighbour-joining tree
-constexpr int kCenterLanes = 8;      // branches of the center graph
 constexpr int kDerrWords = 4;        // msa_ctx::derr
 void selector_free(msa_ctx *ctx, Selector *s);
 

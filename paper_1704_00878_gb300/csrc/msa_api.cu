@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "msa.h"
+#include "center_rows.cuh"
 #include "few.cuh"
 #include "msa_kernels.cuh"
 #include "sw_kernels.cuh"
@@ -413,6 +414,7 @@ struct ClassPlan {
   enum Role { kAlone, kFull, kNear } role = kAlone;
   size_t prefix_off;  // into the concatenated prefix of all planned classes
   int64_t n_items;
+  bool keeps_rows() const { return center_keeps_rows(npass, role == kNear); }
 };
 
 // rows of query pair p in a stream of R-row blocks: the longer of its two
@@ -488,8 +490,8 @@ CenterJob class_job(msa_ctx *ctx, int mode, const ClassPlan &pl, int sub_off, in
   return job;
 }
 
-// Upload the plans' prefixes and size the scratch rows of multi-pass
-// classes (those of a lane run in stream order, so they share one scratch).
+// Upload the plans' prefixes and size the boundary rows of the classes that
+// keep them (those of a lane run in stream order, so they share one area).
 int stage_plans(msa_ctx *ctx, const std::vector<ClassPlan> &plans,
                 const std::vector<int64_t> &prefix_all, const std::vector<int2> &streams) {
   TRY(ensure(ctx, ctx->streams, sizeof(int2) * std::max<size_t>(streams.size(), 1)));
@@ -498,11 +500,11 @@ int stage_plans(msa_ctx *ctx, const std::vector<ClassPlan> &plans,
                        cudaMemcpyHostToDevice, ctx->st));
   size_t scratch = 0;
   for (const ClassPlan &pl : plans)
-    if (pl.npass > 1)
+    if (pl.keeps_rows())
       scratch = std::max(scratch, (size_t)pl.grid * (kCenterThreads / kCenterVariants[pl.cc.variant].G) *
                                       2 * ctx->maxlen * sizeof(int2));
-  // the graph runs its multi-pass classes in two lanes: one boundary-row area each
-  if (scratch) TRY(ensure(ctx, ctx->scratch, 2 * scratch));
+  // the graph runs the classes that keep rows in two lanes: one area each
+  if (scratch) TRY(ensure(ctx, ctx->scratch, kRowLanes * scratch));
   ctx->scratch_half = scratch / sizeof(int2);
   TRY(ensure(ctx, ctx->prefix, sizeof(int64_t) * prefix_all.size()));
   TRY(ensure(ctx, ctx->counters, sizeof(unsigned long long) * std::max<size_t>(plans.size(), 1)));
@@ -557,14 +559,14 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
   // set and buffers, e.g. a repeated step) relaunches the cached graph.
   // The classes run longest queries first, dealt out to the lanes of a fork
   // and a join in the graph, so the CTAs that a class's last, long items leave
-  // free go to the classes after it.  Multi-pass classes take the first two
-  // lanes only, which have a boundary-row area each.  A set of a few hundred
+  // free go to the classes after it.  Classes that keep boundary rows take the
+  // first two lanes only, which have an area each.  A set of a few hundred
   // sequences is all tails: the all-pairs selection of 100 (200) proteins took
   // 463 (505) us in two lanes and 234 (402) in eight.
   std::vector<CenterJob> jobs;
   auto lane_of = [&](size_t c) {
     const size_t order = plans.size() - 1 - c;  // launch position
-    return (int)(order % (plans[c].npass > 1 ? 2 : kCenterLanes));
+    return center_lane((int)order, plans[c].keeps_rows());
   };
   std::vector<int64_t> key = {mode, sub_off, sub_n, (int64_t)ss.res, (int64_t)ss.pstart,
                               (int64_t)ss.len, ss.n, (int64_t)sc.M, sc.K, sc.o, sc.e,
