@@ -1730,10 +1730,11 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
   // so only from 3e9 cells on (2 ms or more: 20,000 unrelated subjects of 400
   // 2,912 us without, 2,920 with; 2,000 similar ones of 1,500 4,285 and 3,234),
   // and only where a subject may match most of the center (a short one leaves no
-  // column out) and there are several passes.
+  // column out) and there are several passes.  (Not while msa_align_autotune times
+  // the full fill's shapes.)
   const int Gs = ctx->align_group_fixed ? G : near_group(G, n);
   const int near_npass = (Lc + Gs * R - 1) / (Gs * R), near_smem = codes_smem_bytes(ctx->K, near_npass * Gs * R);
-  bool near = packed && Gs >= 8 && near_npass > 1 && Lc >= 256 && ctx->smax > 0 &&
+  bool near = packed && !ctx->align_tuning && Gs >= 8 && near_npass > 1 && Lc >= 256 && ctx->smax > 0 &&
                     (cells >= (int64_t)3e9 || ctx->align_group_fixed) && 2 * ctx->residues >= (int64_t)n * Lc;
   const int ngrid = near ? near_grid(Gs, near_smem) : 0;
   const size_t boundary = 2 * (size_t)ctx->maxlen * sizeof(int2);  // rows of a group

@@ -125,3 +125,26 @@ def test_center_of_similar_sequences_matches_full_columns(n, nref, length, odd_e
             got.append((c, b.msa_center_rowsums(h)))
     assert got[0][0] == got[1][0]
     assert (got[0][1] == got[1][1]).all()
+
+
+def test_autotune_times_the_full_fill_of_similar_subjects():
+    """Two launches (fill and traceback) per timed shape: the bounded fill, which
+    has a shape of its own, stays out; the next alignment has it again, and the
+    vote and it are two launches more."""
+    b = binding()
+    rng = np.random.default_rng(3)
+    alph, M = dna_matrix()
+    pool = np.frombuffer(b"ACGT", np.uint8)
+    center = rng.choice(pool, size=1500)
+    letters, offsets = pack_sequences([mutate(rng, center, 0.02, pool) for _ in range(1400)])  # 3.15e9 cells
+    with make_ctx(alph, M, 5, 2) as h:
+        b.msa_load(h, letters, offsets)
+        count = lambda: b.msa_stage_times(h)[1]["launches"]  # noqa: E731
+        before = count()
+        rates, _ = b.msa_align_autotune(h, 0)
+        shapes = int((rates > 0).sum())
+        assert shapes == 15 and count() - before == 2 * 2 * shapes  # (each shape runs twice)
+        b.msa_set_align_group(h, 8)
+        before = count()
+        b.msa_align_to_center(h, 0)
+        assert count() - before == 4
