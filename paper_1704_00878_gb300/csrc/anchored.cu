@@ -45,6 +45,7 @@ namespace {
 constexpr int kAnchThreads = 256, kAnchWarps = kAnchThreads / 32;  // at most
 constexpr int kBoxSide = 80;                         // longest stretch side
 constexpr int kLaneCols = 24;                        // columns of a stretch that one lane aligns
+constexpr int kLaneSort = 16;                        // matches of a segment that one lane orders
 constexpr int kHashBits = 15;                        // bit table of the segments' keys
 constexpr int kNeg = -(1 << 29);                      // stands for minus infinity
 constexpr int kPosBits = 13;                          // match = segment << 13 | position
@@ -362,6 +363,27 @@ __device__ __forceinline__ uint32_t key_bit(unsigned long long key) {
 }
 __device__ __forceinline__ uint32_t key_bit(uint32_t key) { return (key * 0x9e3779b1u) >> (32 - kHashBits); }
 
+// Sorts v[0..n) by the whole warp: a bitonic network whose first step of every
+// size compares mirrored positions, so that all comparisons are ascending and
+// those that reach past n (a place that holds the largest value) do nothing.
+__device__ void warp_sort(uint32_t *v, int n, int lane) {
+  for (int size = 2; size < 2 * n; size <<= 1)
+    for (int d = size >> 1; d > 0; d >>= 1) {
+      const bool mirrored = d == size >> 1;
+      for (int p = lane;; p += 32) {
+        const int i = ((p & ~(d - 1)) << 1) | (p & (d - 1)), j = mirrored ? i ^ (size - 1) : i + d;
+        if (i >= n) break;
+        if (j >= n) continue;
+        const uint32_t a = v[i], b = v[j];
+        if (a > b) {
+          v[i] = b;
+          v[j] = a;
+        }
+      }
+      __syncwarp();
+    }
+}
+
 // Per-warp shared memory: `cap` sorted matches (4 bytes), three 16-bit arrays
 // of cap entries, and an area that holds the unsorted matches and the
 // segments' counts first and the stretch aligners' workspace later.
@@ -477,7 +499,10 @@ __global__ void __launch_bounds__(kAnchThreads, 2) k_anchored(SeqSet ss, Scoring
       continue;
     }
     // (b) order the matches by (segment, position): starts by a scan of the
-    // counts, then a segment's few matches sorted in place
+    // counts, then a segment's few matches sorted in place by one lane, the many
+    // matches of a repeat by the warp (one lane's insertions are quadratic: 20,000
+    // subjects with 208 and 338 matches of one segment 4.1 and 9.9 ms by one lane,
+    // 0.70 and 1.02 by the warp)
     {
       const int per = (S + 31) / 32, s0 = min(S, lane * per), s1 = min(S, s0 + per);
       int sum = 0;
@@ -500,13 +525,18 @@ __global__ void __launch_bounds__(kAnchThreads, 2) k_anchored(SeqSet ss, Scoring
         mbuf[atomicAdd(&segat[v >> kPosBits], 1)] = v;
       }
       __syncwarp();
-      for (int s = lane; s < S; s += 32) {  // segat[s] is now the end of segment s
-        const int b = s > 0 ? segat[s - 1] : 0, end = segat[s];
-        for (int i = b + 1; i < end; ++i) {
+      for (int sb = 0; sb < S; sb += 32) {  // segat[s] is now the end of segment s
+        const int s = sb + lane, end = s < S ? segat[s] : 0, b = s < S && s > 0 ? segat[s - 1] : 0;
+        const bool many = end - b > kLaneSort;
+        for (int i = b + 1; i < end && !many; ++i) {
           const uint32_t v = mbuf[i];
           int j = i;
           for (; j > b && mbuf[j - 1] > v; --j) mbuf[j] = mbuf[j - 1];
           mbuf[j] = v;
+        }
+        for (unsigned left = __ballot_sync(MSA_FULL_MASK, many); left; left &= left - 1) {
+          const int l = __ffs(left) - 1, from = __shfl_sync(MSA_FULL_MASK, b, l);
+          warp_sort(mbuf + from, __shfl_sync(MSA_FULL_MASK, end, l) - from, lane);
         }
       }
       __syncwarp();

@@ -110,3 +110,35 @@ def test_stretch_sizes_and_repeated_segments(k):
         with make_ctx(alph, M, 5, 2) as h:
             b.msa_load(h, letters, offsets)
             _check(b, h, prob, 0, k, letters, offsets)
+
+
+@pytest.mark.parametrize("segments", [1, 2, 3])
+def test_segments_with_many_matches(segments):
+    """A run of one residue over one to three center segments, longer in the
+    subjects: 9 to 90 matches of each of them, around the 16 that one lane
+    orders and the sizes of the warp's network; and runs so long that the
+    subject goes to the local path after the ordering."""
+    b = binding()
+    alph, M = dna_matrix(2, -3)
+    rng = np.random.default_rng(50 + segments)
+    pool = np.frombuffer(b"ACGT", np.uint8)
+    center = rng.choice(pool, size=1300)
+    at = 640
+    center[at:at + 8 * segments] = ord("A")
+    center[at - 1] = center[at + 8 * segments] = ord("C")
+    seqs = [center]
+    for matches in (9, 15, 16, 17, 18, 31, 32, 33, 34, 63, 64, 65, 66, 80, 140):
+        for _ in range(3):
+            s = center.copy()
+            hit = rng.random(s.size) < 0.02
+            s[hit] = rng.choice(pool, size=int(hit.sum()))
+            s[at:at + 8 * segments] = ord("A")
+            s[at - 1] = s[at + 8 * segments] = ord("C")
+            extra = max(0, matches + 7 - 8 * segments)
+            seqs.append(np.concatenate([s[:at], np.full(extra, ord("A"), np.uint8), s[at:]]))
+    letters, offsets = pack_sequences(seqs)
+    prob = oracle_problem(letters, offsets, alph, M, 5, 2)
+    with make_ctx(alph, M, 5, 2) as h:
+        b.msa_load(h, letters, offsets)
+        nf = _check(b, h, prob, 0, 8, letters, offsets)
+    assert 3 <= nf <= 9
