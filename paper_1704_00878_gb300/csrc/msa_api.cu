@@ -575,7 +575,7 @@ int launch_plans(msa_ctx *ctx, int mode, const std::vector<ClassPlan> &plans, in
     CenterJob job = class_job(ctx, mode, plans[c], sub_off, sub_n, cnt + c, self);
     if (plans[c].role != ClassPlan::kAlone) {
       job.similar = similar;
-      job.similar_min = kSimilarSample / 2;
+      job.similar_min = kSimilarCenter;
       job.smax = ctx->smax;
     }
     if (lane_of(c) == 1) job.scratch += ctx->scratch_half;
@@ -1797,7 +1797,7 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
       if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dcounter, 0, sizeof(unsigned long long), ctx->cap_lanes[0]);
       // offsets inside the batch are relative to the batch start
       job.similar = similar;
-      job.similar_min = kSimilarSample / 2;
+      job.similar_min = kSimilarAlign;
       if (near && bi == 0 && e == cudaSuccess) e = launch_similar(ss, n, nullptr, kc, 1, similar, ctx->cap_lanes[0]);
       if (e == cudaSuccess) e = launch_codes(G, packed, ss, sc, job, grid, ctx->cap_lanes[0], false, cta);
       if (near && e == cudaSuccess) {
@@ -1812,7 +1812,7 @@ int msa_align_to_center(msa_ctx *ctx, int64_t center, int32_t *scores_out) {
                              P<int32_t>(ctx->d_perm), ss.res, ss.pstart, kc, sc.M, sc.K, sc.o, sc.e,
                              Lc, G, P<uint16_t>(ctx->ins), P<uint8_t>(ctx->occ), P<int32_t>(ctx->seg),
                              P<int32_t>(ctx->score), ctx->derr, ctx->cap_lanes[0], nullptr, nullptr,
-                             nullptr, similar, kSimilarSample / 2, Gs);
+                             nullptr, similar, kSimilarAlign, Gs);
       if (e == cudaSuccess) e = cudaEventRecordWithFlags(ctx->align_ev[3 * bi + 2], ctx->cap_lanes[0], cudaEventRecordExternal);
     }
     cudaGraph_t graph = nullptr;

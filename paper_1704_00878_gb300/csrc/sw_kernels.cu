@@ -1233,10 +1233,11 @@ __global__ void __launch_bounds__(256, 1) k_codes_near(SeqSet ss, Scoring sc, Co
 }
 
 // Whether the subjects resemble the queries: of kSimilarSample subjects spread
-// over the set, how many share at least 12 of 32 words of 12 residues with a query
-// (residues that differ in 8 % or more share fewer).  A CTA per subject, a word
-// per lane, a quarter of the query per warp: about 3 us.
-constexpr int kWordLen = 12, kWordBits = 5;
+// over the set, how many share at least 6 of 32 words of 12 residues with a query
+// (of pairs that differ in 8 % of their residues 19 in 20 do, of those that differ
+// in 12 % half; unrelated ones share none).  A CTA per subject, a word per lane, a
+// quarter of the query per warp: about 3 us.
+constexpr int kWordLen = 12, kWordBits = 5, kWordsShared = 6;
 
 __global__ void __launch_bounds__(128) k_similar(SeqSet ss, int nsub, const int32_t *qlist, int q0, int nq, unsigned *similar) {
   __shared__ unsigned s_found[4];
@@ -1266,7 +1267,7 @@ __global__ void __launch_bounds__(128) k_similar(SeqSet ss, int nsub, const int3
   const unsigned votes = __ballot_sync(MSA_FULL_MASK, found);
   if (lane == 0) s_found[warp] = votes;
   __syncthreads();
-  if (threadIdx.x == 0 && __popc(s_found[0] | s_found[1] | s_found[2] | s_found[3]) >= 12) atomicAdd(similar, 1u);
+  if (threadIdx.x == 0 && __popc(s_found[0] | s_found[1] | s_found[2] | s_found[3]) >= kWordsShared) atomicAdd(similar, 1u);
 }
 
 }  // namespace

@@ -122,7 +122,14 @@ int codes_threads(bool packed, int threads = 256);  // threads per CTA of the co
 // leave out more columns (a pass has fewer rows), and pay once every warp has
 // four items: with 8 / 16 / 32 lanes 60,000 of 1,500 residues 28.8 / 30.5 / 36.3
 // ms, 20,000 10.3 / 10.6 / 12.8, 10,000 of 2,900 29.9 / 26.5 / 22.2.
-constexpr int kSimilarSample = 64;
+// The bounded kernels take 234 of 256 votes (alignment) and 238 (center).  A warp
+// shares its guess, so one unrelated pair makes its next turn fill every column,
+// and from about 9 and 8 unrelated pairs in 100 on filling every column at once is
+// faster: of 1,500 residues, 20,000 subjects 23.4 ms (bounded, with 0 / 3 / 6 / 10 /
+// 15 / 25 unrelated in 100: 14.7 / 18.9 / 21.5 / 23.6 / 26.4 / 28.5), 3,000 against
+// 100 references 100.5 (with 0 / 4 / 8 / 12 / 19 / 44 unrelated pairs in 100: 47.1 /
+// 82.7 / 101.5 / 109.6 / 121 / 127).
+constexpr int kSimilarSample = 256, kSimilarAlign = 234, kSimilarCenter = 238;
 int near_group(int G, int64_t n);
 int near_grid(int G, int smem);
 cudaError_t near_allow_smem(int G, int smem);
