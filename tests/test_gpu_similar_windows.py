@@ -148,3 +148,99 @@ def test_autotune_times_the_full_fill_of_similar_subjects():
         before = count()
         b.msa_align_to_center(h, 0)
         assert count() - before == 4
+
+
+@pytest.mark.parametrize("kind, o, e", [("dna", 5, 2), ("dna", 2, 1), ("dna", 3, 3), ("protein", 11, 1)])
+@pytest.mark.parametrize("lanes", [8, 16, 32])
+def test_variants_among_many_similar_subjects(kind, o, e, lanes):
+    """The subjects of test_similar_subjects_match_the_oracle, and again as many
+    close ones as make the set a similar one (unrelated ones are few)."""
+    b = binding()
+    rng = np.random.default_rng(o * 1000 + lanes)
+    alph, M = blosum62() if kind == "protein" else dna_matrix()
+    pool = np.frombuffer(("ARNDCQEGHILKMFPSTWYV" if kind == "protein" else "ACGT").encode(), np.uint8)
+    half = rng.choice(pool, size=330)
+    for center in (rng.choice(pool, size=700), np.concatenate([half, mutate(rng, half, 0.03, pool)])):
+        seqs = variants(rng, center, pool)
+        # spread over the lengths: the sample of the vote is taken in their order
+        close = [mutate(rng, center[:center.size - int(k)], 0.02, pool) for k in rng.integers(0, 300, 6 * len(seqs))]
+        letters, offsets = pack_sequences([center] + seqs + close)
+        prob = oracle_problem(letters, offsets, alph, M, o, e)
+        oseg, oins, oocc, _, _, _ = oracle.msa(prob, 0)
+        with make_ctx(alph, M, o, e) as h:
+            b.msa_load(h, letters, offsets)
+            b.msa_set_align_group(h, lanes)
+            b.msa_align_to_center(h, 0)
+            seg, ins, occ = b.msa_alignment_info(h)
+        assert (seg == oseg).all()
+        assert (ins == oins).all() and (occ == oocc).all()
+
+
+def similar_set(rng, n, length, odd_every, pool):
+    """n sequences cut from variants of one, every odd_every-th one unrelated or
+    a repeat of its start."""
+    center = rng.choice(pool, size=length)
+    seqs = [center]
+    for x in range(1, n):
+        if odd_every and x % odd_every == 0:
+            seqs.append(rng.choice(pool, size=int(rng.integers(length // 2, length))) if x & 1
+                        else np.tile(center[:90], length // 100))
+            continue
+        s = mutate(rng, center, (0.0, 0.02, 0.04)[x % 3], pool)
+        a, k = int(rng.integers(0, length // 20)), int(rng.integers(length // 8, length))
+        seqs.append(np.concatenate([s[a:k], s[k + int(rng.integers(0, 40)):]]))
+    return pack_sequences(seqs)
+
+
+@pytest.mark.parametrize("n, length, budget", [(20500, 420, 0), (20500, 420, 1 << 29), (40000, 300, 0), (1500, 1500, 0)])
+@pytest.mark.parametrize("odd_every", [0, 40])
+def test_narrower_bounded_groups_and_batches(n, length, budget, odd_every):
+    """The default shapes from 3e9 cells on: the bounded fill's groups narrower
+    than the full fill's (its codes then lie in a buffer laid out for the wider
+    ones), in one batch of codes and in several, against int32 cells."""
+    b = binding()
+    rng = np.random.default_rng(n + odd_every)
+    alph, M = dna_matrix()
+    letters, offsets = similar_set(rng, n, length, odd_every, np.frombuffer(b"ACGT", np.uint8))
+    got, launches = [], 0
+    for precision in (b.MSA_INT32, b.MSA_AUTO):
+        with make_ctx(alph, M, 5, 2, precision=precision) as h:
+            b.msa_load(h, letters, offsets)
+            if budget:
+                b.msa_set_codes_budget(h, budget)
+            before = b.msa_stage_times(h)[1]["launches"]
+            b.msa_align_to_center(h, 0)
+            launches = b.msa_stage_times(h)[1]["launches"] - before
+            got.append(b.msa_alignment_info(h))
+    # a vote, and per batch the two fills and the traceback
+    assert launches % 3 == 1 and (launches > 4) == (budget > 0)
+    for x, y in zip(*got):
+        assert (x == y).all()
+
+
+# queries of several passes of the full kernel, 2e10 cells and more; few groups
+# (60 x 400) take the 16 x 16 shape, the others 8 x 20
+@pytest.mark.parametrize("n, nref, length", [(1200, 41, 1500), (2600, 24, 1300), (400, 60, 2600), (420, 0, 1300)])
+@pytest.mark.parametrize("odd_every", [0, 60])
+def test_bounded_center_beside_the_full_one(n, nref, length, odd_every):
+    """Row sums over a sample of references (an odd and an even number) and over
+    every pair, where the bounded kernel takes every multi-pass query.  A context
+    under a memory limit plans the full kernel alone, with fewer launches."""
+    b = binding()
+    rng = np.random.default_rng(n + odd_every)
+    alph, M = dna_matrix()
+    letters, offsets = similar_set(rng, n, length, odd_every, np.frombuffer(b"ACGT", np.uint8))
+    refs = np.sort(rng.choice(n, size=max(nref, 1), replace=False))
+    got, launches = [], []
+    for precision, limit in ((b.MSA_AUTO, 0), (b.MSA_AUTO, 1 << 35), (b.MSA_INT32, 0)):
+        with make_ctx(alph, M, 5, 2, precision=precision) as h:
+            b.msa_set_memory_limit(h, limit)
+            b.msa_load(h, letters, offsets)
+            before = b.msa_stage_times(h)[1]["launches"]
+            c = (b.msa_select_center(h, b.MSA_CENTER_EXACT_SAMPLED, refs=refs) if nref
+                 else b.msa_select_center(h, b.MSA_CENTER_EXACT))
+            launches.append(b.msa_stage_times(h)[1]["launches"] - before)
+            got.append((c, b.msa_center_rowsums(h)))
+    assert launches[0] >= launches[1] + 2  # the vote and the bounded launch
+    for c, sums in got[:2]:
+        assert c == got[2][0] and (sums == got[2][1]).all()
