@@ -813,7 +813,7 @@ int run_center(msa_ctx *ctx, int mode, const std::vector<int32_t> &qsorted, cons
   // Cells near the int16 limit (which the precision setting may allow), profiles
   // beyond shared memory and a device memory limit (the narrower groups want more
   // boundary rows) keep the full kernel.
-  const int near_variant = fill(8) < 1.0 ? 14 : 1;
+  const int near_variant = fill(8) < 1.0 ? kNearFewVariant : kNearVariant;
   const int longest = p_end > p_begin ? qlen[std::min(2 * p_end, x1) - 1] : 0;
   const bool may_near = center_cells >= (int64_t)2e10 && longest > 0 && ctx->smax > 0 && !ctx->dev_limit &&
                         (long long)longest * ctx->smax <= sat_thresh(ctx) &&

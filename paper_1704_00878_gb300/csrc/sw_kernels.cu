@@ -1328,20 +1328,11 @@ static center_fn center_kernel(int variant) {
   }
 }
 
-// The paired variants' bounded form.
+// The bounded kernel's two shapes, under the numbers of the full kernel's.
 static center_fn center_near_kernel(int variant) {
   switch (variant) {
-    case 0: return k_center_near<8, 12>;
-    case 1: return k_center_near<8, 20>;
-    case 2: return k_center_near<8, 28>;
-    case 3: return k_center_near<16, 12>;
-    case 4: return k_center_near<16, 20>;
-    case 5: return k_center_near<16, 28>;
-    case 6: return k_center_near<32, 12>;
-    case 7: return k_center_near<32, 20>;
-    case 8: return k_center_near<32, 28>;
-    case 14: return k_center_near<16, 16>;
-    case 15: return k_center_near<16, 24>;
+    case kNearVariant: return k_center_near<8, 20>;
+    case kNearFewVariant: return k_center_near<16, 16>;
     default: return nullptr;
   }
 }

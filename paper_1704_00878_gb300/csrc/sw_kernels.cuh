@@ -79,6 +79,8 @@ struct CodesJob {
 struct CenterVariant { int paired, G, R; bool packed; };
 extern const CenterVariant kCenterVariants[];
 extern const int kNumCenterVariants;
+// the shapes of the bounded kernel: 8 lanes x 20 rows, 16 x 16 for short lists
+constexpr int kNearVariant = 1, kNearFewVariant = 14;
 
 // dynamic shared memory of a center launch whose units need rows_alloc
 // profile rows; center_profile_bytes: the profile part alone
@@ -86,8 +88,8 @@ int center_smem_bytes(int variant, int K, int rows_alloc);
 int center_profile_bytes(int variant, int K, int rows_alloc);
 // set_smem = false: the caller has already raised the kernel's dynamic
 // shared-memory limit with center_allow_smem (required while a stream is
-// being captured into a graph).  near: the bounded form (paired variants, units
-// of one pair each).
+// being captured into a graph).  near: the bounded form (kNearVariant and
+// kNearFewVariant, units of one pair each).
 cudaError_t launch_center(int variant, const SeqSet &ss, const Scoring &sc, const CenterJob &job,
                           int grid, cudaStream_t st, bool set_smem = true, bool near = false);
 cudaError_t center_allow_smem(int variant, bool near = false);
