@@ -513,6 +513,15 @@ int msa_nj_cluster_tree(msa_ctx *ctx, const int64_t *sample, int64_t nsample, in
  * MSA_ECUDA / MSA_ENOMEM if the probe could not run. */
 int msa_debug_wait_timeout(msa_ctx *ctx, int32_t *timed_out);
 
+/* Forces the launch shape of later neighbour-joining calls on this context (no
+ * counterpart in the paper; for tests, which reach at small sizes what the
+ * library chooses at large ones): ctas = 1, 8 or 16 CTAs per launch above 128
+ * rows, threads = 256, 512 or 1024 (256 with one CTA), 0 = the library's choice
+ * by the rows; sums_global != 0: the row sums in global memory.  The result does not
+ * depend on it.  EINVAL for any other value; ERANGE from the joining where its rows
+ * do not fit the shape (one CTA: beyond 9,000). */
+int msa_debug_nj_shape(msa_ctx *ctx, int32_t ctas, int32_t threads, int32_t sums_global);
+
 #ifdef __cplusplus
 }
 #endif

@@ -78,6 +78,7 @@ _SIGS = {
     "msa_set_codes_budget": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64]),
     "msa_set_align_group": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32]),
     "msa_debug_wait_timeout": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
+    "msa_debug_nj_shape": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32]),
     "msa_tree_distances": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
     "msa_set_align_threads": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32]),
     "msa_set_align_mode": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32]),
@@ -367,6 +368,13 @@ def msa_sp_score(ctx):
     v = np.zeros(1, np.int64)
     _check(ctx, lib().msa_sp_score(ctx, _ptr(v)))
     return int(v[0])
+
+
+def msa_debug_nj_shape(ctx, ctas=0, threads=0, sums_global=False):
+    """Forces the launch shape of later neighbour joinings (0: the library's choice)."""
+    rc = lib().msa_debug_nj_shape(ctx, int(ctas), int(threads), int(bool(sums_global)))
+    if rc != MSA_OK:
+        raise MSAError(rc, "ctas must be 0, 1, 8 or 16, threads 0, 256, 512 or 1024")
 
 
 def msa_tree_distances(ctx, out=None):

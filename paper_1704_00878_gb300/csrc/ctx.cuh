@@ -117,6 +117,11 @@ struct msa_ctx {
 
   msa_detail::Selector *sel = nullptr;
 
+  // msa_debug_nj_shape: the joins' cluster and threads (0: chosen by the rows),
+  // their row sums in global memory
+  int nj_ctas = 0, nj_threads = 0;
+  bool nj_sums_global = false;
+
   // autotuner: measured cells/s of each center variant per query-length bucket
   std::vector<int> tune_edges;                 // bucket b = [edges[b], edges[b+1])
   std::vector<std::vector<double>> tune_rate;  // [bucket][variant], 0 = not measured

@@ -10,7 +10,7 @@
 // joined distance within 2^30, else ERANGE -- positions in ascending slot
 // order); one launch of a thread-block cluster runs the joins until half of the
 // positions are left (k_nj_joins), then the matrix is packed to the active ones; the
-// last few hundred positions run in one CTA.
+// last 128 positions run in one CTA.
 #include <algorithm>
 #include <climits>
 #include <vector>
@@ -25,7 +25,8 @@ constexpr int kPlaneWords = 15;  // 32-column words staged per step
 constexpr int kSlab = 16384;     // rows whose planes are held at once
 constexpr long long kDScale = 1LL << 20;
 constexpr long long kDLimit = 1LL << 30;  // |distance| bound of the joins (int32 matrix)
-constexpr int kJoinCtas = 16;      // CTAs of a large matrix's joins: one cluster
+constexpr int kJoinCtas = 16;      // CTAs of a large matrix's joins: one cluster,
+constexpr int kJoinCtasFew = 8;    // smaller where the device has no room for it
 constexpr int kSoloRows = 128;     // a matrix of at most this many positions: one CTA
 constexpr int kScanSeg = 512;      // columns of one warp task of a row scan: 16 per lane
 constexpr int kScanTasks = 256;    // scan results held at once (a row has at most 128 segments)
@@ -772,6 +773,70 @@ __global__ void k_outgroups(const int *__restrict__ D, int m, const int32_t *__r
   if ((threadIdx.x & 31) == 0 && best != ~0ull) atomicMin(&key[c], best);
 }
 
+using join_fn = void (*)(NjJob);
+static join_fn join_kernel(int ctas, int threads) {
+  if (ctas == 1) return k_nj_joins<1, 256>;
+  if (ctas == kJoinCtasFew)
+    return threads == 256 ? k_nj_joins<kJoinCtasFew, 256>
+         : threads == 512 ? k_nj_joins<kJoinCtasFew, 512> : k_nj_joins<kJoinCtasFew, 1024>;
+  return threads == 256 ? k_nj_joins<kJoinCtas, 256>
+       : threads == 512 ? k_nj_joins<kJoinCtas, 512> : k_nj_joins<kJoinCtas, 1024>;
+}
+
+// One launch of the joins of P positions.
+struct JoinShape {
+  int ctas, threads;
+  bool rshared;  // the row sums fit shared memory
+  size_t smem;
+};
+static JoinShape join_shape(int P, int ctas, int threads, bool sums_global) {
+  JoinShape s{ctas, threads, false, 0};
+  const size_t cap = (size_t)(P + ctas - 1) / ctas;
+  s.smem = cap * (sizeof(long long) + 4 * sizeof(int)) + sizeof(unsigned) * (((size_t)P + 31) / 32);
+  s.rshared = !sums_global && s.smem + sizeof(long long) * (size_t)P <= (size_t)kJoinSmem;
+  if (s.rshared) s.smem += sizeof(long long) * (size_t)P;
+  return s;
+}
+
+// Fills cfg and attr for a launch of s (attr must outlive the launch).
+static cudaError_t join_config(const JoinShape &s, cudaStream_t st, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr) {
+  const void *fn = (const void *)join_kernel(s.ctas, s.threads);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kJoinSmem);
+  if (e == cudaSuccess && s.ctas > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)s.ctas;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg = {};
+  cfg.gridDim = dim3((unsigned)s.ctas);
+  cfg.blockDim = dim3((unsigned)s.threads);
+  cfg.dynamicSmemBytes = s.smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = s.ctas > 1 ? 1 : 0;
+  return e;
+}
+
+// fewer threads make the block-wide steps of a join cheaper, more keep more of
+// rows x and y in flight
+static int join_threads(int P) { return P <= 1536 ? 256 : P <= 8192 ? 512 : 1024; }
+
+// CTAs of the joins' cluster: 16 (not portable: a partition of the device, or a
+// GPC with fewer free SMs, may have no room for it), else 8, which every device
+// of this architecture runs.  4,000 rows 30.7 ms with 16,
+// 36.4 with 8; 10,000 139 and 168.
+static int join_ctas(int n) {
+  const JoinShape s = join_shape(n, kJoinCtas, join_threads(n), false);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  int clusters = 0;
+  if (join_config(s, nullptr, cfg, attr) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&clusters, (const void *)join_kernel(s.ctas, s.threads), &cfg) == cudaSuccess &&
+      clusters > 0)
+    return kJoinCtas;
+  cudaGetLastError();
+  return kJoinCtasFew;
+}
+
 // Row sums and the joins of the n x n int32 matrix in D1 (device; repacked in
 // place of copies as positions retire).  derr must be clear.
 int nj_device(msa_ctx *ctx, DevBuf &D1, int n, int32_t *joins_out, double *lengths_out) {
@@ -798,41 +863,24 @@ int nj_device(msa_ctx *ctx, DevBuf &D1, int n, int32_t *joins_out, double *lengt
     DevBuf *cD = &D1, *cR = &r, *cN = &node;
     DevBuf *oD = &D2, *oR = &r2, *oN = &node2;
     int Pn = n, t = 0;
+    const int ctas = ctx->nj_ctas > 0 ? ctx->nj_ctas : n > kSoloRows ? join_ctas(n) : 1;
     while (Pn > 2) {
       // a large matrix until half of its positions are left, then packed
       const bool solo = Pn <= kSoloRows;
-      const int grid = solo ? 1 : kJoinCtas, stop = solo ? 2 : std::max(kSoloRows, Pn / 2);
-      const size_t cap = (size_t)(Pn + grid - 1) / grid;
-      const size_t own = cap * (sizeof(long long) + 4 * sizeof(int)) + sizeof(unsigned) * (((size_t)Pn + 31) / 32);
-      const bool rshared = own + sizeof(long long) * (size_t)Pn <= (size_t)kJoinSmem;
-      if (!rshared) TRY(ensure(ctx, rcopy, sizeof(long long) * (size_t)Pn * grid));
-      const size_t smem = own + (rshared ? sizeof(long long) * (size_t)Pn : 0);
+      const int stop = solo ? 2 : std::max(kSoloRows, Pn / 2), grid = solo ? 1 : ctas;
+      const int threads = grid == 1 ? 256 : ctx->nj_threads > 0 ? ctx->nj_threads : join_threads(Pn);
+      const JoinShape s = join_shape(Pn, grid, threads, ctx->nj_sums_global);
+      if (s.smem > (size_t)kJoinSmem) return fail(ctx, MSA_ERANGE, "%d rows do not fit %d CTAs", Pn, grid);
+      if (!s.rshared) TRY(ensure(ctx, rcopy, sizeof(long long) * (size_t)Pn * grid));
       NjJob job{P<int>(*cD), Pn, stop, t, n, P<long long>(*cR), P<uint8_t>(act), P<int>(*cN),
                 P<int>(joins), P<long long>(lengths), P<int>(stage),
-                rshared ? nullptr : P<long long>(rcopy), ctx->derr};
+                s.rshared ? nullptr : P<long long>(rcopy), ctx->derr};
       ++ctx->launches;
-      // fewer threads make the block-wide steps of a join cheaper, more keep
-      // more of rows x and y in flight
-      const int threads = solo || Pn <= 1536 ? 256 : Pn <= 8192 ? 512 : 1024;
-      const void *fn = solo ? (const void *)k_nj_joins<1, 256>
-                     : threads == 256 ? (const void *)k_nj_joins<kJoinCtas, 256>
-                     : threads == 512 ? (const void *)k_nj_joins<kJoinCtas, 512>
-                                      : (const void *)k_nj_joins<kJoinCtas, 1024>;
-      CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kJoinSmem));
-      if (grid > 8) CK(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      cudaLaunchConfig_t cfg;
       cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = (unsigned)grid;
-      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)grid);
-      cfg.blockDim = dim3((unsigned)threads);
-      cfg.dynamicSmemBytes = smem;
-      cfg.stream = ctx->st;
-      cfg.attrs = &attr;
-      cfg.numAttrs = grid > 1 ? 1 : 0;
+      CK(join_config(s, ctx->st, cfg, attr));
       void *args[] = {&job};
-      CK(cudaLaunchKernelExC(&cfg, fn, args));
+      CK(cudaLaunchKernelExC(&cfg, (const void *)join_kernel(s.ctas, s.threads), args));
       t += Pn - stop;
       if (stop <= 2) break;
       const int m = stop;
@@ -1248,6 +1296,15 @@ int msa_nj(msa_ctx *ctx, const int64_t *dist, int64_t n, int32_t *joins_out, dou
   release(ctx, D);
   release(ctx, D1);
   return rc;
+}
+
+int msa_debug_nj_shape(msa_ctx *ctx, int32_t ctas, int32_t threads, int32_t sums_global) {
+  if (!ctx || (ctas != 0 && ctas != 1 && ctas != kJoinCtasFew && ctas != kJoinCtas)) return MSA_EINVAL;
+  if (threads != 0 && threads != 256 && threads != 512 && threads != 1024) return MSA_EINVAL;
+  ctx->nj_ctas = ctas;
+  ctx->nj_threads = threads;
+  ctx->nj_sums_global = sums_global != 0;
+  return MSA_OK;
 }
 
 int msa_nj_tree(msa_ctx *ctx, int32_t *joins_out, double *lengths_out) {

@@ -176,3 +176,30 @@ def test_distances_around_the_tile_sizes(kind, n, length):
         rows, _ = b.msa_merge_gaps(h)
         d = b.msa_tree_distances(h)
     assert (d == T.msa_distances(rows)).all()
+
+
+def nj_matrix(rng, n, kind):
+    lo, hi = {"ties": (1, 4), "star": (500000, 540000)}[kind]
+    D = np.triu(rng.integers(lo, hi, size=(n, n)).astype(np.int64), 1)
+    return D + D.T
+
+
+@pytest.mark.parametrize("n", [127, 128, 129, 700])
+@pytest.mark.parametrize("kind", ["ties", "star"])
+def test_nj_in_every_launch_shape(n, kind):
+    """One CTA and a cluster around the size where they change over, clusters of
+    8 and 16, every CTA size, row sums in shared and in global memory, and one
+    CTA with several rows per thread: all give the oracle's joins."""
+    b = binding()
+    D = nj_matrix(np.random.default_rng(n), n, kind)
+    oj, ol = T.nj(D)
+    with any_ctx() as h:
+        for ctas, threads in ((0, 0), (1, 0), (8, 256), (8, 512), (8, 1024), (16, 256), (16, 512), (16, 1024)):
+            for sums_global in (False, True):
+                b.msa_debug_nj_shape(h, ctas, threads, sums_global)
+                joins, lengths = b.msa_nj(h, D)
+                assert (joins == oj).all() and (lengths == ol).all(), (ctas, threads, sums_global)
+        for bad in ((2, 0), (16, 128)):
+            with pytest.raises(b.MSAError) as ei:
+                b.msa_debug_nj_shape(h, *bad)
+            assert ei.value.code == b.MSA_EINVAL
