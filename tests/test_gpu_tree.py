@@ -203,3 +203,72 @@ def test_nj_in_every_launch_shape(n, kind):
             with pytest.raises(b.MSAError) as ei:
                 b.msa_debug_nj_shape(h, *bad)
             assert ei.value.code == b.MSA_EINVAL
+
+
+def additive(rng, n):
+    """Path lengths (int64[n, n] on the GPU) of a random binary tree over n leaves
+    with even, distinct edge lengths, the leaves in random order."""
+    import torch
+    depth, meet = np.zeros(n, np.int64), np.zeros(n - 1, np.int64)  # of a leaf; where k and k + 1 part
+    edge = iter(2 * rng.permutation(np.arange(1, 2 * n)))
+    stack = [(0, n, 0)]
+    while stack:
+        lo, hi, d = stack.pop()
+        if hi - lo == 1:
+            depth[lo] = d
+            continue
+        cut = int(rng.integers(lo + 1, hi))
+        meet[cut - 1] = d
+        stack += [(lo, cut, d + int(next(edge))), (cut, hi, d + int(next(edge)))]
+    h, g = torch.tensor(depth, device="cuda"), torch.tensor(meet, device="cuda")
+    D = torch.zeros(n, n, dtype=torch.int64, device="cuda")
+    cols = torch.arange(n - 1, device="cuda")
+    for r0 in range(0, n - 1, 1024):  # two leaves part at the smallest depth between them
+        r = torch.arange(r0, min(n - 1, r0 + 1024), device="cuda")[:, None]
+        part = torch.where(cols[None] < r, 1 << 40, g[None].expand(r.numel(), -1)).cummin(1).values
+        D[r0:r0 + r.numel(), 1:] = torch.where(cols[None] < r, 0, h[r] + h[None, 1:] - 2 * part)
+    D += D.T.clone()
+    order = torch.tensor(rng.permutation(n), device="cuda")
+    return D[order][:, order].contiguous()
+
+
+def path_sums(n, edges, root, probe):
+    """Distance of every leaf from each probe leaf, along the tree's edges."""
+    up = {c: (p, w) for p, c, w in edges}
+    kids = {}
+    for p, c, w in edges:
+        kids.setdefault(p, []).append((c, w))
+    out = []
+    for leaf in probe:
+        dist, v, d, came = {}, leaf, 0.0, None
+        while True:
+            stack = [(v, d)]
+            while stack:
+                u, du = stack.pop()
+                if u < n:
+                    dist[u] = du
+                stack += [(c, du + w) for c, w in kids.get(u, []) if c != came]
+            if v == root:
+                break
+            came, (v, w) = v, up[v]
+            d += w
+        out.append([dist[k] for k in range(n)])
+    return np.array(out)
+
+
+@pytest.mark.parametrize("n", [1536, 1537, 8193, 16500, 23000])
+def test_nj_of_additive_distances_at_large_sizes(n):
+    """Sizes where the default launch changes (threads at 1,537 and 8,193 rows,
+    several rows per thread above 16,384, row sums in global memory above 22,800):
+    the distances of a tree give that tree back, so its path lengths are the matrix."""
+    import torch
+    b = binding()
+    D = additive(np.random.default_rng(n), n)
+    probe = np.random.default_rng(1).choice(n, size=12, replace=False)
+    rows = D[torch.tensor(probe, device="cuda")].cpu().numpy()
+    with any_ctx() as h:
+        joins, lengths = b.msa_nj(h, D)
+    joins, lengths = np.asarray(joins).reshape(-1, 2), np.asarray(lengths).reshape(-1, 2)
+    assert sorted(joins.ravel().tolist()) == list(range(2 * n - 2))
+    edges = [(n + t, int(joins[t, s]), float(lengths[t, s])) for t in range(n - 1) for s in range(2)]
+    assert (path_sums(n, edges, 2 * n - 2, probe.tolist()) == rows).all()
