@@ -691,24 +691,23 @@ __global__ void k_nj_init(long long *__restrict__ r, const int *__restrict__ D, 
   }
 }
 
-// Bit planes of a slab of listed rows (list: device, null = rows r0, ...).
+// Bit planes of a slab of listed rows.
 struct Planes {
-  DevBuf lo, hi;
-  int r0 = 0, rows = 0;
+  uint4 *lo = nullptr;
+  uint2 *hi = nullptr;  // more than seven letters
+  int rows = 0;
 };
 
+// The planes of rows r0, r0 + 1, ... (of the list: device, null = all rows)
+// into p's memory.
 int make_planes(msa_ctx *ctx, Planes &p, const int32_t *list, int r0, int rows, int words) {
   const size_t cells = (size_t)rows * words;
-  const bool wide = ctx->K > 7;
-  TRY(ensure(ctx, p.lo, sizeof(uint4) * cells));
-  if (wide) TRY(ensure(ctx, p.hi, sizeof(uint2) * cells));
   const int blocks = (int)std::min<size_t>((cells + 31) / 32, 1 << 14);  // four words per warp or more
   ++ctx->launches;
-  auto fn = wide ? k_planes<true> : k_planes<false>;
+  auto fn = ctx->K > 7 ? k_planes<true> : k_planes<false>;
   fn<<<std::max(blocks, 1), 256, 0, ctx->st>>>(P<uint8_t>(ctx->msa), ctx->W, list, r0, rows, words,
-                                               ctx->dSymLut, ctx->K, P<uint4>(p.lo), P<uint2>(p.hi));
+                                               ctx->dSymLut, ctx->K, p.lo, p.hi);
   CK(cudaGetLastError());
-  p.r0 = r0;
   p.rows = rows;
   return MSA_OK;
 }
@@ -717,19 +716,41 @@ int make_planes(msa_ctx *ctx, Planes &p, const int32_t *list, int r0, int rows, 
 // ib[0..nB): into the matrix D (near null: both lists the same, nA x nA, T =
 // int or long long), or each row of A's nearest row of B into near.  The
 // planes are held a slab of rows at a time, fewer where a device memory limit
-// leaves less.
+// leaves less; where it leaves no room for them they take the place of the
+// traceback codes, which nothing reads between two calls.
 template <class T>
 int distances(msa_ctx *ctx, const int32_t *ia, int nA, const int32_t *ib, int nB, T *D,
               unsigned long long *near) {
   const int words = (int)((ctx->W + 32 * kPlaneWords - 1) / (32 * kPlaneWords)) * kPlaneWords;
-  int slab = kSlab;
+  const size_t row = (size_t)words * (sizeof(uint4) + (ctx->K > 7 ? sizeof(uint2) : 0));
+  int slab = std::min(kSlab, (std::max(nA, nB) + kTile - 1) / kTile * kTile);
+  auto bytes = [&](int rows) { return row * rows * (near || nA > rows ? 2 : 1); };  // one slab, or two
+  DevBuf own;
+  char *mem = nullptr;
   if (ctx->dev_limit) {
     const size_t left = ctx->dev_limit > ctx->dev_bytes ? ctx->dev_limit - ctx->dev_bytes : 0;
-    const size_t per = 2 * sizeof(uint4) * 2 * (size_t)words;  // two slabs' rows
-    while (slab > kTile && (size_t)slab * per > left) slab /= 2;
+    while (slab > kTile && bytes(slab) + 256 > left) slab = std::max(kTile, slab / 2 / kTile * kTile);
+    if (bytes(slab) + 256 > left) {
+      int rows = std::min(slab, std::max(nA, nB));
+      while (rows > 1 && bytes(rows) > ctx->codes.cap) rows /= 2;
+      if (bytes(rows) <= ctx->codes.cap) {
+        slab = rows;
+        mem = P<char>(ctx->codes);
+      }
+    }
   }
-  Planes pa, pb;
   int rc = [&]() -> int {
+    if (!mem) {
+      TRY(ensure(ctx, own, bytes(slab)));
+      mem = P<char>(own);
+    }
+    Planes pa, pb;
+    // (both slabs' 16-byte words first, so that every plane is aligned)
+    const size_t cells = (size_t)slab * words;
+    pa.lo = reinterpret_cast<uint4 *>(mem);
+    pb.lo = pa.lo + cells;
+    pa.hi = reinterpret_cast<uint2 *>(pa.lo + bytes(slab) / row * words);
+    pb.hi = pa.hi + cells;
     for (int a0 = 0; a0 < nA; a0 += slab) {
       const int ra = std::min(slab, nA - a0);
       TRY(make_planes(ctx, pa, ia, a0, ra, words));
@@ -738,8 +759,7 @@ int distances(msa_ctx *ctx, const int32_t *ia, int nA, const int32_t *ib, int nB
         const bool same = !near && b0 == a0;
         if (!same && (nB > slab || pb.rows == 0)) TRY(make_planes(ctx, pb, ib, b0, rb, words));
         Planes &q = same ? pa : pb;
-        PdistJob job{P<uint4>(pa.lo), P<uint4>(q.lo), P<uint2>(pa.hi), P<uint2>(q.hi), words,
-                     ra, rb, a0, b0, (size_t)nA, near};
+        PdistJob job{pa.lo, q.lo, pa.hi, q.hi, words, ra, rb, a0, b0, (size_t)nA, near};
         ++ctx->launches;
         auto fn = ctx->K > 7 ? k_pdist<true, T> : k_pdist<false, T>;
         fn<<<dim3((rb + kTile - 1) / kTile, (ra + kTile - 1) / kTile), 256, 0, ctx->st>>>(job, D);
@@ -748,7 +768,7 @@ int distances(msa_ctx *ctx, const int32_t *ia, int nA, const int32_t *ib, int nB
     }
     return MSA_OK;
   }();
-  for (DevBuf *b : {&pa.lo, &pa.hi, &pb.lo, &pb.hi}) release(ctx, *b);
+  release(ctx, own);
   return rc;
 }
 

@@ -103,3 +103,40 @@ def test_rows_whose_staging_fills_the_default_shared_memory():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", ROWS_OF_6120], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr
+
+
+@pytest.mark.parametrize("kind, n, length", [("protein", 130, 300), ("dna", 70, 500), ("protein", 40, 60)])
+def test_tree_distances_in_no_more_than_their_matrix(kind, n, length):
+    """A limit that leaves room for the n x n distances alone, and for a few
+    kilobytes more: the same distances as without one."""
+    from seqgen import blosum62
+    b = binding()
+    rng = np.random.default_rng(n)
+    alph, M = blosum62() if kind == "protein" else dna_matrix()
+    pool = np.frombuffer(alph[:20].encode(), np.uint8)
+    base = rng.choice(pool, size=length)
+    seqs = []
+    for _ in range(n):
+        s = base[:int(rng.integers(length // 2, length + 1))].copy()
+        hit = rng.random(s.size) < 0.1
+        s[hit] = rng.choice(pool, size=int(hit.sum()))
+        seqs.append(s)
+    letters, offsets = pack_sequences(seqs)
+    with make_ctx(alph, M, 11, 1) as h:
+        b.msa_load(h, letters, offsets)
+        b.msa_align_to_center(h, 0)
+        b.msa_merge_gaps(h, want_rows=False)
+        want = b.msa_tree_distances(h)
+        held = b.msa_memory(h)[0]
+        for more in (0, 4096, 20000, 60000, 200000):
+            b.msa_set_memory_limit(h, held + (8 * n * n + 255) // 256 * 256 + more)
+            assert (b.msa_tree_distances(h) == want).all()
+        b.msa_set_memory_limit(h, held + 8 * n * n - 4096)
+        with pytest.raises(b.MSAError) as ei:
+            b.msa_tree_distances(h)
+        assert ei.value.code == b.MSA_ENOMEM
+        # the alignment is still there, and another one starts from it
+        b.msa_set_memory_limit(h, 0)
+        before = b.msa_alignment_info(h)
+        b.msa_align_to_center(h, 0)
+        assert all((x == y).all() for x, y in zip(before, b.msa_alignment_info(h)))
