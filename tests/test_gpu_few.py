@@ -85,3 +85,36 @@ def test_few_subjects_at_the_ring_s_wrap(lc):
     seqs += [rng.choice(pool, size=L) for L in (769, 833, 1025)]
     letters, offsets = pack_sequences(seqs)
     check(letters, offsets, alph, M, 11, 1, 0)
+
+
+@pytest.mark.parametrize("precision", ["AUTO", "INT32"])
+def test_many_subjects_keep_the_codes_kernels(precision):
+    """12,000 subjects, where one CTA per subject would be the slower choice: the
+    default alignment (a fill and a traceback) and the anchored path's left-over
+    subjects (all of them: no segment matches) against the oracle."""
+    b = binding()
+    rng = np.random.default_rng(12)
+    alph, M = dna_matrix()
+    pool = np.frombuffer(b"ACGT", np.uint8)
+    center = rng.choice(pool, size=150)
+    seqs = [center] + [related(rng, center, int(L), pool) for L in rng.integers(100, 151, 12000)]
+    letters, offsets = pack_sequences(seqs)
+    n = len(seqs)
+    prob = oracle_problem(letters, offsets, alph, M, 5, 2)
+    oseg, oins, oocc, _, _, _ = oracle.msa(prob, 0)
+    foreign = pack_sequences([center] + [rng.choice(pool, size=int(L)) for L in rng.integers(100, 151, 12000)])
+    fprob = oracle_problem(*foreign, alph, M, 5, 2)
+    fseg, fins, focc = oracle.anchored_all(fprob, 0, 24)
+    with make_ctx(alph, M, 5, 2, precision=getattr(b, "MSA_" + precision)) as h:
+        b.msa_load(h, letters, offsets)
+        before = b.msa_stage_times(h)[1]["launches"]
+        b.msa_align_to_center(h, 0)
+        assert b.msa_stage_times(h)[1]["launches"] - before == 2
+        seg, ins, occ = b.msa_alignment_info(h)
+        assert (seg == oseg).all() and (ins == oins).all() and (occ == oocc).all()
+        b.msa_load(h, *foreign)
+        before = b.msa_stage_times(h)[1]["launches"]
+        assert b.msa_align_anchored(h, 0, 24) == n - 1
+        assert b.msa_stage_times(h)[1]["launches"] - before == 3
+        seg, ins, occ = b.msa_alignment_info(h)
+        assert (seg == fseg).all() and (ins == fins).all() and (occ == focc).all()
