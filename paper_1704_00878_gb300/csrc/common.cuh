@@ -3,6 +3,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+#include <vector>
+
 #include "msa.h"
 
 #define MSA_FULL_MASK 0xffffffffu
@@ -139,17 +142,31 @@ static inline int64_t round_up_i64(int64_t x, int64_t m) { return (x + m - 1) / 
 // that the device leaves beside its static part (*most, where given).  The
 // limit belongs to the kernel in the process and not to a context: set to one
 // call's size, another thread's smaller call could lower it before the first
-// one has launched.
+// one has launched.  The size is looked up once per kernel and device (at 320 us
+// a small alignment would spend 1.6 on it) and set each time.
 static inline cudaError_t allow_smem(const void *fn, int *most = nullptr) {
-  int dev = 0, all = 0;
-  cudaFuncAttributes a;
+  struct Size {
+    const void *fn;
+    int dev, bytes;
+  };
+  static std::mutex lock;
+  static std::vector<Size> sizes;
+  int dev = 0, all = -1;
   cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
   if (e != cudaSuccess) return e;
-  all -= (int)a.sharedSizeBytes;
+  {
+    std::lock_guard<std::mutex> guard(lock);
+    for (const Size &s : sizes)
+      if (s.fn == fn && s.dev == dev) all = s.bytes;
+    if (all < 0) {
+      cudaFuncAttributes a;
+      e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+      if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
+      if (e != cudaSuccess) return e;
+      all -= (int)a.sharedSizeBytes;
+      sizes.push_back({fn, dev, all});
+    }
+  }
   if (most) *most = all;
-  return a.maxDynamicSharedSizeBytes == all
-             ? cudaSuccess
-             : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, all);
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, all);
 }
