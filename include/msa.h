@@ -353,10 +353,11 @@ int msa_dims(msa_ctx *ctx, int64_t *dims_out);
 
 /* Device milliseconds of the stages of the last calls, CUDA events on the
  * context stream: [0] encode, [1] center selection, [2] align DP, [3]
- * traceback, [4] merge, [5] rows, [6] SP, [7] center DP kernels alone, [8]
- * align DP kernels alone, [9] selector (embedding or training), [10] tree
- * (distances and neighbour joining), and the passes of the last MSA_ALIGN_BOX
- * alignment: [11] score pass, [12] reverse pass, [13] box codes (their sum is
+ * traceback (0 where few subjects are aligned with their traceback in one
+ * launch: [2] and [8] are that launch then), [4] merge, [5] rows, [6] SP,
+ * [7] center DP kernels alone, [8] align DP kernels alone, [9] selector
+ * (embedding or training), [10] tree (distances and neighbour joining), and the
+ * passes of the last MSA_ALIGN_BOX alignment: [11] score pass, [12] reverse pass, [13] box codes (their sum is
  * [8] then).  counters_out (nullable, int64[3]): DP cells of the last center
  * selection, DP cells of the last alignment (the whole matrices', in either
  * mode), kernels launched by this context since msa_create. */
@@ -404,10 +405,11 @@ int msa_align_autotune(msa_ctx *ctx, int64_t center, double *rates_out, int32_t 
 /* Lanes per subject group of the alignment kernels (1, 2, 4, 8, 16 or 32;
  * each lane holds 16 center rows, so a pass covers 16 x lanes rows; with 1
  * lane every lane aligns its own subjects, pass after pass), or 0 for the
- * choice of the library's cost model among 8, 16 and 32 (the default).  Under
- * MSA_ALIGN_BOX a width set here holds for all three passes; otherwise the
- * score and reverse passes take the full pass's width and the box pass the
- * cost model's pick for the boxes' mean size.  A tuning knob: the result does
+ * choice of the library's cost model (the default): 8, 16 or 32 lanes, or,
+ * where the subjects are too few to fill the GPU so, a CTA per subject that
+ * also traces back.  Under MSA_ALIGN_BOX a width set here holds for all three
+ * passes; otherwise the score and reverse passes take the full pass's width
+ * and the box pass the cost model's pick for the boxes' mean size.  A tuning knob: the result does
  * not depend on it.  EINVAL for any other value. */
 int msa_set_align_group(msa_ctx *ctx, int32_t lanes);
 

@@ -841,9 +841,9 @@ static cudaError_t join_config(const JoinShape &s, cudaStream_t st, cudaLaunchCo
 static int join_threads(int P) { return P <= 1536 ? 256 : P <= 8192 ? 512 : 1024; }
 
 // CTAs of the joins' cluster: 16 (not portable: a partition of the device, or a
-// GPC with fewer free SMs, may have no room for it), else 8, which every device
-// of this architecture runs.  4,000 rows 30.7 ms with 16,
-// 36.4 with 8; 10,000 139 and 168.
+// GPC with fewer SMs, may have no room for it), else 8, which every device of
+// this architecture runs.  4,000 rows 30.7 ms with 16, 36.4 with 8; 10,000 139
+// and 168.
 static int join_ctas(int n) {
   const JoinShape s = join_shape(n, kJoinCtas, join_threads(n), false);
   cudaLaunchConfig_t cfg;
